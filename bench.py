@@ -119,7 +119,7 @@ def render_program_sha1(cfs, wl, fast_trig=False):
                                cfs.Chain(wl.chain, 2, fast_trig=fast_trig), wl.targets)
     h = hashlib.sha1(_code_only(src).encode())
     csrc = os.path.join(ROOT, "paper_2606_02226_gb300", "csrc")
-    for name in ("cfs_args.h", "cfs_device.cuh", "cfs_kernels.cuh"):
+    for name in ("cfs_args.h", "cfs_device.cuh", "cfs_window.cuh", "cfs_kernels.cuh"):
         with open(os.path.join(csrc, name)) as fh:
             h.update(_code_only(fh.read()).encode())
     return h.hexdigest()
@@ -586,7 +586,7 @@ def batch_program_sha1(cfs, frames):
                                [W.animation_target(fr.W)], mode=2)
     h = hashlib.sha1(_code_only(src).encode())
     csrc = os.path.join(ROOT, "paper_2606_02226_gb300", "csrc")
-    for name in ("cfs_args.h", "cfs_device.cuh", "cfs_kernels.cuh"):
+    for name in ("cfs_args.h", "cfs_device.cuh", "cfs_window.cuh", "cfs_kernels.cuh"):
         with open(os.path.join(csrc, name)) as fh:
             h.update(_code_only(fh.read()).encode())
     return h.hexdigest()

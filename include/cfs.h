@@ -350,7 +350,8 @@ cfs_status cfs_batch_windows(cfs_batch* batch, int32_t* out);
  * four fields shape the compiled program; chunk is the default work-item
  * size of every frame.  cfs_batch_create starts from the measured default
  * plan (ilp 2, window on when the chain splats once into a histogram, 53248
- * words, warp aggregation off, 4096 points per item). */
+ * words, warp aggregation off, 4096 points per item); a batch as created whose
+ * items of 4096 points would leave CTAs without work has smaller ones. */
 typedef struct {
     int ilp;                /* trajectories stepped together per thread: 1 or 2 */
     int window;             /* privatized shared-memory window for the chain's histogram

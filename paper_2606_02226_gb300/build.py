@@ -1,7 +1,7 @@
 """Builds ``libcfs.so`` in-tree (``paper_2606_02226_gb300/_build/``).
 
 Steps: embed the device sources handed to NVRTC at run time
-(``cfs_args.h``, ``cfs_device.cuh``, ``cfs_kernels.cuh``) as C++ raw string
+(``cfs_args.h`` and the ``.cuh`` files) as C++ raw string
 literals; compile every translation unit with nvcc for sm_103a in parallel;
 link one shared library against the CUDA runtime and NVRTC.
 """
@@ -23,7 +23,7 @@ LIB = os.path.join(BUILD, "libcfs.so")
 
 GENCODE = "arch=compute_103a,code=sm_103a"
 EMBEDDED = [("kSrcArgs", "cfs_args.h"), ("kSrcDevice", "cfs_device.cuh"),
-            ("kSrcKernels", "cfs_kernels.cuh")]
+            ("kSrcKernels", "cfs_kernels.cuh"), ("kSrcWindow", "cfs_window.cuh")]
 SOURCES = ["cfs_api.cpp", "cfs_batch.cpp", "cfs_codegen.cpp", "cfs_runtime.cpp",
            "cfs_builtin.cu", "cfs_sort.cu", "cfs_sampler.cu", "cfs_noalloc.cu", "cfs_display.cu", "cfs_scribble.cpp",
            "cfs_embed.cpp"]

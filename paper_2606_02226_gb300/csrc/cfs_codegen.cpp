@@ -108,7 +108,7 @@ static void emit_splat(std::ostringstream& s, const ProgramSpec& sp, size_t si)
       << 4 * si + 2 << "] = qz; rec[" << 4 * si + 3 << "] = alive ? 1.0f : 0.0f; } ";
     s << "if (do_splat) ";
     if (t.kind == CFS_TARGET_HIST_U32 && sp.tile && si == 0)
-        s << "cfs_splat_hist_tile(tg[" << t.slot << "], tile, qx, qy, alive, kc % " << t.channels
+        s << "cfs_splat_hist_tile(tg[" << t.slot << "], tile, qx, qy, alive, kc, " << t.channels
           << ", disc[" << t.slot << "]);";
     else if (t.kind == CFS_TARGET_HIST_U32)
         s << "cfs_splat_hist(tg[" << t.slot << "], qx, qy, alive, kc % " << t.channels
@@ -284,7 +284,7 @@ static void emit_chain(std::ostringstream& s, const ProgramSpec& sp)
               << "] = alive ? 1.0f : 0.0f; }\n";
             s << "    if (do_splat) ";
             if (t.kind == CFS_TARGET_HIST_U32 && sp.tile && si == 0)
-                s << "cfs_splat_hist_tile(tg[" << t.slot << "], tile, qx, qy, alive, kc % "
+                s << "cfs_splat_hist_tile(tg[" << t.slot << "], tile, qx, qy, alive, kc, "
                   << t.channels << ", disc[" << t.slot << "]);\n";
             else if (t.kind == CFS_TARGET_HIST_U32)
                 s << "cfs_splat_hist(tg[" << t.slot << "], qx, qy, alive, kc % " << t.channels

@@ -46,6 +46,44 @@ __device__ __forceinline__ uint4 cfs_philox(const cfs_launch_args& a, u32 c0, u3
     return cfs_philox_rk(a.rk, c0, c1, c2, c3);
 }
 
+/* The step stream of one trajectory: blocks (i, nb, s, 0) for nb = 0, 1, ...
+ * Of the first three rounds' six multiplies four depend on (i, s) alone and
+ * one on (nb, s) alone; the trajectory's four words below hold what the first
+ * four leave, so a block costs 15 multiplies and one that every lane of the
+ * launch shares, instead of 20. */
+struct CfsStream {
+    u32 a, b, c, d;
+};
+
+__device__ __forceinline__ CfsStream cfs_stream(const unsigned int (&rk)[10][2], u32 i, u32 sid)
+{
+    const u64 p0 = (u64)0xD2511F53u * (u64)i, p1 = (u64)0xCD9E8D57u * (u64)sid;
+    /* round 1 leaves c1 = lo(p1), c2 = hi(p0) ^ key, c3 = lo(p0) (and c0 the
+     * block's own); round 2 turns c2 and c1 into round 3's c0 and c1 */
+    const u64 q1 = (u64)0xCD9E8D57u * (u64)((u32)(p0 >> 32) ^ rk[0][1]);
+    const u64 r0 = (u64)0xD2511F53u * (u64)((u32)(q1 >> 32) ^ (u32)p1 ^ rk[1][0]);
+    return CfsStream{(u32)p0 ^ rk[1][1], (u32)q1 ^ rk[2][0], (u32)(r0 >> 32) ^ rk[2][1], (u32)r0};
+}
+
+__device__ __forceinline__ uint4 cfs_stream_block(const unsigned int (&rk)[10][2],
+                                                  const CfsStream& t, u32 nb, u32 sid)
+{
+    const u32 s = __umulhi(0xCD9E8D57u, sid) ^ rk[0][0];
+    const u64 q0 = (u64)0xD2511F53u * (u64)(nb ^ s);      /* round 2, the same in every lane */
+    const u64 r1 = (u64)0xCD9E8D57u * (u64)((u32)(q0 >> 32) ^ t.a);         /* round 3 */
+    u32 c0 = (u32)(r1 >> 32) ^ t.b, c1 = (u32)r1, c2 = (u32)q0 ^ t.c, c3 = t.d;
+#pragma unroll
+    for (int r = 3; r < 10; ++r) {
+        const u64 p0 = (u64)0xD2511F53u * (u64)c0;
+        const u64 p1 = (u64)0xCD9E8D57u * (u64)c2;
+        c0 = (u32)(p1 >> 32) ^ c1 ^ rk[r][0];
+        c1 = (u32)p1;
+        c2 = (u32)(p0 >> 32) ^ c3 ^ rk[r][1];
+        c3 = (u32)p0;
+    }
+    return make_uint4(c0, c1, c2, c3);
+}
+
 __device__ __forceinline__ u32 cfs_word(uint4 r, u32 s)
 {
     return s == 0 ? r.x : (s == 1 ? r.y : (s == 2 ? r.z : r.w));
@@ -435,79 +473,7 @@ __device__ __forceinline__ void cfs_splat_hist(const cfs_dev_target& t, float x,
     }
 }
 
-/* What a windowed batch splat reads of its target: the frame's values,
- * copied to the batch kernel's locals once per frame so that they stay in
- * registers instead of being read from shared memory on every splat. */
-struct CfsBinTarget {
-    unsigned long long data;
-    int W, H;
-    float x0, x1, sx, y0, y1, sy;
-};
-
-/* The privatized window of a batch frame's u32 histogram: one pixel box
- * per channel (a channel's splats come from its own maps, whose images are
- * smaller copies of the attractor, so each channel's box sits over that
- * channel's densest region), the channels' counters packed one after the
- * other in shared memory. */
-struct CfsTile {
-    u32* cnt;           /* shared counters */
-    const int4* win;    /* shared, per channel: (x0, y0, w | h << 16, first counter);
-                           w = 0: no window */
-};
-
-/* u32 histogram splat that adds to the shared window of its channel when
- * the bin lies in it (one shared atomic per group of lanes hitting the same
- * counter with CFS_WARP_AGG) and to global memory otherwise. */
-template <class T>
-__device__ __forceinline__ void cfs_splat_hist_tile(const T& t, const CfsTile& tl, float x,
-                                                    float y, bool alive, int ch, u32& disc)
-{
-    bool okx, oky;
-    const int ix = cfs_bin_ok(x, t.x0, t.x1, t.sx, t.W, okx);
-    const int iy = cfs_bin_ok(y, t.y0, t.y1, t.sy, t.H, oky);
-    const bool ok = alive && okx && oky;
-    const int4 g = tl.win[ch];
-    const u32 lx = (u32)(ix - g.x), ly = (u32)(iy - g.y);
-    const u32 w = (u32)g.z & 0xFFFFu, h = (u32)g.z >> 16;
-    if (ok && lx < w && ly < h) {
-        const u32 idx = (u32)g.w + ly * w + lx;
-#if CFS_WARP_AGG
-        const u32 act = __activemask();
-        const u32 peers = __match_any_sync(act, idx);
-        if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(tl.cnt + idx, __popc(peers));
-#else
-        atomicAdd(tl.cnt + idx, 1u);
-#endif
-    } else if (ok) {
-        u32* base = reinterpret_cast<u32*>(t.data);
-        const size_t off = ((size_t)ch * (size_t)t.H + (size_t)iy) * (size_t)t.W + (size_t)ix;
-        cfs_red_add_u32(base + off, 1u);
-    } else {
-        disc += 1;
-    }
-}
-
-/* Adds the windows' nonzero counters to the global histogram and zeroes
- * them; every thread of the CTA takes part. */
-__device__ __forceinline__ void cfs_flush_tile(const cfs_dev_target& t, const CfsTile& tl, int C)
-{
-    u32* base = reinterpret_cast<u32*>(t.data);
-    for (int ch = 0; ch < C; ++ch) {
-        const int4 g = tl.win[ch];
-        const u32 w = (u32)g.z & 0xFFFFu, h = (u32)g.z >> 16;
-        u32* cc = tl.cnt + (u32)g.w;
-        for (u32 e = threadIdx.x; e < w * h; e += blockDim.x) {
-            const u32 v = cc[e];
-            cc[e] = 0u;
-            if (v) {
-                const u32 ly = e / w, lx = e - ly * w;
-                const size_t off = ((size_t)ch * (size_t)t.H + (size_t)(g.y + (int)ly)) *
-                                       (size_t)t.W + (size_t)(g.x + (int)lx);
-                cfs_red_add_u32(base + off, v);
-            }
-        }
-    }
-}
+#include "cfs_window.cuh"
 
 /* f32 RGBA [H][W][4]: += colour (one 16-byte vector reduction). */
 __device__ __forceinline__ void cfs_splat_rgba(const cfs_dev_target& t, float x, float y,

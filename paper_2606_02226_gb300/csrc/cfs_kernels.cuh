@@ -55,44 +55,6 @@ struct CfsChooseTab {
     }
 };
 
-#if CFS_BATCH
-/* Map choice of a batch frame through a bucket table: the top 12 bits of the
- * word pick one of 4096 buckets of 2^20 words; a bucket without a threshold
- * inside gives every word in it the same k (the table holds it), the at most
- * n_cmp buckets with one fall back to the comparisons.  Same k as
- * CfsChooseTab for every word. */
-#define CFS_KTAB_BITS 12
-struct CfsChooseKtab {
-    const u32* T;               /* shared memory */
-    const unsigned char* kt;    /* shared memory, 2^CFS_KTAB_BITS entries; 0xFF: compare */
-    int n_cmp;
-    __device__ __forceinline__ int operator()(u32 w) const
-    {
-        const u32 e = kt[w >> (32 - CFS_KTAB_BITS)];
-        if (e != 0xFFu) return (int)e;
-        int k = 0;
-#pragma unroll
-        for (int j = 0; j < CFS_NCMP; ++j) k += (j < n_cmp && w >= T[j]) ? 1 : 0;
-        return k;
-    }
-};
-
-/* the frame's bucket table from its thresholds (all threads; the caller
- * synchronizes before and after) */
-__device__ __forceinline__ void cfs_build_ktab(const u32* T, int n_cmp, unsigned char* kt)
-{
-    for (u32 b = threadIdx.x; b < (1u << CFS_KTAB_BITS); b += blockDim.x) {
-        const u32 w0 = b << (32 - CFS_KTAB_BITS), w1 = w0 | ((1u << (32 - CFS_KTAB_BITS)) - 1u);
-        int k0 = 0, k1 = 0;
-        for (int j = 0; j < n_cmp; ++j) {
-            k0 += w0 >= T[j] ? 1 : 0;
-            k1 += w1 >= T[j] ? 1 : 0;
-        }
-        kt[b] = k0 == k1 ? (unsigned char)k0 : (unsigned char)0xFFu;
-    }
-}
-#endif
-
 /* start point: Philox block (i, 0, s, 1), coordinates (word >> 8) * 2^-24,
  * or the caller's SoA start array (index j of this launch) */
 __device__ __forceinline__ void cfs_start(const cfs_launch_args& a, u32 i, u32 sid, u32 j,
@@ -169,6 +131,7 @@ __device__ __forceinline__ void cfs_run_point(const cfs_launch_args& a, const CH
 {
     const u32 b0 = a.step_begin, b1 = a.iters;
     const bool whole = ((b0 | b1) & 3u) == 0u;
+    const CfsStream ps = cfs_stream(a.rk, i, sid);
 #if !CFS_REUSE && !(CFS_BATCH && CFS_ILP == 2)
     /* (the two-trajectory batch program calls this only for a frame's odd
      * last point: the general loop keeps its code small) */
@@ -181,7 +144,7 @@ __device__ __forceinline__ void cfs_run_point(const cfs_launch_args& a, const CH
         u32 nb = b0 >> 2;
 #pragma unroll 1
         for (; nb < nbs; ++nb) {
-            const uint4 r = cfs_philox(a, i, nb, sid, 0u);
+            const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
             cfs_gen_map(a, choose(r.x), x, y, z, sm);
             cfs_gen_map(a, choose(r.y), x, y, z, sm);
             cfs_gen_map(a, choose(r.z), x, y, z, sm);
@@ -189,7 +152,7 @@ __device__ __forceinline__ void cfs_run_point(const cfs_launch_args& a, const CH
         }
 #pragma unroll 1
         for (; nb < nb1; ++nb) {
-            const uint4 r = cfs_philox(a, i, nb, sid, 0u);
+            const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
             const uint4 ra = cfs_aux_block(a, i, nb, sid);
 #if CFS_UNROLL == 4
             cfs_step_splat(a, choose, tg, sm, r.x, ra.x, x, y, z, disc, tile);
@@ -220,7 +183,7 @@ __device__ __forceinline__ void cfs_run_point(const cfs_launch_args& a, const CH
 #endif
 #pragma unroll 1
     for (u32 nb = b0 >> 2; (nb << 2) < b1; ++nb) {
-        const uint4 r = cfs_philox(a, i, nb, sid, 0u);
+        const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
         const uint4 ra = cfs_aux_block(a, i, nb, sid);
         const u32 n = nb << 2;
 #if CFS_UNROLL == 4
@@ -269,6 +232,7 @@ __device__ __forceinline__ void cfs_run_point2(const cfs_launch_args& a, const C
 {
     const u32 b0 = a.step_begin, b1 = a.iters;
     const bool whole = ((b0 | b1) & 3u) == 0u;
+    const CfsStream ps0 = cfs_stream(a.rk, i0, sid), ps1 = cfs_stream(a.rk, i1, sid);
 #if !CFS_REUSE
     if (whole && (a.burn_in & 3u) == 0u) {
         /* every block whole and the burn-in ending on a block boundary: the
@@ -279,8 +243,8 @@ __device__ __forceinline__ void cfs_run_point2(const cfs_launch_args& a, const C
         u32 nb = b0 >> 2;
 #pragma unroll 1
         for (; nb < nbs; ++nb) {
-            const uint4 r0 = cfs_philox(a, i0, nb, sid, 0u);
-            const uint4 r1 = cfs_philox(a, i1, nb, sid, 0u);
+            const uint4 r0 = cfs_stream_block(a.rk, ps0, nb, sid);
+            const uint4 r1 = cfs_stream_block(a.rk, ps1, nb, sid);
             const u32 w0[4] = {r0.x, r0.y, r0.z, r0.w};
             const u32 w1[4] = {r1.x, r1.y, r1.z, r1.w};
 #pragma unroll
@@ -291,8 +255,8 @@ __device__ __forceinline__ void cfs_run_point2(const cfs_launch_args& a, const C
         }
 #pragma unroll 1
         for (; nb < nb1; ++nb) {
-            const uint4 r0 = cfs_philox(a, i0, nb, sid, 0u);
-            const uint4 r1 = cfs_philox(a, i1, nb, sid, 0u);
+            const uint4 r0 = cfs_stream_block(a.rk, ps0, nb, sid);
+            const uint4 r1 = cfs_stream_block(a.rk, ps1, nb, sid);
             const uint4 a0 = cfs_aux_block(a, i0, nb, sid);
             const uint4 a1 = cfs_aux_block(a, i1, nb, sid);
             const u32 w0[4] = {r0.x, r0.y, r0.z, r0.w};
@@ -310,8 +274,8 @@ __device__ __forceinline__ void cfs_run_point2(const cfs_launch_args& a, const C
 #endif
 #pragma unroll 1
     for (u32 nb = b0 >> 2; (nb << 2) < b1; ++nb) {
-        const uint4 r0 = cfs_philox(a, i0, nb, sid, 0u);
-        const uint4 r1 = cfs_philox(a, i1, nb, sid, 0u);
+        const uint4 r0 = cfs_stream_block(a.rk, ps0, nb, sid);
+        const uint4 r1 = cfs_stream_block(a.rk, ps1, nb, sid);
         const uint4 a0 = cfs_aux_block(a, i0, nb, sid);
         const uint4 a1 = cfs_aux_block(a, i1, nb, sid);
         const u32 n = nb << 2;
@@ -351,10 +315,11 @@ cfs_cloud_kernel(const __grid_constant__ cfs_launch_args a)
         const u32 i = a.point_begin + j;
         float x, y, z;
         cfs_start(a, i, sid, j, n_pts, x, y, z);
+        const CfsStream ps = cfs_stream(a.rk, i, sid);
         int k = 0;
 #pragma unroll 1
         for (u32 nb = 0; (nb << 2) < a.iters; ++nb) {
-            const uint4 r = cfs_philox(a, i, nb, sid, 0u);
+            const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
             const u32 w[4] = {r.x, r.y, r.z, r.w};
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -421,7 +386,7 @@ cfs_points_kernel(const __grid_constant__ cfs_launch_args a)
         float4 Z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (CFS_DIM == 3) Z = cfs_ld_stream_f4(xs + 2 * (size_t)n_pts + o, policy);
         const u32 K = cfs_ld_stream_u32(fn + o, policy);
-        const CfsTile nt{0, 0};
+        const CfsTile nt{0, 0, 0};
         float qx, qy, qz;
         cfs_chain(a, a.tg, sm, X.x, Y.x, Z.x, (int)(K & 0xFFu), 0u, disc, true, (float*)0, qx, qy, qz,
                   nt);
@@ -456,7 +421,7 @@ cfs_render_kernel(const __grid_constant__ cfs_launch_args a)
         float x, y, z;
         cfs_start(a, i, a.system_id, j, a.n_points, x, y, z);
         cfs_run_point(a, choose, a.tg, sm, i, a.system_id, x, y, z, disc,
-                      CfsTile{0, 0});
+                      CfsTile{0, 0, 0});
     }
     cfs_flush_discards(a, disc, CFS_NT);
 }
@@ -489,7 +454,7 @@ cfs_trace_kernel(const __grid_constant__ cfs_launch_args a)
         float qx, qy, qz;
         const bool alive = cfs_chain(a, a.tg, sm, x, y, z, k, aux, disc, false,
                                      qout + s * (size_t)CFS_NSPLAT_ARR * 4, qx, qy, qz,
-                                     CfsTile{0, 0});
+                                     CfsTile{0, 0, 0});
 #if CFS_REUSE
         if (alive) { x = qx; y = qy; z = qz; }
 #else
@@ -537,223 +502,62 @@ __device__ __forceinline__ void cfs_load_frame(const cfs_dev_frame& fr, CfsSmem&
 }
 
 #if CFS_TILE
-/* The first blockDim points of a frame, run for up to 32 splat steps past
- * the burn-in: calls visit(ix, iy, k) for every sample that lands in target
- * 0 (k: the generator map of the step). */
-template <class Visit>
-__device__ __forceinline__ void cfs_window_samples(const cfs_launch_args& a,
-                                                   const cfs_dev_frame& fr,
-                                                   const CfsChooseTab& choose,
-                                                   const cfs_dev_target* s_tg, const CfsSmem& sm,
-                                                   Visit visit)
-{
-    const u32 j = threadIdx.x;
-    if (j >= fr.n_points) return;
-    const u32 i = fr.point_begin + j, sid = fr.system_id;
-    const uint4 r0 = cfs_philox(a, i, 0u, sid, 1u);
-    float x = (float)(r0.x >> 8) * CFS_INV_2_24;
-    float y = (float)(r0.y >> 8) * CFS_INV_2_24;
-    float z = CFS_DIM == 3 ? (float)(r0.z >> 8) * CFS_INV_2_24 : 0.0f;
-    const u32 n1 = min(a.iters, a.burn_in + 32u);
-    const cfs_dev_target& t0 = s_tg[0];
-    u32 disc[CFS_NT_ARR];
-    for (u32 n = 0; n < n1; ++n) {
-        const uint4 r = cfs_philox(a, i, n >> 2, sid, 0u);
-        const int k = choose(cfs_word(r, n & 3u));
-        cfs_gen_map(a, k, x, y, z, sm);
-        if (n < a.burn_in) continue;
-        const u32 aux = cfs_word(cfs_aux_block(a, i, n >> 2, sid), n & 3u);
-        float rec[4 * CFS_NSPLAT_ARR];
-        float qx, qy, qz;
-        cfs_chain(a, s_tg, sm, x, y, z, k, aux, disc, false, rec, qx, qy, qz,
-                  CfsTile{0, 0});
-        const int ix = cfs_bin(rec[0], t0.x0, t0.x1, t0.sx, t0.W);
-        const int iy = cfs_bin(rec[1], t0.y0, t0.y1, t0.sy, t0.H);
-        if (rec[3] != 0.0f && ix >= 0 && iy >= 0) visit(ix, iy, k);
-    }
-}
-
-#define CFS_WG 64                        /* coarse density grid: CFS_WG x CFS_WG cells */
-#define CFS_WIN_SHAPES 5                 /* window aspect ratios 1/4, 1/2, 1, 2, 4 */
-
-/* Window shape q of the pre-pass (width / height = 2^(q - 2), q = 0..4):
- * at most cap pixels, inside a bw x bh box, widened to the cap once the
- * height is clamped. */
-__device__ __forceinline__ void cfs_window_shape(int q, int cap, int bw, int bh, int& ww, int& wh)
-{
-    ww = (int)sqrtf((float)cap * ldexpf(1.0f, q - 2));
-    ww = max(1, min(ww, bw));
-    wh = max(1, min(bh, cap / ww));
-    ww = max(1, min(bw, cap / wh));
-}
-
-/* Pre-pass of the privatized windows: one CTA per frame samples the frame's
- * first blockDim trajectories (see cfs_window_samples) and writes, for each
- * channel c of target 0, the pixel box its window covers to
- * frame_bbox[f * CFS_A_MAX_MAPS + c] (empty when no sample of the channel
- * landed).  The channels share the tile_cap counters in proportion to
- * their sampled splats (a channel's capacity, in pixels, is its share,
- * rounded down, so the windows together never pass tile_cap).  A sample's
+/* Pre-pass of the privatized windows (cfs_place_windows), one CTA per frame:
+ * channel c's box goes to frame_bbox[f * CFS_A_MAX_MAPS + c].  A sample's
  * channel is its map index mod CFS_TILE_C (a chain that recolours moves
  * splats to other channels; they then miss the window more often, nothing
- * else).
- * When the channel's sampled box fits its window, the window is that box.
- * Otherwise the channel's samples are binned into a coarse grid over the
- * box, and of the windows of the channel's capacity (five aspect ratios,
- * positions on the grid's cell boundaries) the one holding the most
- * samples wins: attractors are far from uniform, and the densest region is
- * where privatizing the counters saves the most L2 reductions.  Splats
- * outside the windows still go to global memory, so the choice changes the
- * speed only, never the histogram.  The trajectories are run again for
- * every pass (one for the channels' splat counts, then two per channel at
- * most): that is cheaper than storing the samples. */
+ * else). */
 extern "C" __global__ void __launch_bounds__(CFS_BLOCK)
 cfs_bbox_kernel(const __grid_constant__ cfs_launch_args a)
 {
+    extern __shared__ u32 s_samples[];
     __shared__ CfsSmem sm;
     cfs_chain_prologue(a, sm);   /* per-CTA tables of the chain (before the first barrier) */
     __shared__ u32 s_T[CFS_A_MAX_MAPS];
     __shared__ cfs_dev_target s_tg[CFS_NT_ARR];
-    __shared__ int s_box[4];
-    __shared__ u32 s_grid[CFS_WG * CFS_WG];
-    __shared__ unsigned long long s_best;
-    __shared__ u32 s_mass[CFS_TILE_C];
+    __shared__ CfsPlace s_place;
     const int f = blockIdx.x;
     const cfs_dev_frame& fr = reinterpret_cast<const cfs_dev_frame*>(a.frames)[f];
     cfs_load_frame(fr, sm, s_T, s_tg);
+    __syncthreads();
     const CfsChooseTab choose{s_T, fr.n_cmp};
-    if (threadIdx.x < CFS_TILE_C) s_mass[threadIdx.x] = 0u;
-    __syncthreads();
-    {
-        /* the channels' sampled splats */
-        u32 m[CFS_TILE_C];
-#pragma unroll
-        for (int c = 0; c < CFS_TILE_C; ++c) m[c] = 0u;
-        cfs_window_samples(a, fr, choose, s_tg, sm, [&](int ix, int iy, int k) {
-            (void)ix; (void)iy;
-            const int ch = k % CFS_TILE_C;
-#pragma unroll
-            for (int c = 0; c < CFS_TILE_C; ++c) m[c] += ch == c ? 1u : 0u;
-        });
-#pragma unroll
-        for (int c = 0; c < CFS_TILE_C; ++c)
-            if (m[c]) atomicAdd(&s_mass[c], m[c]);
-    }
-    __syncthreads();
-    u32 total = 0;
-    for (int c = 0; c < CFS_TILE_C; ++c) total += s_mass[c];
-    int4* out = reinterpret_cast<int4*>(a.frame_bbox) + (size_t)f * CFS_A_MAX_MAPS;
-    for (int c = 0; c < CFS_TILE_C; ++c) {
-        /* window pixels of this channel */
-        const int cap = total ? (int)(((unsigned long long)a.tile_cap * s_mass[c]) / total) : 0;
-        if (threadIdx.x == 0) {
-            s_box[0] = 0x7fffffff; s_box[1] = 0x7fffffff; s_box[2] = -1; s_box[3] = -1;
-            s_best = 0ull;
+    const cfs_dev_target& t0 = s_tg[0];
+    cfs_place_windows(t0, CFS_TILE_C, a.tile_cap, s_place, s_samples,
+                      reinterpret_cast<unsigned char*>(s_samples + CFS_WIN_SAMPLES * blockDim.x),
+                      reinterpret_cast<int4*>(a.frame_bbox) + (size_t)f * CFS_A_MAX_MAPS,
+                      [&](auto emit) {
+        const u32 j = threadIdx.x;
+        if (j >= fr.n_points) return;
+        const u32 i = fr.point_begin + j, sid = fr.system_id;
+        const uint4 r0 = cfs_philox(a, i, 0u, sid, 1u);
+        float x = (float)(r0.x >> 8) * CFS_INV_2_24;
+        float y = (float)(r0.y >> 8) * CFS_INV_2_24;
+        float z = CFS_DIM == 3 ? (float)(r0.z >> 8) * CFS_INV_2_24 : 0.0f;
+        const CfsStream ps = cfs_stream(a.rk, i, sid);
+        const u32 n1 = min(a.iters, a.burn_in + (u32)CFS_WIN_SAMPLES);
+        u32 disc[CFS_NT_ARR];
+#pragma unroll 1
+        for (u32 nb = 0; 4u * nb < n1; ++nb) {
+            uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
+            uint4 ra = cfs_aux_block(a, i, nb, sid);
+#pragma unroll 1
+            for (u32 n = 4u * nb; n < min(n1, 4u * nb + 4u); ++n) {
+                const int k = choose(r.x);
+                cfs_gen_map(a, k, x, y, z, sm);
+                const u32 aux = ra.x;
+                r = make_uint4(r.y, r.z, r.w, 0u);
+                ra = make_uint4(ra.y, ra.z, ra.w, 0u);
+                if (n < a.burn_in) continue;
+                float rec[4 * CFS_NSPLAT_ARR];
+                float qx, qy, qz;
+                cfs_chain(a, s_tg, sm, x, y, z, k, aux, disc, false, rec, qx, qy, qz,
+                          CfsTile{0, 0, 0});
+                const int ix = cfs_bin(rec[0], t0.x0, t0.x1, t0.sx, t0.W);
+                const int iy = cfs_bin(rec[1], t0.y0, t0.y1, t0.sy, t0.H);
+                if (rec[3] != 0.0f && ix >= 0 && iy >= 0) emit(ix, iy, k % CFS_TILE_C);
+            }
         }
-        for (int e = threadIdx.x; e < CFS_WG * CFS_WG; e += blockDim.x) s_grid[e] = 0u;
-        __syncthreads();
-        int bx0 = 0x7fffffff, by0 = 0x7fffffff, bx1 = -1, by1 = -1;
-        cfs_window_samples(a, fr, choose, s_tg, sm, [&](int ix, int iy, int k) {
-            if (k % CFS_TILE_C != c) return;
-            bx0 = min(bx0, ix); by0 = min(by0, iy);
-            bx1 = max(bx1, ix); by1 = max(by1, iy);
-        });
-        atomicMin(&s_box[0], bx0); atomicMin(&s_box[1], by0);
-        atomicMax(&s_box[2], bx1); atomicMax(&s_box[3], by1);
-        __syncthreads();
-        int4 box = make_int4(s_box[0], s_box[1], s_box[2], s_box[3]);
-        const int bw = box.z - box.x + 1, bh = box.w - box.y + 1;
-        if (box.z >= box.x && box.w >= box.y && cap >= 1 && (long long)bw * bh > cap) {
-            /* the grid: cells of cw x ch pixels over the box, gx x gy of them */
-            const int cw = (bw + CFS_WG - 1) / CFS_WG, ch = (bh + CFS_WG - 1) / CFS_WG;
-            const int gx = (bw + cw - 1) / cw, gy = (bh + ch - 1) / ch;
-            cfs_window_samples(a, fr, choose, s_tg, sm, [&](int ix, int iy, int k) {
-                if (k % CFS_TILE_C == c && ix >= box.x && ix <= box.z && iy >= box.y &&
-                    iy <= box.w)
-                    atomicAdd(&s_grid[((iy - box.y) / ch) * CFS_WG + (ix - box.x) / cw], 1u);
-            });
-            __syncthreads();
-            /* summed-area table: rows, then columns */
-            for (int r = threadIdx.x; r < gy; r += blockDim.x) {
-                u32 s = 0u;
-                for (int q = 0; q < gx; ++q) s_grid[r * CFS_WG + q] = (s += s_grid[r * CFS_WG + q]);
-            }
-            __syncthreads();
-            for (int q = threadIdx.x; q < gx; q += blockDim.x) {
-                u32 s = 0u;
-                for (int r = 0; r < gy; ++r) s_grid[r * CFS_WG + q] = (s += s_grid[r * CFS_WG + q]);
-            }
-            __syncthreads();
-            /* candidates: shape q, cell position (i0, j0); the window's whole
-             * cells nw x nh are counted */
-            const int per = CFS_WG * CFS_WG;
-            for (int cand = threadIdx.x; cand < CFS_WIN_SHAPES * per; cand += blockDim.x) {
-                const int q = cand / per, pos = cand - q * per;
-                const int j0 = pos / CFS_WG, i0 = pos - j0 * CFS_WG;
-                int ww, wh;
-                cfs_window_shape(q, cap, bw, bh, ww, wh);
-                const int nw = max(1, ww / cw), nh = max(1, wh / ch);
-                if (i0 + nw > gx || j0 + nh > gy) continue;
-                auto at = [&](int r, int col) -> u32 {
-                    return (r < 0 || col < 0) ? 0u : s_grid[r * CFS_WG + col];
-                };
-                const int r1 = j0 + nh - 1, c1 = i0 + nw - 1;
-                const u32 mass = at(r1, c1) - at(j0 - 1, c1) - at(r1, i0 - 1) + at(j0 - 1, i0 - 1);
-                /* most samples; ties to the lowest candidate number */
-                const unsigned long long key =
-                    ((unsigned long long)mass << 32) | (unsigned long long)(0xffffffffu - (u32)cand);
-                atomicMax(&s_best, key);
-            }
-            __syncthreads();
-            int ww, wh, x0, y0;
-            if (s_best != 0ull) {
-                const u32 cand = 0xffffffffu - (u32)(s_best & 0xffffffffull);
-                const int q = (int)(cand / (u32)per), pos = (int)(cand % (u32)per);
-                const int j0 = pos / CFS_WG, i0 = pos - j0 * CFS_WG;
-                cfs_window_shape(q, cap, bw, bh, ww, wh);
-                const int nw = max(1, ww / cw), nh = max(1, wh / ch);
-                /* centre the window on the counted cells */
-                x0 = box.x + i0 * cw + (nw * cw - ww) / 2;
-                y0 = box.y + j0 * ch + (nh * ch - wh) / 2;
-            } else {                   /* (no candidate) the square shape, centred */
-                cfs_window_shape(2, cap, bw, bh, ww, wh);
-                x0 = box.x + (bw - ww) / 2;
-                y0 = box.y + (bh - wh) / 2;
-            }
-            /* inside the box */
-            x0 = max(box.x, min(x0, box.z - ww + 1));
-            y0 = max(box.y, min(y0, box.w - wh + 1));
-            box = make_int4(x0, y0, x0 + ww - 1, y0 + wh - 1);
-        } else if (cap < 1) {
-            box = make_int4(0, 0, -1, -1);
-        }
-        if (threadIdx.x == 0) out[c] = box;
-        __syncthreads();                /* s_box, s_grid and s_best are reused */
-    }
-}
-
-/* Windows of frame f into s_win (thread 0 writes them): the pre-pass's
- * boxes, their counters packed one channel after the other; none when the
- * frame's shape class runs without a window (and, as a guard, for a box
- * that would pass the counters' end). */
-__device__ __forceinline__ void cfs_frame_window(const cfs_launch_args& a, int f, int4* s_win)
-{
-    if (threadIdx.x != 0) return;
-    const bool off = (reinterpret_cast<const cfs_dev_frame*>(a.frames)[f].flags &
-                      CFS_FRAME_NO_WINDOW) != 0;
-    const int4* box = reinterpret_cast<const int4*>(a.frame_bbox) + (size_t)f * CFS_A_MAX_MAPS;
-    u32 used = 0;
-    for (int c = 0; c < CFS_TILE_C; ++c) {
-        const int4 b = box[c];
-        const long long w = (long long)b.z - b.x + 1, h = (long long)b.w - b.y + 1;
-        if (off || w < 1 || h < 1 || w > 0xFFFF || h > 0x7FFF ||
-            (long long)used + w * h > (long long)a.tile_cap) {
-            s_win[c] = make_int4(0, 0, 0, 0);
-            continue;
-        }
-        s_win[c] = make_int4(b.x, b.y, (int)((u32)w | ((u32)h << 16)), (int)used);
-        used += (u32)(w * h);
-    }
+    });
 }
 #endif
 
@@ -780,15 +584,16 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
     __shared__ const float* s_start;
     __shared__ u32 s_scount;
     __shared__ int s_ncmp;
-    __shared__ unsigned char s_kt[1u << CFS_KTAB_BITS];   /* the frame's bucket table */
+    __shared__ CfsKtab s_kt;
 #if CFS_TILE
     extern __shared__ u32 s_cnt[];
-    __shared__ int4 s_win[CFS_TILE_C];
+    __shared__ int4 s_win[CFS_TILE_C];                /* per channel (cfs_pack_windows) */
+    __shared__ int4 s_mapwin[CFS_A_MAX_MAPS];         /* per map (CfsTile) */
+    __shared__ u32 s_maprow[CFS_A_MAX_MAPS];
     for (u32 e = threadIdx.x; e < a.tile_cap; e += blockDim.x) s_cnt[e] = 0u;
-    if (threadIdx.x < CFS_TILE_C) s_win[threadIdx.x] = make_int4(0, 0, 0, 0);
-    const CfsTile tile{s_cnt, s_win};
+    const CfsTile tile{s_mapwin, s_maprow, s_tg};
 #else
-    const CfsTile tile{0, 0};
+    const CfsTile tile{0, 0, 0};
 #endif
     const cfs_dev_frame* frames = reinterpret_cast<const cfs_dev_frame*>(a.frames);
     u32* counter = reinterpret_cast<u32*>(a.work_counter);
@@ -827,7 +632,7 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
             if (cur >= 0) {
                 cfs_flush_frame_discards(a, cur, disc);
 #if CFS_TILE
-                cfs_flush_tile(s_tg[0], tile, CFS_TILE_C);
+                cfs_flush_tile(s_tg[0], s_cnt, s_win, CFS_TILE_C);
 #endif
             }
             __syncthreads();
@@ -844,18 +649,25 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
                 s_scount = fr.start_count;
             }
 #if CFS_TILE
-            cfs_frame_window(a, f, s_win);
+            if (threadIdx.x == 0)
+                cfs_pack_windows(reinterpret_cast<const int4*>(a.frame_bbox) +
+                                     (size_t)f * CFS_A_MAX_MAPS,
+                                 CFS_TILE_C, a.tile_cap, (fr.flags & CFS_FRAME_NO_WINDOW) != 0,
+                                 s_win);
 #endif
             __syncthreads();
             cfs_build_ktab(s_T, s_ncmp, s_kt);
-            __syncthreads();
 #if CFS_TILE
-            bt[0] = CfsBinTarget{s_tg[0].data, s_tg[0].W, s_tg[0].H, s_tg[0].x0, s_tg[0].x1,
-                                 s_tg[0].sx, s_tg[0].y0, s_tg[0].y1, s_tg[0].sy};
+            if (threadIdx.x < CFS_A_MAX_MAPS) {
+                const int c = threadIdx.x % CFS_TILE_C;
+                s_mapwin[threadIdx.x] = cfs_win_record(s_win[c], s_cnt);
+                s_maprow[threadIdx.x] = (u32)(c * s_tg[0].H) - CFS_BIN_MAGIC;
+            }
+            bt[0] = cfs_bin_target(s_tg[0]);
 #endif
+            __syncthreads();
             cur = f;
         }
-        const CfsChooseKtab choose{s_T, s_kt, s_ncmp};
         const u32 sid = s_sid, pbeg = s_pbeg;
         const u32 j0 = (item - s_ibeg) * s_chunk;
         const u32 j1 = min(j0 + s_chunk, s_npts);
@@ -878,35 +690,41 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
                 z = CFS_DIM == 3 ? (float)(r.z >> 8) * CFS_INV_2_24 : 0.0f;
             }
         };
+        /* (two copies of the step code: the frames whose buckets all hold at
+         * most one threshold, and the others) */
+        auto run_item = [&](const auto& choose) {
 #if CFS_ILP == 2
-        /* two trajectories per thread, stepped in lockstep: their
-         * independent dependency chains hide each other's latency */
-        for (u32 j = j0 + threadIdx.x; j < j1; j += 2 * blockDim.x) {
-            const u32 j2 = j + blockDim.x;
-            float x, y, z;
-            start_of(j, x, y, z);
-            if (j2 < j1) {
-                float x2, y2, z2;
-                start_of(j2, x2, y2, z2);
-                cfs_run_point2(a, choose, CFS_BATCH_TG, sm, pbeg + j, pbeg + j2, sid, x, y, z, x2, y2,
-                               z2, disc, tile);
-            } else {
+            /* two trajectories per thread, stepped in lockstep: their
+             * independent dependency chains hide each other's latency */
+            for (u32 j = j0 + threadIdx.x; j < j1; j += 2 * blockDim.x) {
+                const u32 j2 = j + blockDim.x;
+                float x, y, z;
+                start_of(j, x, y, z);
+                if (j2 < j1) {
+                    float x2, y2, z2;
+                    start_of(j2, x2, y2, z2);
+                    cfs_run_point2(a, choose, CFS_BATCH_TG, sm, pbeg + j, pbeg + j2, sid, x, y, z, x2, y2,
+                                   z2, disc, tile);
+                } else {
+                    cfs_run_point(a, choose, CFS_BATCH_TG, sm, pbeg + j, sid, x, y, z, disc, tile);
+                }
+            }
+#else
+            for (u32 j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+                float x, y, z;
+                start_of(j, x, y, z);
                 cfs_run_point(a, choose, CFS_BATCH_TG, sm, pbeg + j, sid, x, y, z, disc, tile);
             }
-        }
-#else
-        for (u32 j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-            float x, y, z;
-            start_of(j, x, y, z);
-            cfs_run_point(a, choose, CFS_BATCH_TG, sm, pbeg + j, sid, x, y, z, disc, tile);
-        }
 #endif
+        };
+        if (s_kt.more <= 1) run_item(CfsChooseKtab<false>{s_kt, 1});
+        else run_item(CfsChooseKtab<true>{s_kt, s_kt.more});
         __syncthreads();
     }
     if (cur >= 0) {
         cfs_flush_frame_discards(a, cur, disc);
 #if CFS_TILE
-        cfs_flush_tile(s_tg[0], tile, CFS_TILE_C);
+        cfs_flush_tile(s_tg[0], s_cnt, s_win, CFS_TILE_C);
 #endif
     }
 }

@@ -25,6 +25,7 @@ namespace cfs {
 extern const char* const kSrcArgs;
 extern const char* const kSrcDevice;
 extern const char* const kSrcKernels;
+extern const char* const kSrcWindow;
 
 // ---- error reporting ---------------------------------------------------------
 static thread_local std::string t_err;
@@ -121,9 +122,9 @@ cfs_status compile(const std::string& src, std::vector<char>* cubin, std::string
                    bool verbose)
 {
     nvrtcProgram prog;
-    const char* headers[] = {kSrcArgs, kSrcDevice, kSrcKernels};
-    const char* names[] = {"cfs_args.h", "cfs_device.cuh", "cfs_kernels.cuh"};
-    nvrtcResult r = nvrtcCreateProgram(&prog, src.c_str(), "cfs_generated.cu", 3, headers, names);
+    const char* headers[] = {kSrcArgs, kSrcDevice, kSrcKernels, kSrcWindow};
+    const char* names[] = {"cfs_args.h", "cfs_device.cuh", "cfs_kernels.cuh", "cfs_window.cuh"};
+    nvrtcResult r = nvrtcCreateProgram(&prog, src.c_str(), "cfs_generated.cu", 4, headers, names);
     if (r != NVRTC_SUCCESS)
         return fail(CFS_ERR_COMPILE, std::string("nvrtcCreateProgram: ") + nvrtcGetErrorString(r));
     const char* opts[] = {"--gpu-architecture=sm_103a", "--fmad=false", "--std=c++17",
