@@ -565,19 +565,20 @@ cfs_status cfs_sampler_start_points(cfs_sampler* s, const cfs_system* sys, float
  *    CFS_ERR_INVALID_ARG); each frame: a 2D system of affine maps, at most
  *    2^32 - 1024 points, and targets[0] a u32 histogram; other targets are
  *    ignored.
- *  - The array (about 140 KB) exists on every GPU that loads the library,
+ *  - The array (about 200 KB) exists on every GPU that loads the library,
  *    until the process exits, and every call shares it: calls whose GPU
  *    work overlaps (other streams, other threads) race and corrupt each
  *    other.  The work and discard counters are reset on the stream at the
  *    start of each call.
  *  - The first call on a device looks up the array's device address and
- *    the grid size (cudaGetSymbolAddress, occupancy query); make that first
- *    call before any stream capture.
+ *    the SM count and raises its kernels' shared-memory limits
+ *    (cudaGetSymbolAddress, cudaFuncSetAttribute); make that first call
+ *    before any stream capture.
  *  - clear != 0 zeroes the histograms first (on the stream).
  *  - discards, if not NULL: device u64 [n_frames], set to the discarded
  *    splats of each frame.
- *  - Frame descriptors are copied from host memory with cudaMemcpyAsync,
- *    which has read its (pageable) source when it returns. */
+ *  - Frame descriptors travel as kernel arguments, which are copied at the
+ *    launch: every host array has been read when the call returns. */
 #define CFS_NOALLOC_MAX_FRAMES 256
 cfs_status cfs_render_batch_noalloc(const cfs_frame* frames, int n_frames, uint32_t iters,
                                     uint32_t burn_in, uint64_t seed, int clear,

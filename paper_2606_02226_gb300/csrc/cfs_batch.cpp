@@ -196,6 +196,20 @@ uint32_t batch_spec_defaults(ProgramSpec& sp)
     if (sp.dyn_smem > 112 * 1024) sp.min_blocks = 1;
     return tile_cap;
 }
+// Points per item of a batch as created: the plan's 4096 unless that leaves
+// CTAs without work.  With `per_cta` points for each CTA of the grid, measured
+// on GB300 (300 steps, 152 CTAs): 233 points 149 us with items of 256 against
+// 529 with 4096; 1470 points 270 us with 1024 against 555; 5500 points 702 us
+// with 2048 against 887; from 30 thousand points on 2048 and 4096 are equal,
+// and smaller items lose (a CTA that leaves a frame flushes its windows).
+uint32_t default_item_points(uint64_t points, uint32_t grid)
+{
+    const uint64_t per_cta = points / std::max(1u, grid);
+    if (per_cta >= 16384) return 4096;
+    if (per_cta >= 4096) return 2048;
+    return (uint32_t)std::min<uint64_t>(1024, std::max<uint64_t>(256, (per_cta + 255) / 256 * 256));
+}
+
 }  // namespace cfs
 
 namespace {
@@ -235,20 +249,6 @@ cfs_status plan_items(cfs_batch* b, const std::vector<uint8_t>* active = nullptr
 // dynamic shared memory of the window pre-pass: 1024 threads' 32 samples of 5
 // bytes (CFS_WIN_SMEM in cfs_window.cuh)
 constexpr int kWindowSampleBytes = 1024 * 32 * 5;
-
-// Points per item of a batch as created: the plan's 4096 unless that leaves
-// CTAs without work.  With `per_cta` points for each CTA of the grid, measured
-// on GB300 (300 steps, 152 CTAs): 233 points 149 us with items of 256 against
-// 529 with 4096; 1470 points 270 us with 1024 against 555; 5500 points 702 us
-// with 2048 against 887; from 30 thousand points on 2048 and 4096 are equal,
-// and smaller items lose (a CTA that leaves a frame flushes its windows).
-uint32_t default_item_points(uint64_t points, uint32_t grid)
-{
-    const uint64_t per_cta = points / std::max(1u, grid);
-    if (per_cta >= 16384) return 4096;
-    if (per_cta >= 4096) return 2048;
-    return (uint32_t)std::min<uint64_t>(1024, std::max<uint64_t>(256, (per_cta + 255) / 256 * 256));
-}
 
 bool window_allowed(const ProgramSpec& sp)
 {

@@ -115,6 +115,8 @@ cfs_status scribble_expand(const std::string& source, const std::string& poem, s
 // (block, occupancy, privatized window, warp aggregation, ILP); returns the
 // window's capacity in u32 counters and sets dyn_smem.
 uint32_t batch_spec_defaults(ProgramSpec& sp);
+// points per work item of a batch of `points` points on `grid` persistent CTAs
+uint32_t default_item_points(uint64_t points, uint32_t grid);
 
 // ---- density-estimation display (cfs_display.cu) ---------------------------
 // One layer as the display kernels read it.  Work is cut into items of

@@ -115,8 +115,8 @@ __device__ __forceinline__ void cfs_step_splat(const cfs_launch_args& a, const C
 
 /* Runs steps step_begin .. iters-1 of point i of system sid: one Philox
  * block per four steps.  Blocks cut by step_begin or iters run their steps
- * under warp-uniform guards (when none is cut and the burn-in ends on a
- * block boundary, a guard-free loop runs instead).  CFS_UNROLL (4, 2 or 1) is how many copies of
+ * under warp-uniform guards (when the start and the burn-in lie on block
+ * boundaries, a guard-free loop runs the whole blocks).  CFS_UNROLL (4, 2 or 1) is how many copies of
  * the step code the loop holds: the generated chain can be long, and
  * instruction-cache pressure trades against the scheduler's freedom to
  * overlap consecutive steps. */
@@ -130,18 +130,16 @@ __device__ __forceinline__ void cfs_run_point(const cfs_launch_args& a, const CH
                                               const CfsTile& tile)
 {
     const u32 b0 = a.step_begin, b1 = a.iters;
-    const bool whole = ((b0 | b1) & 3u) == 0u;
     const CfsStream ps = cfs_stream(a.rk, i, sid);
-#if !CFS_REUSE && !(CFS_BATCH && CFS_ILP == 2)
-    /* (the two-trajectory batch program calls this only for a frame's odd
-     * last point: the general loop keeps its code small) */
-    if (whole && (a.burn_in & 3u) == 0u) {
-        /* every block whole and the burn-in ending on a block boundary: the
-         * burn-in blocks move the point without the chain, the rest splat
-         * every step, and no step needs a guard (the same steps, in the same
-         * order, as the general loop below) */
+    u32 nb = b0 >> 2;
+#if !CFS_REUSE
+    if (((b0 | a.burn_in) & 3u) == 0u) {
+        /* the start and the burn-in lie on block boundaries: the burn-in
+         * blocks move the point without the chain, the other whole blocks
+         * splat every step, and no step needs a guard (the same steps, in the
+         * same order, as the general loop below, which does the last, cut
+         * block) */
         const u32 nb1 = b1 >> 2, nbs = min(max(b0, a.burn_in) >> 2, nb1);
-        u32 nb = b0 >> 2;
 #pragma unroll 1
         for (; nb < nbs; ++nb) {
             const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
@@ -178,11 +176,11 @@ __device__ __forceinline__ void cfs_run_point(const cfs_launch_args& a, const CH
             }
 #endif
         }
-        return;
     }
 #endif
 #pragma unroll 1
-    for (u32 nb = b0 >> 2; (nb << 2) < b1; ++nb) {
+    for (; (nb << 2) < b1; ++nb) {
+        const bool whole = (nb << 2) >= b0 && (nb << 2) + 4u <= b1;
         const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
         const uint4 ra = cfs_aux_block(a, i, nb, sid);
         const u32 n = nb << 2;
@@ -231,16 +229,12 @@ __device__ __forceinline__ void cfs_run_point2(const cfs_launch_args& a, const C
                                                const CfsTile& tile)
 {
     const u32 b0 = a.step_begin, b1 = a.iters;
-    const bool whole = ((b0 | b1) & 3u) == 0u;
+    u32 nb = b0 >> 2;
     const CfsStream ps0 = cfs_stream(a.rk, i0, sid), ps1 = cfs_stream(a.rk, i1, sid);
 #if !CFS_REUSE
-    if (whole && (a.burn_in & 3u) == 0u) {
-        /* every block whole and the burn-in ending on a block boundary: the
-         * burn-in blocks move the points without the chain, the rest splat
-         * every step, and no step needs a guard (the same steps, in the same
-         * order, as the general loop below) */
+    if (((b0 | a.burn_in) & 3u) == 0u) {
+        /* as in cfs_run_point: whole blocks without guards */
         const u32 nb1 = b1 >> 2, nbs = min(max(b0, a.burn_in) >> 2, nb1);
-        u32 nb = b0 >> 2;
 #pragma unroll 1
         for (; nb < nbs; ++nb) {
             const uint4 r0 = cfs_stream_block(a.rk, ps0, nb, sid);
@@ -269,11 +263,11 @@ __device__ __forceinline__ void cfs_run_point2(const cfs_launch_args& a, const C
                 cfs_step_splat(a, choose, tg, sm, w1[q], v1[q], x1, y1, z1, disc, tile);
             }
         }
-        return;
     }
 #endif
 #pragma unroll 1
-    for (u32 nb = b0 >> 2; (nb << 2) < b1; ++nb) {
+    for (; (nb << 2) < b1; ++nb) {
+        const bool whole = (nb << 2) >= b0 && (nb << 2) + 4u <= b1;
         const uint4 r0 = cfs_stream_block(a.rk, ps0, nb, sid);
         const uint4 r1 = cfs_stream_block(a.rk, ps1, nb, sid);
         const uint4 a0 = cfs_aux_block(a, i0, nb, sid);

@@ -223,13 +223,29 @@ __device__ __forceinline__ void cfs_flush_tile(const F& t, u32* cnt, const int4*
 #define CFS_WIN_THREADS 1024
 #define CFS_WIN_SMEM (CFS_WIN_THREADS * CFS_WIN_SAMPLES * 5)   /* dynamic shared bytes */
 
+#define CFS_WGP (CFS_WG + 1)             /* row pitch of the grid: a column's cells in 32 banks */
 struct CfsPlace {
-    u32 grid[CFS_WG * CFS_WG];
+    u32 grid[CFS_WG * CFS_WGP];
     u32 mass[CFS_A_MAX_MAPS];
-    int box[4];
+    int box[CFS_A_MAX_MAPS][4];
     int2 shape[CFS_WIN_SHAPES];
     unsigned long long best;
 };
+
+/* inclusive scan of 64 values of stride `step`, two per lane, by one warp */
+__device__ __forceinline__ void cfs_scan64(u32* v, int step)
+{
+    const int lane = (int)(threadIdx.x & 31u);
+    const u32 a = v[2 * lane * step], b = v[(2 * lane + 1) * step];
+    u32 s = a + b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u32 t = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += t;
+    }
+    v[2 * lane * step] = s - b;
+    v[(2 * lane + 1) * step] = s;
+}
 
 /* Window shape q (width / height = 2^(q - 2), q = 0..4): at most cap pixels,
  * inside a bw x bh box, widened to the cap once the height is clamped. */
@@ -250,70 +266,75 @@ __device__ __forceinline__ void cfs_place_windows(const F& t0, int C, u32 counte
                                                   u32* pos, unsigned char* chan, int4* out, Run run)
 {
     const u32 nt = blockDim.x, tid = threadIdx.x;
-    if (tid < CFS_A_MAX_MAPS) p.mass[tid] = 0u;
-    __syncthreads();
+    if (tid < CFS_A_MAX_MAPS) {
+        p.mass[tid] = 0u;
+        p.box[tid][0] = 0x7fffffff; p.box[tid][1] = 0x7fffffff;
+        p.box[tid][2] = -1; p.box[tid][3] = -1;
+    }
     u32 mine = 0;                       /* samples of this thread */
     run([&](int ix, int iy, int ch) {
         pos[mine * nt + tid] = (u32)ix | ((u32)iy << 16);
         chan[mine * nt + tid] = (unsigned char)ch;
-        atomicAdd(&p.mass[ch], 1u);
         ++mine;
     });
     const int2 safe_x = cfs_safe_bins(t0.x0, t0.x1, t0.sx, t0.W);
     const int2 safe_y = cfs_safe_bins(t0.y0, t0.y1, t0.sy, t0.H);
     __syncthreads();
-    u32 total = 0;
-    for (int c = 0; c < C; ++c) total += p.mass[c];
+    /* every channel's samples and box */
     for (int c = 0; c < C; ++c) {
-        /* window pixels of this channel */
-        const int cap = total ? (int)(((unsigned long long)counters * p.mass[c]) / total) : 0;
-        if (tid == 0) {
-            p.box[0] = 0x7fffffff; p.box[1] = 0x7fffffff; p.box[2] = -1; p.box[3] = -1;
-            p.best = 0ull;
-        }
-        for (u32 e = tid; e < CFS_WG * CFS_WG; e += nt) p.grid[e] = 0u;
-        __syncthreads();
         int bx0 = 0x7fffffff, by0 = 0x7fffffff, bx1 = -1, by1 = -1;
+        u32 n = 0;
         for (u32 q = 0; q < mine; ++q) {
             if (chan[q * nt + tid] != c) continue;
             const u32 v = pos[q * nt + tid];
             const int ix = (int)(v & 0xFFFFu), iy = (int)(v >> 16);
             bx0 = min(bx0, ix); by0 = min(by0, iy);
             bx1 = max(bx1, ix); by1 = max(by1, iy);
+            ++n;
         }
+        n = __reduce_add_sync(0xffffffffu, n);
+        if (n == 0u) continue;
         bx0 = __reduce_min_sync(0xffffffffu, bx0);
         by0 = __reduce_min_sync(0xffffffffu, by0);
         bx1 = __reduce_max_sync(0xffffffffu, bx1);
         by1 = __reduce_max_sync(0xffffffffu, by1);
         if ((tid & 31) == 0) {
-            atomicMin(&p.box[0], bx0); atomicMin(&p.box[1], by0);
-            atomicMax(&p.box[2], bx1); atomicMax(&p.box[3], by1);
+            atomicAdd(&p.mass[c], n);
+            atomicMin(&p.box[c][0], bx0); atomicMin(&p.box[c][1], by0);
+            atomicMax(&p.box[c][2], bx1); atomicMax(&p.box[c][3], by1);
         }
-        __syncthreads();
-        int4 box = make_int4(p.box[0], p.box[1], p.box[2], p.box[3]);
+    }
+    __syncthreads();
+    u32 total = 0;
+    for (int c = 0; c < C; ++c) total += p.mass[c];
+    for (int c = 0; c < C; ++c) {
+        /* window pixels of this channel */
+        const int cap = total ? (int)(((unsigned long long)counters * p.mass[c]) / total) : 0;
+        int4 box = make_int4(p.box[c][0], p.box[c][1], p.box[c][2], p.box[c][3]);
         const int bw = box.z - box.x + 1, bh = box.w - box.y + 1;
         if (box.z >= box.x && box.w >= box.y && cap >= 1 && (long long)bw * bh > cap) {
             /* the grid: cells of cw x ch pixels over the box, gx x gy of them */
             const int cw = (bw + CFS_WG - 1) / CFS_WG, ch = (bh + CFS_WG - 1) / CFS_WG;
             const int gx = (bw + cw - 1) / cw, gy = (bh + ch - 1) / ch;
             if (tid < CFS_WIN_SHAPES) p.shape[tid] = cfs_window_shape((int)tid, cap, bw, bh);
+            if (tid == 0) p.best = 0ull;
+            for (u32 e = tid; e < CFS_WG * CFS_WGP; e += nt) p.grid[e] = 0u;
+            __syncthreads();
+            /* a sample's cell: (v + 1/2) / cw is at least 1 / 2048 from an
+             * integer and below 64, so its rounding never moves the floor */
+            const float rw = 1.0f / (float)cw, rh = 1.0f / (float)ch;
             for (u32 q = 0; q < mine; ++q) {
                 if (chan[q * nt + tid] != c) continue;
                 const u32 v = pos[q * nt + tid];
-                atomicAdd(&p.grid[((v >> 16) - (u32)box.y) / (u32)ch * CFS_WG +
-                                  ((v & 0xFFFFu) - (u32)box.x) / (u32)cw], 1u);
+                const int i0 = (int)(((float)((int)(v & 0xFFFFu) - box.x) + 0.5f) * rw);
+                const int j0 = (int)(((float)((int)(v >> 16) - box.y) + 0.5f) * rh);
+                atomicAdd(&p.grid[j0 * CFS_WGP + i0], 1u);
             }
             __syncthreads();
             /* summed-area table: rows, then columns */
-            for (int r = (int)tid; r < gy; r += (int)nt) {
-                u32 s = 0u;
-                for (int q = 0; q < gx; ++q) p.grid[r * CFS_WG + q] = (s += p.grid[r * CFS_WG + q]);
-            }
+            for (u32 r = tid >> 5; r < CFS_WG; r += nt >> 5) cfs_scan64(p.grid + r * CFS_WGP, 1);
             __syncthreads();
-            for (int q = (int)tid; q < gx; q += (int)nt) {
-                u32 s = 0u;
-                for (int r = 0; r < gy; ++r) p.grid[r * CFS_WG + q] = (s += p.grid[r * CFS_WG + q]);
-            }
+            for (u32 r = tid >> 5; r < CFS_WG; r += nt >> 5) cfs_scan64(p.grid + r, CFS_WGP);
             __syncthreads();
             /* candidates: shape q, cell position (i0, j0); the window's whole
              * cells nw x nh are counted */
@@ -325,7 +346,7 @@ __device__ __forceinline__ void cfs_place_windows(const F& t0, int C, u32 counte
                     const int j0 = (int)(at / CFS_WG), i0 = (int)(at % CFS_WG);
                     if (i0 + nw > gx || j0 + nh > gy) continue;
                     auto sum = [&](int r, int col) -> u32 {
-                        return (r < 0 || col < 0) ? 0u : p.grid[r * CFS_WG + col];
+                        return (r < 0 || col < 0) ? 0u : p.grid[r * CFS_WGP + col];
                     };
                     const int r1 = j0 + nh - 1, c1 = i0 + nw - 1;
                     const u32 mass = sum(r1, c1) - sum(j0 - 1, c1) - sum(r1, i0 - 1) +
@@ -372,7 +393,7 @@ __device__ __forceinline__ void cfs_place_windows(const F& t0, int C, u32 counte
                         min(box.z, safe_x.x + safe_x.y - 1), min(box.w, safe_y.x + safe_y.y - 1));
         if (box.z < box.x || box.w < box.y) box = make_int4(0, 0, -1, -1);
         if (tid == 0) out[c] = box;
-        __syncthreads();                /* box, grid and best are reused */
+        __syncthreads();                /* grid, shape and best are reused */
     }
 }
 

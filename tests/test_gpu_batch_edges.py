@@ -1,4 +1,4 @@
-"""Batches whose splats meet every edge of the windowed splat and of the map
+"""Batches, and batches without allocation, whose splats meet every edge of the windowed splat and of the map
 choice table: views that cut the attractor, sizes down to one pixel, bounds
 whose scaled upper end rounds to the size or below it, several thresholds in
 one bucket, maps of probability 0.  Histograms and discards are whole numbers
@@ -60,3 +60,35 @@ def test_batch_edges_equal_the_oracle(view, iters):
             got = tens[j].cpu().numpy().view(np.uint32)
             assert np.array_equal(got.reshape(ref.buf.shape), ref.buf), (j, ilp)
             assert int(got.sum()) + int(disc[j, 0]) == n[j] * (iters - 20), (j, ilp)
+
+
+@pytest.mark.parametrize("view", VIEWS)
+@pytest.mark.parametrize("iters,burn_in", [(60, 20), (41, 18), (23, 23), (3, 0)])
+def test_noalloc_edges_equal_the_oracle(view, iters, burn_in):
+    torch = pytest.importorskip("torch")
+    from oracle import oracle as O
+    from paper_2606_02226_gb300 import cfs
+    box, w, h, c = view
+    d = W.Target("hist_u32", w, h, c, box)
+    # 51 frames (more than one launch's descriptors); frames 3 and up share one
+    # small system, so that the oracle runs it once
+    systems = _systems() + [W.sierpinski_system()] * 48
+    n = [1, 700, 2049] + [65] * 48
+    size = c * h * w
+    # targets packed without gaps: most start on no 16-byte boundary
+    flat = torch.full((size * len(systems) + 1,), 7, dtype=torch.int32, device="cuda")
+    tens = [flat[1 + size * j:1 + size * (j + 1)].view(c, h, w) for j in range(len(systems))]
+    frames = [(cfs.System(s), m, 5 * min(j, 3), min(j, 3), [d], [t])
+              for j, (s, m, t) in enumerate(zip(systems, n, tens))]
+    disc = torch.full((len(frames),), 9, dtype=torch.int64, device="cuda")
+    for _ in range(2):
+        cfs.render_batch_noalloc(frames, iters=iters, burn_in=burn_in, seed=9, discards=disc)
+    torch.cuda.synchronize()
+    assert int(flat[0]) == 7
+    for j in range(len(frames)):
+        if j <= 3:
+            ref = O.render(systems[j], [W.Op("splat", (0,))], [d], n_points=n[j], iters=iters,
+                           burn_in=burn_in, seed=9, system_id=j, point_begin=5 * j)[0].buf
+        got = tens[j].cpu().numpy().view(np.uint32)
+        assert np.array_equal(got.reshape(ref.shape), ref), j
+        assert int(got.sum()) + int(disc[j]) == n[j] * (iters - burn_in), j
