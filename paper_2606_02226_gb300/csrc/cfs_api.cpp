@@ -70,6 +70,16 @@ void derive_op_params(const cfs_transform& op, float out[CFS_OP_PARAMS])
         out[5] = v[5]; out[6] = v[6] - v[5];
         out[7] = v[7]; out[8] = v[8] - v[7];
         break;
+    case CFS_OP_BANDS: {
+        // axis, freq, phase as given; then, as integers' bits, n, base and
+        // the two constants of the modulo (cfs_bands_by)
+        out[0] = v[0]; out[1] = v[1]; out[2] = v[2];
+        const uint32_t n = (uint32_t)v[3];
+        const uint32_t w[4] = {n, (uint32_t)(int)v[4], 0xFFFFFFFFu / n,
+                               ((1u << 30) + n - 1) / n * n};
+        std::memcpy(&out[3], w, sizeof(w));
+        break;
+    }
     default:
         std::memcpy(out, v, sizeof(float) * CFS_OP_PARAMS);
         break;

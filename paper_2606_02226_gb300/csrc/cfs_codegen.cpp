@@ -270,8 +270,9 @@ static void emit_chain(std::ostringstream& s, const ProgramSpec& sp)
             break;
         case CFS_OP_BANDS: {
             const char* coord = sp.op_axis[o] == 0 ? "qx" : (sp.op_axis[o] == 1 ? "qy" : "qz");
-            s << "kc = cfs_bands(" << coord << ", " << P(o, 1) << ", " << P(o, 2) << ", (int)"
-              << P(o, 3) << ", (int)" << P(o, 4) << ");\n";
+            s << "kc = cfs_bands_by(" << coord << ", " << P(o, 1) << ", " << P(o, 2)
+              << ", __float_as_int(" << P(o, 3) << "), __float_as_int(" << P(o, 4)
+              << "), __float_as_uint(" << P(o, 5) << "), __float_as_uint(" << P(o, 6) << "));\n";
             break;
         }
         case CFS_OP_RESET:
