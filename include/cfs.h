@@ -279,7 +279,9 @@ cfs_status cfs_render_points(const cfs_chain* chain, const float* xyz, const uin
  * keys keep their order), so the permutation is unique.  Inputs xyz [dim][n]
  * and fn [n]; outputs xyz_out, fn_out (not in place) and, if not NULL,
  * perm_out [n] with xyz_out[d][j] = xyz[d][perm_out[j]].  Allocates its
- * scratch (about 16 bytes per point) stream-ordered on `stream`. */
+ * scratch (about 28 bytes per point, or 12 where that is not to be had)
+ * stream-ordered on `stream`; until its last kernel xyz_out holds
+ * intermediate keys. */
 cfs_status cfs_pointcloud_reorder(const float* xyz, const uint8_t* fn, uint32_t n, int dim,
                                   float* xyz_out, uint8_t* fn_out, uint32_t* perm_out,
                                   void* stream);
