@@ -204,6 +204,36 @@ __device__ __forceinline__ void tc_ld16_nowait(u32 taddr, u32 (&r)[16])
         : "r"(taddr));
 }
 
+// the loads of this thread so far have arrived; r (one of them) may be used
+// from here on
+__device__ __forceinline__ void tc_wait_ld(u32 (&r)[16])
+{
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
+
+// f(c0, the 16 FP32 columns c0 .. c0 + 15 of this thread's TMEM lane) for the
+// 128 columns from taddr: the next 16 are on their way while f works
+template <class F>
+__device__ __forceinline__ void tc_for_columns(u32 taddr, F f)
+{
+    u32 a[16], b[16];
+    tc_ld16_nowait(taddr, a);
+#pragma unroll 1
+    for (int c0 = 0; c0 < 128; c0 += 32) {
+        tc_wait_ld(a);
+        tc_ld16_nowait(taddr + (u32)(c0 + 16), b);
+        f(c0, a);
+        tc_wait_ld(b);
+        if (c0 + 32 < 128) tc_ld16_nowait(taddr + (u32)(c0 + 32), a);
+        f(c0 + 16, b);
+    }
+}
+
 // 16 consecutive FP32 columns of this thread's TMEM lane
 __device__ __forceinline__ void tc_ld16(u32 taddr, float (&v)[16])
 {
@@ -1638,6 +1668,20 @@ __device__ __forceinline__ void it_st16(u32 addr, u32 a, u32 b, u32 c, u32 d)
                  : "memory");
 }
 
+// a [128][K] BF16 weight matrix (16-byte aligned) into a K-major tile (K
+// groups 2048 B apart), 16 bytes = 8 columns of one row at a time: a warp's
+// lanes take 32 consecutive rows of one K group, whose shared-memory places
+// are consecutive (element by element the loop was 15 us of every launch)
+template <int K, int THREADS>
+__device__ __forceinline__ void it_stage_weights(u32 dst, const bf16r* __restrict__ w)
+{
+    for (int e = threadIdx.x; e < 128 * (K / 8); e += THREADS) {
+        const int n = e & 127, kg = e >> 7;
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(w + (size_t)n * K + 8 * kg));
+        it_st16(dst + (u32)kg * 2048u + (u32)n * 16u, v.x, v.y, v.z, v.w);
+    }
+}
+
 __device__ __forceinline__ void it_fence_async_smem()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1693,12 +1737,8 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // weights into the B-operand layout (rows = output features n, K = inputs)
-    for (int e = tid; e < HID * HID; e += IT_THREADS) {
-        const int n = e / HID, k = e % HID;
-        const u32 o = it_off(n, k, 2048u);
-        *reinterpret_cast<bf16r*>(sm + o) = wb[OFF_W2 + e];
-        *reinterpret_cast<bf16r*>(sm + IT_W + o) = wb[OFF_W3 + e];
-    }
+    it_stage_weights<HID, IT_THREADS>(sW2, wb + OFF_W2);
+    it_stage_weights<HID, IT_THREADS>(sW3, wb + OFF_W3);
     for (int e = tid; e < IT_N4 * HID; e += IT_THREADS) {
         const int n = e / HID, k = e % HID;
         *reinterpret_cast<bf16r*>(sm + 2 * IT_W + it_off(n, k, (u32)IT_N4 * 16u)) =
@@ -1766,48 +1806,59 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
     // epilogue of a hidden layer: bias, SiLU, BF16, written as the next A tile
     auto hidden_epilogue = [&](const float* bias) {
         const float4* b4 = reinterpret_cast<const float4*>(bias);
-#pragma unroll 1
-        for (int c0 = 0; c0 < HID; c0 += 16) {
-            float v[16];
-            tc_ld16(tlane + (u32)c0, v);
+        tc_for_columns(tlane, [&](int c0, const u32 (&v)[16]) {
             u32 q[8];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float4 bb = b4[c0 / 4 + j];
-                q[2 * j] = it_bf16x2(silu_fast(v[4 * j] + bb.x), silu_fast(v[4 * j + 1] + bb.y));
-                q[2 * j + 1] = it_bf16x2(silu_fast(v[4 * j + 2] + bb.z),
-                                         silu_fast(v[4 * j + 3] + bb.w));
+                q[2 * j] = it_bf16x2(silu_fast(__uint_as_float(v[4 * j]) + bb.x),
+                                     silu_fast(__uint_as_float(v[4 * j + 1]) + bb.y));
+                q[2 * j + 1] = it_bf16x2(silu_fast(__uint_as_float(v[4 * j + 2]) + bb.z),
+                                         silu_fast(__uint_as_float(v[4 * j + 3]) + bb.w));
             }
             it_st16(sA + it_off(r, c0, 2048u), q[0], q[1], q[2], q[3]);
             it_st16(sA + it_off(r, c0 + 8, 2048u), q[4], q[5], q[6], q[7]);
-        }
+        });
     };
 
     const u32 tiles = fs.tile_begin[fs.n_sys];
-    for (u32 tile = blockIdx.x * IT_GROUPS + (u32)g; tile < tiles;
-         tile += gridDim.x * IT_GROUPS) {
+    // a tile's frame, row and noise; those of the group's next tile are
+    // computed while this tile's first MMAs run
+    struct Tile {
+        int f;
+        u32 row;
+        float n0, n1;
+    };
+    auto tile_of = [&](u32 tile) {
         // the frame of this tile: last f with tile_begin[f] <= tile
         int lo = 0, hi = fs.n_sys;
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (fs.tile_begin[mid] <= tile) lo = mid; else hi = mid;
         }
-        const int f = lo;
-        const u32 row = (tile - fs.tile_begin[f]) * 128u + (u32)r;
+        Tile t;
+        t.f = lo;
+        t.row = (tile - fs.tile_begin[lo]) * 128u + (u32)r;
+        // Box-Muller on Philox (row, 0, 0, 3)
+        const uint4 q = philox_key(fs.seed[lo], t.row, 0u, 0u, TAG_NOISE);
+        const float u1 = ((float)(q.x >> 8) + 0.5f) * CFS_INV_2_24;
+        const float u2 = (float)(q.y >> 8) * CFS_INV_2_24;
+        const float rad = sqrtf(-2.0f * logf(u1));
+        float sn, cs;
+        sincosf(6.28318530717958647692f * u2, &sn, &cs);
+        t.n0 = from_bf16(to_bf16(rad * cs));
+        t.n1 = from_bf16(to_bf16(rad * sn));
+        return t;
+    };
+    u32 tile = blockIdx.x * IT_GROUPS + (u32)g;
+    Tile next = {};
+    if (tile < tiles) next = tile_of(tile);
+    for (; tile < tiles; tile += gridDim.x * IT_GROUPS) {
+        const int f = next.f;
+        const u32 row = next.row;
+        const float n0 = next.n0, n1 = next.n1;
         const u32 n = fs.count[f];
         const float* c1 = fs.c1 + (size_t)f * HID;
-        // noise of this row (Box-Muller on Philox (row, 0, 0, 3))
-        float n0, n1;
-        {
-            const uint4 q = philox_key(fs.seed[f], row, 0u, 0u, TAG_NOISE);
-            const float u1 = ((float)(q.x >> 8) + 0.5f) * CFS_INV_2_24;
-            const float u2 = (float)(q.y >> 8) * CFS_INV_2_24;
-            const float rad = sqrtf(-2.0f * logf(u1));
-            float sn, cs;
-            sincosf(6.28318530717958647692f * u2, &sn, &cs);
-            n0 = from_bf16(to_bf16(rad * cs));
-            n1 = from_bf16(to_bf16(rad * sn));
-        }
         // layer 1 (rank-2 update) into the A tile (16-byte loads of c1 and
         // of the two noise columns of W1, shared by the whole group)
         const float4* c14 = reinterpret_cast<const float4*>(c1);
@@ -1828,6 +1879,7 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
             it_st16(sA + it_off(r, c0, 2048u), q[0], q[1], q[2], q[3]);
         }
         mma_layer(sW2, 2048u, idesc128);
+        if (tile + gridDim.x * IT_GROUPS < tiles) next = tile_of(tile + gridDim.x * IT_GROUPS);
         if (!(ok = wait_layer())) break;
         hidden_epilogue(s_b2);
         mma_layer(sW3, 2048u, idesc128);
@@ -1902,16 +1954,9 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     // weights into the B-operand layout (rows = output features, K = inputs)
-    for (int e = tid; e < HID * D_IN; e += TF_THREADS) {
-        const int n = e / D_IN, k = e % D_IN;
-        *reinterpret_cast<bf16r*>(sm + it_off(n, k, 2048u)) = wb[OFF_W1 + e];
-    }
-    for (int e = tid; e < HID * HID; e += TF_THREADS) {
-        const int n = e / HID, k = e % HID;
-        const u32 o = it_off(n, k, 2048u);
-        *reinterpret_cast<bf16r*>(sm + TF_W1 + o) = wb[OFF_W2 + e];
-        *reinterpret_cast<bf16r*>(sm + TF_W1 + IT_W + o) = wb[OFF_W3 + e];
-    }
+    it_stage_weights<D_IN, TF_THREADS>(sW1, wb + OFF_W1);
+    it_stage_weights<HID, TF_THREADS>(sW2, wb + OFF_W2);
+    it_stage_weights<HID, TF_THREADS>(sW3, wb + OFF_W3);
     for (int j = tid; j < HID; j += TF_THREADS) {
         s_b1[j] = w[OFF_B1 + j];
         s_b2[j] = w[OFF_B2 + j];
@@ -1974,10 +2019,10 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
     // tile, and into global memory (row-major and / or transposed)
     auto hidden_epilogue = [&](const float* bias, int row, bool in, bf16r* H, bf16r* HT) {
         const float4* b4 = reinterpret_cast<const float4*>(bias);
-#pragma unroll 1
-        for (int c0 = 0; c0 < HID; c0 += 16) {
+        tc_for_columns(tlane, [&](int c0, const u32 (&acc)[16]) {
             float v[16];
-            tc_ld16(tlane + (u32)c0, v);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(acc[j]);
             float h[16];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
@@ -2003,7 +2048,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
                 for (int j = 0; j < 16; ++j)
                     HT[(size_t)(c0 + j) * g.ldt + row] = (bf16r)(q[j >> 1] >> (16 * (j & 1)));
             }
-        }
+        });
     };
 
     const int n_tiles = (g.B + 127) / 128;
@@ -2030,14 +2075,11 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
         // layer 3: Z3 (FP32) and H3 (BF16) out, then the output layer on
         // the BF16 activations, columns in order
         float y0 = 0.0f, y1 = 0.0f;
-#pragma unroll 1
-        for (int c0 = 0; c0 < HID; c0 += 16) {
-            float v[16];
-            tc_ld16(tlane + (u32)c0, v);
+        tc_for_columns(tlane, [&](int c0, const u32 (&v)[16]) {
             float z[16];
             u32 q[8];
 #pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = v[j] + s_b3[c0 + j];
+            for (int j = 0; j < 16; ++j) z[j] = __uint_as_float(v[j]) + s_b3[c0 + j];
 #pragma unroll
             for (int j = 0; j < 8; ++j) q[j] = pack_bf16x2(silu_f(z[2 * j]), silu_f(z[2 * j + 1]));
 #pragma unroll
@@ -2055,7 +2097,7 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
                 hp[0] = make_uint4(q[0], q[1], q[2], q[3]);
                 hp[1] = make_uint4(q[4], q[5], q[6], q[7]);
             }
-        }
+        });
         tc_fence_before();          // TMEM read: the next tile's MMAs may overwrite it
         if (in) {
             g.Y[2 * (size_t)row] = y0 + s_b4[0];
