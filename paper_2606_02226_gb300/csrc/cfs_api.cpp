@@ -333,6 +333,13 @@ void fill_args(cfs_launch_args* a, const cfs_system* sys, const cfs_chain* ch,
     a->sys.n_maps = sys->n_maps;
     a->sys.n_cmp = sys->n_cmp;
     a->sys.dim = sys->dim;
+    // equal probabilities: k = w >> shift for every word
+    for (int b = 1; b <= 4; ++b) {
+        bool equal = sys->n_cmp == (1 << b) - 1;
+        for (int j = 0; equal && j < sys->n_cmp; ++j)
+            equal = sys->T[j] == (uint32_t)(j + 1) << (32 - b);
+        if (equal) a->sys.shift = 32 - b;
+    }
     for (int k = 0; k < sys->n_maps; ++k)
         for (int j = 0; j < 12; ++j) a->sys.prm[j][k] = sys->maps[k].params[j];
     for (int o = 0; o < ch->n_xops; ++o) derive_op_params(ch->xops[o], a->op[o]);

@@ -24,7 +24,8 @@ typedef struct {
 
 typedef struct {
     unsigned int T[CFS_A_MAX_MAPS];     /* thresholds < 2^32, ascending; n_cmp used */
-    int n_maps, n_cmp, dim, pad;
+    int n_maps, n_cmp, dim;
+    int shift;                          /* 32 - b for 2^b (b >= 1) equally likely maps, else 0 */
     float prm[12][CFS_A_MAX_MAPS];      /* map parameters, SoA: prm[j][k] */
 } cfs_dev_system;
 
