@@ -104,7 +104,8 @@ int device_sm_count();
 // 2D tensor map (TMA) of a BF16 matrix [rows][cols], row stride ld elements,
 // box_rows x box_cols boxes, no swizzle, zeros outside (cfs_runtime.cpp)
 cfs_status make_tmap_2d_bf16(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows,
-                             uint64_t ld, uint32_t box_cols, uint32_t box_rows);
+                             uint64_t ld, uint32_t box_cols, uint32_t box_rows,
+                             bool swizzle = false);
 
 // Expands poem `poem` of a scribble program into a chain body; splat(N)
 // calls become CFS_SCRIBBLE_SPLAT_i() with their slots in splat_slots.

@@ -154,9 +154,10 @@ cfs_status compile(const std::string& src, std::vector<char>* cubin, std::string
 }  // namespace
 
 // 2D tensor map of a BF16 matrix [rows][cols] (row stride ld elements), boxes
-// of box_rows x box_cols elements, no swizzle, zero fill outside the matrix
+// of box_rows x box_cols elements, without swizzle or (rows of 128 bytes in the
+// box) with the 128-byte swizzle, zero fill outside the matrix
 cfs_status make_tmap_2d_bf16(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows,
-                             uint64_t ld, uint32_t box_cols, uint32_t box_rows)
+                             uint64_t ld, uint32_t box_cols, uint32_t box_rows, bool swizzle)
 {
     Driver& d = driver();
     if (!d.ok) return fail(CFS_ERR_CUDA, d.why);
@@ -169,7 +170,8 @@ cfs_status make_tmap_2d_bf16(CUtensorMap* map, const void* base, uint64_t cols, 
     const cuuint32_t estr[2] = {1, 1};
     return check_cu(d.encode_tiled(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base),
                                    dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                   swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                                   CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE),
                     "cuTensorMapEncodeTiled");
 }

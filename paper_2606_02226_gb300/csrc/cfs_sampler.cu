@@ -763,50 +763,108 @@ __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
     }
 }
 
-// ---------------------------------------------------------------------------
-// Weight gradients dW[M = 128][N] += A[128][K] B[N][K]^T (A = dZ^T, B = H^T or
-// U^T, both K-major over the rows, N = 128 or 64) split over K: CTA b takes
-// a run of 64-row K chunks.  Warp 0 loads each chunk's A and B with TMA into
-// a ring of SK_STAGES slots, one thread of warp 1 accumulates the chunks into
-// one TMEM accumulator, and warps 2..5 add it to dW with vector reductions at
-// the end.  Every wait is bounded, as in tc_rows_kernel.
-// ---------------------------------------------------------------------------
-constexpr int SK_STAGES = 4;
-constexpr int SK_THREADS = 32 * 6;
-constexpr int SK_SLOT = 2 * 128 * TC_K * 2;   // A and B chunk (64 K) of 128 rows each
-constexpr int SK_SMEM = 1024 + SK_STAGES * SK_SLOT + 256;
-
-__global__ void __launch_bounds__(SK_THREADS, 1) tc_splitk_kernel(
-    const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-    const __grid_constant__ TcArgs g)
+// sums of the gradient copies in bias_part (the output layer's and the bias
+// gradients) added to grads, by one block
+constexpr int OB_PART = 3 * HID + 4;
+constexpr int PART_FLOATS = TC_COPIES * (2 * HID + OB_PART);
+__device__ __forceinline__ void part_reduce(const float* __restrict__ part, float* grads)
 {
-    extern __shared__ unsigned char sk_smem_raw[];
+    for (int e = threadIdx.x; e < 2 * HID + 3 * HID + 2; e += blockDim.x) {
+        float s = 0.0f;
+        if (e < 2 * HID) {
+            const int l = e / HID, c = e % HID;
+            for (int k = 0; k < TC_COPIES; ++k) s += part[((size_t)l * TC_COPIES + k) * HID + c];
+            grads[(l == 0 ? OFF_B2 : OFF_B1) + c] += s;
+        } else {
+            const int q = e - 2 * HID;
+            const float* ob = part + (size_t)2 * TC_COPIES * HID;
+            for (int k = 0; k < TC_COPIES; ++k) s += ob[(size_t)k * OB_PART + q];
+            grads[q < 2 * HID ? OFF_W4 + q : (q < 3 * HID ? OFF_B3 + q - 2 * HID
+                                                          : OFF_B4 + q - 3 * HID)] += s;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The three weight gradients dW_l[128][N] += dZ_l^T A (A: the layer's input, N
+// = 128, 128 or 64) in one launch, split over the rows: the CTAs are dealt to
+// the gradients in proportion to what they read, and each takes a run of
+// 64-row chunks.  Both operands are the row-major activations themselves:
+// their rows are the contraction, so they are MN-major operands (transpose
+// bits of the instruction descriptor) and nothing has to be stored
+// transposed.  A chunk is one or two TMA boxes of 64 rows x 64 features an
+// operand (128-byte swizzle).  Warp 0 loads the chunks into a ring of
+// DW_STAGES slots, one thread of warp 1 accumulates them into one TMEM
+// accumulator, and warps 2..5 add it to dW with vector reductions at the end.
+// One more CTA sums the bias-gradient copies.  Every wait is bounded, as in
+// tc_rows_kernel.
+// What it measured (65536 rows): 54 us for three launches on K-major operands,
+// whose 16-byte box rows the TMA unit took one by one, besides the transposed
+// copies that every producer wrote.
+// ---------------------------------------------------------------------------
+constexpr int DW_STAGES = 4;
+constexpr int DW_THREADS = 32 * 6;
+constexpr int DW_ROWS = 64;
+constexpr int DW_BOX = DW_ROWS * 128;         // 64 rows x 64 BF16 features
+constexpr int DW_SLOT = 4 * DW_BOX;           // A and B chunk of up to 128 features each
+constexpr int DW_SMEM = 1024 + DW_STAGES * DW_SLOT + 256;
+
+// MN-major operand with the 128-byte swizzle: 64 features of 8 rows are one
+// 1024-byte atom; 8-row groups 1024 B apart (stride offset), 64-feature
+// blocks DW_BOX apart (leading offset); swizzle mode 2 at bit 61
+__device__ __forceinline__ u64 tc_desc_mn(u32 saddr)
+{
+    return (u64)((saddr >> 4) & 0x3FFFu) | ((u64)((u32)DW_BOX >> 4) << 16) |
+           ((u64)(1024u >> 4) << 32) | ((u64)1 << 46) | ((u64)2 << 61);
+}
+
+struct DwArgs {
+    int chunks;                  // of DW_ROWS rows
+    int cta0[4];                 // first CTA of each gradient, and the end
+    int N[3];
+    float* C[3];                 // [128][N]
+    const float* part;           // the bias-gradient copies and
+    float* grads;                // where their sums go
+};
+
+struct DwMaps {
+    CUtensorMap a[3], b[3];
+};
+
+__global__ void __launch_bounds__(DW_THREADS, 1) tc_dw_kernel(const __grid_constant__ DwMaps maps,
+                                                              const __grid_constant__ DwArgs g)
+{
+    extern __shared__ unsigned char dw_smem_raw[];
+    if ((int)blockIdx.x >= g.cta0[3]) {
+        part_reduce(g.part, g.grads);
+        return;
+    }
     unsigned char* sm = reinterpret_cast<unsigned char*>(
-        (reinterpret_cast<uintptr_t>(sk_smem_raw) + 1023) & ~(uintptr_t)1023);
+        (reinterpret_cast<uintptr_t>(dw_smem_raw) + 1023) & ~(uintptr_t)1023);
     const u32 s0 = smem_addr(sm);
-    u64* bars = reinterpret_cast<u64*>(sm + SK_STAGES * SK_SLOT);
+    u64* bars = reinterpret_cast<u64*>(sm + DW_STAGES * DW_SLOT);
     auto full = [&](int s) { return smem_addr(&bars[s]); };
-    auto empty = [&](int s) { return smem_addr(&bars[SK_STAGES + s]); };
-    const u32 tdone = smem_addr(&bars[2 * SK_STAGES]);
+    auto empty = [&](int s) { return smem_addr(&bars[DW_STAGES + s]); };
+    const u32 tdone = smem_addr(&bars[2 * DW_STAGES]);
     u32* s_tmem = reinterpret_cast<u32*>(bars + 16);
     __shared__ int s_err;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_chunks = (g.K + TC_K - 1) / TC_K;
-    const int per = (n_chunks + gridDim.x - 1) / gridDim.x;
-    const int c_first = blockIdx.x * per, c_last = min(n_chunks, c_first + per);
-    const u32 chunk_bytes = (u32)((128 + g.N) * TC_K * 2);
-    const u32 ncols = g.N <= 64 ? 64u : 128u;
+    const int p = (int)blockIdx.x < g.cta0[1] ? 0 : ((int)blockIdx.x < g.cta0[2] ? 1 : 2);
+    const int ctas = g.cta0[p + 1] - g.cta0[p], N = g.N[p];
+    const int per = (g.chunks + ctas - 1) / ctas;
+    const int c_first = min(g.chunks, ((int)blockIdx.x - g.cta0[p]) * per);
+    const int c_last = min(g.chunks, c_first + per);
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :
-                     : "r"(smem_addr(s_tmem)), "r"(ncols)
+                     : "r"(smem_addr(s_tmem)), "r"(128u)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x == 0) {
         s_err = 0;
-        for (int s = 0; s < SK_STAGES; ++s) {
+        for (int s = 0; s < DW_STAGES; ++s) {
             mbar_init(full(s), 1u);
             mbar_init(empty(s), 1u);
         }
@@ -817,42 +875,44 @@ __global__ void __launch_bounds__(SK_THREADS, 1) tc_splitk_kernel(
     __syncthreads();
     tc_fence_after();
     const u32 tmem = *s_tmem;
-    // slot s: A at s0 + s SLOT ([8 K columns][128 rows][16 B]), B after 16 KB
+    // slot s: A at s0 + s DW_SLOT (two boxes), B after it (N / 64 boxes)
     if (warp == 0) {
         if (lane == 0) {
+            const CUtensorMap* ma = &maps.a[p];
+            const CUtensorMap* mb = &maps.b[p];
             int i = 0, issued = 0;
             for (int c = c_first; c < c_last; ++c, ++i) {
-                const int s = i % SK_STAGES;
-                if (i >= SK_STAGES && !mbar_wait(empty(s), (u32)(i / SK_STAGES - 1) & 1u)) {
+                const int s = i % DW_STAGES;
+                if (i >= DW_STAGES && !mbar_wait(empty(s), (u32)(i / DW_STAGES - 1) & 1u)) {
                     atomicExch(&s_err, 1);
                     break;
                 }
-                mbar_expect_tx(full(s), chunk_bytes);
-                const u32 a = s0 + (u32)(s * SK_SLOT), b = a + 128 * TC_K * 2;
-                for (int kc = 0; kc < TC_K / 8; ++kc) {
-                    tma_load_2d(a + kc * 2048, &tmA, c * TC_K + kc * 8, 0, full(s));
-                    tma_load_2d(b + kc * (u32)(g.N * 16), &tmB, c * TC_K + kc * 8, 0, full(s));
-                }
+                mbar_expect_tx(full(s), (u32)((2 + N / 64) * DW_BOX));
+                const u32 a = s0 + (u32)(s * DW_SLOT);
+                tma_load_2d(a, ma, 0, c * DW_ROWS, full(s));
+                tma_load_2d(a + DW_BOX, ma, 64, c * DW_ROWS, full(s));
+                tma_load_2d(a + 2 * DW_BOX, mb, 0, c * DW_ROWS, full(s));
+                if (N == 128) tma_load_2d(a + 3 * DW_BOX, mb, 64, c * DW_ROWS, full(s));
                 issued = i + 1;
             }
-            for (int j = (issued > SK_STAGES ? issued - SK_STAGES : 0); j < issued; ++j)
-                mbar_wait(full(j % SK_STAGES), (u32)(j / SK_STAGES) & 1u);
+            for (int j = (issued > DW_STAGES ? issued - DW_STAGES : 0); j < issued; ++j)
+                mbar_wait(full(j % DW_STAGES), (u32)(j / DW_STAGES) & 1u);
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const u32 idesc = tc_idesc(g.N);
+            // both operands MN-major: transpose bits 15 and 16
+            const u32 idesc = tc_idesc(N) | (1u << 15) | (1u << 16);
             bool ok = true;
             int i = 0;
             for (int c = c_first; c < c_last; ++c, ++i) {
-                const int s = i % SK_STAGES;
-                if (!mbar_wait(full(s), (u32)(i / SK_STAGES) & 1u)) { ok = false; break; }
+                const int s = i % DW_STAGES;
+                if (!mbar_wait(full(s), (u32)(i / DW_STAGES) & 1u)) { ok = false; break; }
                 tc_fence_after();
-                const u32 a = s0 + (u32)(s * SK_SLOT), b = a + 128 * TC_K * 2;
+                const u32 a = s0 + (u32)(s * DW_SLOT);
 #pragma unroll
-                for (int kk = 0; kk < TC_K / 16; ++kk)
-                    tc_mma(tmem, tc_desc_kn(a + kk * 4096, 2048u, 128u),
-                           tc_desc_kn(b + kk * (u32)(g.N * 32), (u32)(g.N * 16), 128u), idesc,
-                           (i > 0 || kk > 0) ? 1u : 0u);
+                for (int kk = 0; kk < DW_ROWS / 16; ++kk)      // 16 rows: two 1024-byte groups
+                    tc_mma(tmem, tc_desc_mn(a + kk * 2048), tc_desc_mn(a + 2 * DW_BOX + kk * 2048),
+                           idesc, (i > 0 || kk > 0) ? 1u : 0u);
                 tc_commit(empty(s));
             }
             if (!ok) atomicExch(&s_err, 1);
@@ -867,11 +927,14 @@ __global__ void __launch_bounds__(SK_THREADS, 1) tc_splitk_kernel(
             tc_fence_after();
             const int row = quad * 32 + lane;
             const u32 base = tmem + ((u32)(quad * 32) << 16);
-            const float zi[16] = {};
-            for (int c0 = 0; c0 < g.N; c0 += 16) {
+            for (int c0 = 0; c0 < N; c0 += 16) {
                 float v[16];
                 tc_ld16(base + (u32)c0, v);
-                tc_epilogue(g, row, c0, v, zi, nullptr, nullptr);
+                float* c = g.C[p] + (size_t)row * N + c0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    cfs_red_add_v4f32(c + 4 * q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2],
+                                                             v[4 * q + 3]));
             }
         }
     }
@@ -881,7 +944,7 @@ __global__ void __launch_bounds__(SK_THREADS, 1) tc_splitk_kernel(
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(ncols)
+                     "r"(128u)
                      : "memory");
     }
 }
@@ -916,34 +979,18 @@ __global__ void __launch_bounds__(256) out_forward_kernel(const bf16r* __restric
     Y[2 * r + 1] = y1 + w[OFF_B4 + 1];
 }
 
-// gradient partial sums gathered in TC_COPIES copies to spread the atomics:
+// bias_part: gradient partial sums in TC_COPIES copies to spread the atomics:
 // [2][TC_COPIES][HID] bias gradients b2 and b1 (GEMM epilogues), then
 // [TC_COPIES][OB_PART] of the output layer's backward: W4 rows 0 and 1
 // (2 x HID), b3 (HID), b4 (2), padding
-constexpr int OB_PART = 3 * HID + 4;
-constexpr int PART_FLOATS = TC_COPIES * (2 * HID + OB_PART);
-
-// sums the copies and adds them to grads
 __global__ void __launch_bounds__(512) part_reduce_kernel(const float* __restrict__ part,
                                                           float* grads)
 {
-    for (int e = threadIdx.x; e < 2 * HID + 3 * HID + 2; e += blockDim.x) {
-        float s = 0.0f;
-        if (e < 2 * HID) {
-            const int l = e / HID, c = e % HID;
-            for (int k = 0; k < TC_COPIES; ++k) s += part[((size_t)l * TC_COPIES + k) * HID + c];
-            grads[(l == 0 ? OFF_B2 : OFF_B1) + c] += s;
-        } else {
-            const int q = e - 2 * HID;
-            const float* ob = part + (size_t)2 * TC_COPIES * HID;
-            for (int k = 0; k < TC_COPIES; ++k) s += ob[(size_t)k * OB_PART + q];
-            grads[q < 2 * HID ? OFF_W4 + q : (q < 3 * HID ? OFF_B3 + q - 2 * HID
-                                                          : OFF_B4 + q - 3 * HID)] += s;
-        }
-    }
+    part_reduce(part, grads);
 }
 
-// U [rows][D_IN] -> UT [D_IN][ldt] (the K-major operand of dW1)
+// U [rows][D_IN] -> UT [D_IN][ldt] (the K-major operand of dW1; batches of
+// fewer than 128 rows)
 __global__ void __launch_bounds__(256) transpose_in_kernel(const bf16r* __restrict__ U, int rows,
                                                            bf16r* UT, int ldt)
 {
@@ -964,8 +1011,8 @@ __global__ void __launch_bounds__(256) transpose_in_kernel(const bf16r* __restri
 // dH3 * silu'(Z3) written as dZ3 and its transpose dZ3^T; dW4 = dY^T H3,
 // db3 = sum dZ3, db4 = sum dY.  A block takes OB_ROWS rows, a warp one row
 // at a time, lane l the four units 4l .. 4l+3 (16-byte loads of Z3, 8-byte
-// loads of H3); the block's dZ3 tile is transposed in shared memory, and its
-// sums combine across warps there before one atomic per value into copy
+// loads of H3); with dZ3T (batches of fewer than 128 rows) the block's dZ3
+// tile is transposed in shared memory; its sums combine across warps there before one atomic per value into copy
 // blockIdx.x % TC_COPIES of `part`.
 constexpr int OB_ROWS = 64;
 constexpr int OB_THREADS = 256;
@@ -1007,7 +1054,7 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
             const float dh = fmaf(y0, w0[j], y1 * w1[j]);
             const float d = dh * silu_grad_f(zz[j]);
             db[j] = to_bf16(d);
-            tT[c + j][k] = db[j];
+            if (dZ3T) tT[c + j][k] = db[j];
             ab[j] += d;
             a0[j] = fmaf(y0, h[j], a0[j]);
             a1[j] = fmaf(y1, h[j], a1[j]);
@@ -1029,7 +1076,7 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
         atomicAdd(&s_sum[3 * HID + 1], b41);
     }
     // dZ3^T rows: a warp writes 64 consecutive rows of one unit as 32 words
-    for (int e = threadIdx.x; e < HID * (OB_ROWS / 2); e += OB_THREADS) {
+    for (int e = threadIdx.x; dZ3T && e < HID * (OB_ROWS / 2); e += OB_THREADS) {
         const int u = e / (OB_ROWS / 2), jp = 2 * (e % (OB_ROWS / 2));
         const int r = r0 + jp;
         if (r + 1 < B) {
@@ -1918,11 +1965,8 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
 // group's A tile; layer 1 (K = 64), layer 2 and layer 3 run as tcgen05.mma
 // chains into the group's TMEM columns, each epilogue adding the bias,
 // applying SiLU and writing the next A tile in place.  What the backward
-// pass reads is written on the way: H1 (row-major: the input of the
-// recomputed Z2) and its transpose, H2's transpose, H3 and Z3 (the output
-// layer's backward); the output layer itself (N = 2) runs on the CUDA cores
-// in the layer-3 epilogue.  H2 in row-major form, which only the next
-// layer's GEMM read, never leaves the chip.
+// pass reads is written on the way, row-major: H1, H2, H3 and Z3; the output
+// layer itself (N = 2) runs on the CUDA cores in the layer-3 epilogue.
 // ---------------------------------------------------------------------------
 constexpr int TF_GROUPS = 4;
 constexpr int TF_THREADS = 128 * TF_GROUPS;
@@ -1932,8 +1976,7 @@ constexpr int TF_SMEM = 1024 + TF_W1 + 2 * IT_W + TF_GROUPS * IT_A + 256;
 struct TrainFwdArgs {
     const bf16r* U;                // [B][D_IN]
     int B;
-    bf16r *H1, *H1T, *H2T, *H3;    // H1, H3 [B][HID]; transposes [HID][ldt]
-    int ldt;
+    bf16r *H1, *H2, *H3;           // [B][HID]
     float *Z3, *Y;                 // Z3 [B][HID], Y [B][2]
 };
 
@@ -2016,39 +2059,41 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
         return done;
     };
     // epilogue of layers 1 and 2: H = SiLU(acc + b) as BF16 into the next A
-    // tile, and into global memory (row-major and / or transposed)
-    auto hidden_epilogue = [&](const float* bias, int row, bool in, bf16r* H, bf16r* HT) {
+    // tile
+    auto hidden_epilogue = [&](const float* bias) {
         const float4* b4 = reinterpret_cast<const float4*>(bias);
         tc_for_columns(tlane, [&](int c0, const u32 (&acc)[16]) {
-            float v[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(acc[j]);
-            float h[16];
+            u32 q[8];
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const float4 bb = b4[c0 / 4 + j];
-                h[4 * j] = silu_f(v[4 * j] + bb.x);
-                h[4 * j + 1] = silu_f(v[4 * j + 1] + bb.y);
-                h[4 * j + 2] = silu_f(v[4 * j + 2] + bb.z);
-                h[4 * j + 3] = silu_f(v[4 * j + 3] + bb.w);
+                q[2 * j] = pack_bf16x2(silu_f(__uint_as_float(acc[4 * j]) + bb.x),
+                                       silu_f(__uint_as_float(acc[4 * j + 1]) + bb.y));
+                q[2 * j + 1] = pack_bf16x2(silu_f(__uint_as_float(acc[4 * j + 2]) + bb.z),
+                                           silu_f(__uint_as_float(acc[4 * j + 3]) + bb.w));
             }
-            u32 q[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) q[j] = pack_bf16x2(h[2 * j], h[2 * j + 1]);
             it_st16(sA + it_off(r, c0, 2048u), q[0], q[1], q[2], q[3]);
             it_st16(sA + it_off(r, c0 + 8, 2048u), q[4], q[5], q[6], q[7]);
-            if (in && H) {
-                uint4* hp = reinterpret_cast<uint4*>(H + (size_t)row * HID + c0);
-                hp[0] = make_uint4(q[0], q[1], q[2], q[3]);
-                hp[1] = make_uint4(q[4], q[5], q[6], q[7]);
-            }
-            if (in && HT) {
-                // consecutive lanes hold consecutive rows: each column's stores coalesce
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    HT[(size_t)(c0 + j) * g.ldt + row] = (bf16r)(q[j >> 1] >> (16 * (j & 1)));
-            }
         });
+    };
+    // the group's A tile to rows row0 .. of H, while the MMAs read it too: a
+    // warp's lanes take 8 rows x 4 K groups, which leave shared memory
+    // without conflicts and arrive in 64-byte runs (a row per lane, straight
+    // from the epilogue, was 32 lines an instruction)
+    auto store_tile = [&](bf16r* H, int row0) {
+        const int rr = lane & 7, kq = lane >> 3;
+#pragma unroll 4
+        for (int e = 0; e < 16; ++e) {
+            const int rt = wq * 32 + (e >> 2) * 8 + rr, kg = (e & 3) * 4 + kq;
+            u32 v[4];
+            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                         : "r"(sA + it_off(rt, 8 * kg, 2048u))
+                         : "memory");
+            if (row0 + rt < g.B)
+                *reinterpret_cast<uint4*>(H + (size_t)(row0 + rt) * HID + 8 * kg) =
+                    make_uint4(v[0], v[1], v[2], v[3]);
+        }
     };
 
     const int n_tiles = (g.B + 127) / 128;
@@ -2066,11 +2111,13 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
         }
         mma_layer(sW1, D_IN);
         if (!(ok = wait_layer())) break;
-        hidden_epilogue(s_b1, row, in, g.H1, g.H1T);
+        hidden_epilogue(s_b1);
         mma_layer(sW2, HID);
+        store_tile(g.H1, tile * 128);
         if (!(ok = wait_layer())) break;
-        hidden_epilogue(s_b2, row, in, nullptr, g.H2T);
+        hidden_epilogue(s_b2);
         mma_layer(sW3, HID);
+        store_tile(g.H2, tile * 128);
         if (!(ok = wait_layer())) break;
         // layer 3: Z3 (FP32) and H3 (BF16) out, then the output layer on
         // the BF16 activations, columns in order
@@ -2093,12 +2140,14 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
                     zp[j] = make_float4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
-                uint4* hp = reinterpret_cast<uint4*>(g.H3 + (size_t)row * HID + c0);
-                hp[0] = make_uint4(q[0], q[1], q[2], q[3]);
-                hp[1] = make_uint4(q[4], q[5], q[6], q[7]);
             }
+            it_st16(sA + it_off(r, c0, 2048u), q[0], q[1], q[2], q[3]);
+            it_st16(sA + it_off(r, c0 + 8, 2048u), q[4], q[5], q[6], q[7]);
         });
         tc_fence_before();          // TMEM read: the next tile's MMAs may overwrite it
+        it_group_sync(gi);
+        store_tile(g.H3, tile * 128);
+        it_group_sync(gi);          // the next tile's inputs go into the A tile
         if (in) {
             g.Y[2 * (size_t)row] = y0 + s_b4[0];
             g.Y[2 * (size_t)row + 1] = y1 + s_b4[1];
@@ -2143,11 +2192,12 @@ struct cfs_sampler {
     bool upload_pending = false;
     // activations for B rows (grown on demand)
     int cap_rows = 0;
-    int ldt = 0;             // row stride of the transposed copies (>= cap_rows)
+    int ldt = 0;             // row stride of the transposed copies (TC_M)
     unsigned char* act = nullptr;
     float *Z1, *Z2, *Z3, *Y;
     bf16r *H1, *H2, *H3, *dZ1, *dZ2, *dZ3;
     // transposed copies [features][ldt]: the K-major operands of dW = dZ^T A
+    // of batches of fewer than TC_M rows
     bf16r *UT, *H1T, *H2T, *dZ1T, *dZ2T, *dZ3T;
 };
 
@@ -2161,7 +2211,7 @@ cfs_status ensure_rows(cfs_sampler* s, int B)
     s->act = nullptr;
     s->cap_rows = 0;
     const size_t fz = (size_t)B * HID * 4, fh = (size_t)B * HID * 2;
-    const int ldt = (B + 63) / 64 * 64;
+    const int ldt = TC_M;    // the transposed copies serve batches of fewer rows only
     const size_t ft = (size_t)ldt * HID * 2, fu = (size_t)ldt * D_IN * 2;
     const size_t bytes = 3 * fz + (size_t)B * 2 * 4 + 6 * fh + 5 * ft + fu + 13 * 256;
     cfs_status st = check_cuda(cudaMalloc(&s->act, bytes), "cudaMalloc(sampler activations)");
@@ -2274,38 +2324,8 @@ cfs_status tc_rows(cudaStream_t st, int M, int K, const bf16r* A, int lda, const
     return CFS_OK;
 }
 
-// weight gradient C[128][N] += A[128][K] B[N][K]^T on the split-K TMA kernel
-// (N = 128 or 64)
-cfs_status tc_splitk(cudaStream_t st, int N, int K, const bf16r* A, int lda, const bf16r* Bm,
-                     int ldb, float* C, int ldc)
-{
-    // fewer rows than one chunk: the register-staged kernel (as in tc_rows)
-    if (K > 0 && K < TC_K) {
-        const int splits = std::max(1, std::min(256, K / 256));
-        return tc_gemm(st, HID, N, K, A, lda, Bm, ldb, EPI_ATOMIC, nullptr, C, ldc, nullptr, 0,
-                       nullptr, 0, nullptr, 0, nullptr, splits);
-    }
-    if (K < 1) return CFS_OK;
-    if (!(N == 64 || N == 128) || lda % 8 || ldb % 8 || (uintptr_t)C % 16 || ldc % 4)
-        return fail(CFS_ERR_INVALID_ARG, "weight-gradient GEMM operands not aligned");
-    CUtensorMap ta, tb;
-    cfs_status r = make_tmap_2d_bf16(&ta, A, (uint64_t)K, 128u, (uint64_t)lda, 8u, 128u);
-    if (r == CFS_OK)
-        r = make_tmap_2d_bf16(&tb, Bm, (uint64_t)K, (uint64_t)N, (uint64_t)ldb, 8u, (uint32_t)N);
-    if (r != CFS_OK) return r;
-    TcArgs g;
-    std::memset(&g, 0, sizeof(g));
-    g.M = HID; g.N = N; g.K = K;
-    g.A = A; g.lda = lda; g.B = Bm; g.ldb = ldb;
-    g.k_split = K;
-    g.mode = EPI_ATOMIC; g.C = C; g.ldc = ldc;
-    const int chunks = (K + TC_K - 1) / TC_K;
-    const int sms = std::max(1, device_sm_count());
-    tc_splitk_kernel<<<std::min(chunks, sms), SK_THREADS, SK_SMEM, st>>>(ta, tb, g);
-    return CFS_OK;
-}
-
-// forward of B rows of U: Z1..Z3 (fp32), H1..H3 (bf16), H1^T, H2^T, Y (fp32 [B][2])
+// forward of B rows of U: H1..H3 (bf16), Z3 (fp32), Y (fp32 [B][2]); with fewer
+// rows than one tile also Z1, Z2, H1^T, H2^T
 cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
 {
     const bf16r* wb = s->wb;
@@ -2322,23 +2342,22 @@ cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
         }
         TrainFwdArgs a;
         a.U = U; a.B = B;
-        a.H1 = s->H1; a.H1T = s->H1T; a.H2T = s->H2T; a.H3 = s->H3;
-        a.ldt = s->ldt; a.Z3 = s->Z3; a.Y = s->Y;
+        a.H1 = s->H1; a.H2 = s->H2; a.H3 = s->H3;
+        a.Z3 = s->Z3; a.Y = s->Y;
         const int tiles = (B + 127) / 128;
         const int grid = std::max(1, std::min(device_sm_count(), (tiles + TF_GROUPS - 1) / TF_GROUPS));
         train_fwd_kernel<<<grid, TF_THREADS, TF_SMEM, st>>>(wb, s->w, a);
         return check_cuda(cudaGetLastError(), "train_fwd_kernel launch");
     }
-    // Z1 and Z2 only where the backward reads them (it recomputes them on
-    // tc_rows_kernel); Z3 always (the output layer's backward reads it)
-    const bool keep_z = !rows_on_tma(B);
+    // Z1, Z2 and the transposed copies only where the backward reads them
+    const bool small = !rows_on_tma(B);
     cfs_status r = tc_rows(st, B, D_IN, U, D_IN, wb + OFF_W1, D_IN, EPI_SILU, s->w + OFF_B1,
-                           keep_z ? s->Z1 : nullptr, HID, s->H1, HID, s->H1T, s->ldt, nullptr, 0,
-                           nullptr);
+                           small ? s->Z1 : nullptr, HID, s->H1, HID, small ? s->H1T : nullptr,
+                           s->ldt, nullptr, 0, nullptr);
     if (r == CFS_OK)
         r = tc_rows(st, B, HID, s->H1, HID, wb + OFF_W2, HID, EPI_SILU, s->w + OFF_B2,
-                    keep_z ? s->Z2 : nullptr, HID, s->H2, HID, s->H2T, s->ldt, nullptr, 0,
-                    nullptr);
+                    small ? s->Z2 : nullptr, HID, s->H2, HID, small ? s->H2T : nullptr, s->ldt,
+                    nullptr, 0, nullptr);
     if (r == CFS_OK)
         r = tc_rows(st, B, HID, s->H2, HID, wb + OFF_W3, HID, EPI_SILU, s->w + OFF_B3, s->Z3, HID,
                     s->H3, HID, nullptr, 0, nullptr, 0, nullptr);
@@ -2347,35 +2366,78 @@ cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
     return CFS_OK;
 }
 
+// the weight gradients of W1..W3 and the sums of the bias-gradient copies
+// (B >= 128 rows)
+cfs_status tc_dw(cfs_sampler* s, const bf16r* U, int B, float* grads, cudaStream_t st)
+{
+    const bf16r* dz[3] = {s->dZ3, s->dZ2, s->dZ1};
+    const bf16r* in[3] = {s->H2, s->H1, U};
+    DwMaps m;
+    DwArgs g;
+    std::memset(&g, 0, sizeof(g));
+    g.chunks = (B + DW_ROWS - 1) / DW_ROWS;
+    g.part = s->bias_part;
+    g.grads = grads;
+    const int off[3] = {OFF_W3, OFF_W2, OFF_W1};
+    // CTAs in proportion to the bytes read (256, 256 and 192 B a row)
+    const int sms = std::max(3, device_sm_count());
+    const int n01 = std::max(1, std::min(g.chunks, sms * 256 / 704));
+    const int n2 = std::max(1, std::min(g.chunks, sms - 2 * n01));
+    g.cta0[1] = n01;
+    g.cta0[2] = 2 * n01;
+    g.cta0[3] = 2 * n01 + n2;
+    for (int l = 0; l < 3; ++l) {
+        g.N[l] = l == 2 ? D_IN : HID;
+        g.C[l] = grads + off[l];
+        cfs_status r = make_tmap_2d_bf16(&m.a[l], dz[l], HID, (uint64_t)B, HID, 64u, DW_ROWS, true);
+        if (r == CFS_OK)
+            r = make_tmap_2d_bf16(&m.b[l], in[l], (uint64_t)g.N[l], (uint64_t)B, (uint64_t)g.N[l],
+                                  64u, DW_ROWS, true);
+        if (r != CFS_OK) return r;
+    }
+    if ((uintptr_t)grads % 16)
+        return fail(CFS_ERR_INVALID_ARG, "weight-gradient GEMM operands not aligned");
+    tc_dw_kernel<<<g.cta0[3] + 1, DW_THREADS, DW_SMEM, st>>>(m, g);
+    return check_cuda(cudaGetLastError(), "tc_dw_kernel launch");
+}
+
 // backward of sum(dY * Y) after forward(): adds into grads [N_PARAMS]
 cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, float* grads,
                     cudaStream_t st)
 {
     const bf16r* wb = s->wb;
+    // fewer rows than one tile: the register-staged GEMMs, whose weight
+    // gradients read transposed copies
+    const bool small = !rows_on_tma(B);
     // gradient sums of the output layer and of the biases gather in copies
     // (bias_part) first: fewer atomics on the same address
     cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
     out_backward_kernel<<<(B + OB_ROWS - 1) / OB_ROWS, OB_THREADS, 0, st>>>(
-        dY, wb, s->H3, s->Z3, B, s->dZ3, s->dZ3T, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
+        dY, wb, s->H3, s->Z3, B, s->dZ3, small ? s->dZ3T : nullptr, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
     // dZ2 = (dZ3 W3) * silu'(Z2): the K-major B operand is W3^T
     // (on tc_rows_kernel the pre-activations Z2 = H1 W2^T + b2 and Z1 = U W1^T
     // + b1 are recomputed, bit for bit, instead of read)
     cfs_status r = tc_rows(st, B, HID, s->dZ3, HID, s->wbT + HID * HID, HID, EPI_SILU_GRAD,
-                           nullptr, nullptr, 0, s->dZ2, HID, s->dZ2T, s->ldt, s->Z2, HID,
+                           nullptr, nullptr, 0, s->dZ2, HID, small ? s->dZ2T : nullptr, s->ldt,
+                           s->Z2, HID,
                            s->bias_part, s->H1, HID, wb + OFF_W2, HID, HID, s->w + OFF_B2);
     if (r == CFS_OK)
         r = tc_rows(st, B, HID, s->dZ2, HID, s->wbT, HID, EPI_SILU_GRAD, nullptr, nullptr, 0,
-                    nullptr, 0, s->dZ1T, s->ldt, s->Z1, HID, s->bias_part + TC_COPIES * HID, U,
+                    small ? nullptr : s->dZ1, HID, small ? s->dZ1T : nullptr, s->ldt, s->Z1, HID,
+                    s->bias_part + TC_COPIES * HID, U,
                     D_IN, wb + OFF_W1, D_IN, D_IN, s->w + OFF_B1);
     if (r != CFS_OK) return r;
+    if (rows_on_tma(B)) return tc_dw(s, U, B, grads, st);
     part_reduce_kernel<<<1, 512, 0, st>>>(s->bias_part, grads);
     transpose_in_kernel<<<(B + 31) / 32, 256, 0, st>>>(U, B, s->UT, s->ldt);
-    // weight gradients dW = dZ^T A: K = the rows, split over CTAs, atomic
-    r = tc_splitk(st, HID, B, s->dZ3T, s->ldt, s->H2T, s->ldt, grads + OFF_W3, HID);
-    if (r == CFS_OK)
-        r = tc_splitk(st, HID, B, s->dZ2T, s->ldt, s->H1T, s->ldt, grads + OFF_W2, HID);
-    if (r == CFS_OK)
-        r = tc_splitk(st, D_IN, B, s->dZ1T, s->ldt, s->UT, s->ldt, grads + OFF_W1, D_IN);
+    // weight gradients dW = dZ^T A from the transposed copies: K = the rows
+    auto dw = [&](int N, const bf16r* dZT, const bf16r* AT, float* C) {
+        return tc_gemm(st, HID, N, B, dZT, s->ldt, AT, s->ldt, EPI_ATOMIC, nullptr, C, N, nullptr,
+                       0, nullptr, 0, nullptr, 0, nullptr);
+    };
+    r = dw(HID, s->dZ3T, s->H2T, grads + OFF_W3);
+    if (r == CFS_OK) r = dw(HID, s->dZ2T, s->H1T, grads + OFF_W2);
+    if (r == CFS_OK) r = dw(D_IN, s->dZ1T, s->UT, grads + OFF_W1);
     return r;
 }
 
@@ -2523,9 +2585,9 @@ cfs_status cfs_sampler_create(const float* params, uint64_t seed, cfs_sampler** 
                                              TrCfg<true>::SMEM),
                         "cudaFuncSetAttribute(tc_rows_kernel)");
     if (st == CFS_OK)
-        st = check_cuda(cudaFuncSetAttribute(tc_splitk_kernel,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, SK_SMEM),
-                        "cudaFuncSetAttribute(tc_splitk_kernel)");
+        st = check_cuda(cudaFuncSetAttribute(tc_dw_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM),
+                        "cudaFuncSetAttribute(tc_dw_kernel)");
     if (st == CFS_OK) st = sw_init();
     if (st == CFS_OK) st = check_cuda(cudaMalloc(&s->d_step, 256), "cudaMalloc(step)");
     if (st == CFS_OK) st = check_cuda(cudaMemset(s->m, 0, sizeof(float) * N_PARAMS * 2), "memset");
