@@ -1485,23 +1485,38 @@ __device__ __forceinline__ float lr_at(u32 step, u32 first, u32 total, float lr,
 
 __global__ void __launch_bounds__(256) adam_kernel(float* w, float* m, float* v,
                                                    const float* g, bf16r* wb, bf16r* wbT, int n,
-                                                   const u32* step, u32 t_explicit, float lr0,
+                                                   u32* step, u32 t_explicit, float lr0,
                                                    float lr_final, u32 first, u32 total,
-                                                   float b1, float b2, float eps)
+                                                   float b1, float b2, float eps,
+                                                   const float* loss, float* hist)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const u32 t = step ? (*step + 1u) : t_explicit;
-    const float lr = step ? lr_at(*step, first, total, lr0, lr_final) : lr0;
-    const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    const float gi = g[i];
-    const float mi = fmaf(b1, m[i], (1.0f - b1) * gi);
-    const float vi = fmaf(b2, v[i], (1.0f - b2) * gi * gi);
-    m[i] = mi;
-    v[i] = vi;
-    const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    w[i] = wi;
-    store_bf16_weight(wb, wbT, i, wi);
+    if (i < n) {
+        const u32 t = step ? (*step + 1u) : t_explicit;
+        const float lr = step ? lr_at(*step, first, total, lr0, lr_final) : lr0;
+        const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
+        const float gi = g[i];
+        const float mi = fmaf(b1, m[i], (1.0f - b1) * gi);
+        const float vi = fmaf(b2, v[i], (1.0f - b2) * gi * gi);
+        m[i] = mi;
+        v[i] = vi;
+        const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+        w[i] = wi;
+        store_bf16_weight(wb, wbT, i, wi);
+    }
+    if (!step) return;
+    // training: the block that finishes last (every block has read *step by
+    // then) puts the step's loss into the run's history and counts the step;
+    // step[1] holds the blocks done and is back at 0 after the last
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicInc(step + 1, gridDim.x - 1) == gridDim.x - 1) {
+            const u32 at = *step - first;
+            if (at < total) hist[at] = *loss;
+            *step += 1u;
+        }
+    }
 }
 
 __global__ void to_bf16_kernel(const float* w, bf16r* wb, bf16r* wbT, int n)
@@ -1538,24 +1553,13 @@ __device__ __forceinline__ uint4 philox_key(u64 seed, u32 c0, u32 c1, u32 c2, u3
 
 constexpr u32 TAG_NOISE = 3, TAG_PROJ = 4, TAG_DATA = 8, TAG_DATA_INIT = 9, TAG_PICK = 10;
 
-// per step: pick the systems of the batch and the projection angles
-__global__ void prep_kernel(const u32* step, u64 seed, int n_sys, int S, u32* sel, float* phi,
-                            int P)
-{
-    const int j = threadIdx.x;
-    const u32 st = *step;
-    if (j < S) sel[j] = philox_key(seed, (u32)j, st, 0u, TAG_PICK).x % (u32)n_sys;
-    const float u = (float)(philox_key(seed, 0u, st, 0u, TAG_PROJ).x >> 8) * CFS_INV_2_24;
-    if (j < P) phi[j] = ((float)j + u) * (6.28318530717958647692f / (float)P);
-}
-
 // network inputs of row r: Gaussian noise (Box-Muller on a Philox block),
 // the conditioning vector of its system and t, written as eight 16-byte
 // vectors
-__device__ __forceinline__ void write_inputs_row(const SysRec& q, int r, u32 st, u64 seed,
-                                                 bf16r* U)
+__device__ __forceinline__ void write_inputs_row(const SysRec& q, int r, u32 st,
+                                                 const unsigned int (&rk)[10][2], bf16r* U)
 {
-    const uint4 w = philox_key(seed, (u32)r, st, 0u, TAG_NOISE);
+    const uint4 w = cfs_philox_rk(rk, (u32)r, st, 0u, TAG_NOISE);
     const float u1 = ((float)(w.x >> 8) + 0.5f) * CFS_INV_2_24;
     const float u2 = (float)(w.y >> 8) * CFS_INV_2_24;
     const float rad = sqrtf(-2.0f * logf(u1));
@@ -1575,48 +1579,80 @@ __device__ __forceinline__ void write_inputs_row(const SysRec& q, int r, u32 st,
         row[v] = make_uint4(w32[4 * v], w32[4 * v + 1], w32[4 * v + 2], w32[4 * v + 3]);
 }
 
-// the records of the systems that rows r0 .. r0 + blockDim.x - 1 belong to
-// (row r: system sel[r / N]; at most 8 with N >= 32) into shared memory
-__device__ __forceinline__ int stage_systems(const SysRec* __restrict__ sys,
-                                            const u32* __restrict__ sel, int N, int rows,
-                                            SysRec* s_sys)
+struct DataArgs {
+    unsigned int rk[10][2];      // Philox round keys of the run's seed
+    const SysRec* sys;           // [n_sys]: the family
+    int n_sys;
+    const u32* step;
+    int N, rows, steps, P;       // rows a system, all rows, chaos-game steps, projections
+    float* T;                    // [rows][2]: the targets
+    bf16r* U;                    // [rows][D_IN]: the network's inputs
+    float* phi;                  // [P]: the projection angles
+    float *zero_a, *zero_b, *dY; // cleared for the step: gradients and loss, the
+    int n_a, n_b;                // gradient copies, and dL/dY [rows][2]
+};
+
+// One training step's inputs.  Row r = s * N + j gets the chaos-game point of
+// its system after `steps` steps from a uniform start (the target) and its
+// network inputs; the systems are picked per step, the angles rotated.  What
+// the step accumulates into is cleared here too: a launch of its own each for
+// that, the picks and the angles were a sixth of the step's launches.  The
+// comparisons of the map choice are unrolled over registers (looping over
+// the record's thresholds in shared memory was 18 us of a 65536-row step).
+__global__ void __launch_bounds__(256) data_kernel(const __grid_constant__ DataArgs a)
 {
+    __shared__ SysRec s_sys[256 / 32];   // rows of a block: at most 8 systems (N >= 32)
+    __shared__ u32 s_sel[256 / 32];
+    const u32 st = *a.step;
     const int r0 = blockIdx.x * blockDim.x;
-    const int first = r0 / N;
-    const int last = min(r0 + (int)blockDim.x - 1, rows - 1) / N;
-    constexpr int W = (int)(sizeof(SysRec) / 4);
-    for (int e = threadIdx.x; e < (last - first + 1) * W; e += blockDim.x) {
-        const int q = e / W, w = e % W;
-        reinterpret_cast<u32*>(&s_sys[q])[w] =
-            reinterpret_cast<const u32*>(&sys[sel ? sel[first + q] : 0])[w];
+    const int first = r0 / a.N, last = min(r0 + (int)blockDim.x - 1, a.rows - 1) / a.N;
+    const int tid = threadIdx.x, all = gridDim.x * blockDim.x, me = r0 + tid;
+    if (tid <= last - first)
+        s_sel[tid] = cfs_philox_rk(a.rk, (u32)(first + tid), st, 0u, TAG_PICK).x % (u32)a.n_sys;
+    for (int e = me; e < a.n_a; e += all) a.zero_a[e] = 0.0f;
+    for (int e = me; e < a.n_b; e += all) a.zero_b[e] = 0.0f;
+    if (me < a.P) {
+        const float u = (float)(cfs_philox_rk(a.rk, 0u, st, 0u, TAG_PROJ).x >> 8) * CFS_INV_2_24;
+        a.phi[me] = ((float)me + u) * (6.28318530717958647692f / (float)a.P);
+    }
+    for (int j = me + all; j < a.P; j += all) {       // fewer rows than projections
+        const float u = (float)(cfs_philox_rk(a.rk, 0u, st, 0u, TAG_PROJ).x >> 8) * CFS_INV_2_24;
+        a.phi[j] = ((float)j + u) * (6.28318530717958647692f / (float)a.P);
     }
     __syncthreads();
-    return first;
-}
-
-// training rows of one step: row r = s * N + j gets the chaos-game point of
-// its system after `steps` steps from a uniform start (the target) and, when
-// U is given, its network inputs
-__global__ void __launch_bounds__(256) data_kernel(const SysRec* __restrict__ sys,
-                                                   const u32* __restrict__ sel, const u32* step,
-                                                   u64 seed, int N, int rows, int steps,
-                                                   float* out, bf16r* U)
-{
-    __shared__ SysRec s_sys[256 / 32];
-    const int first = stage_systems(sys, sel, N, rows, s_sys);
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= rows) return;
-    const SysRec& q = s_sys[r / N - first];
-    const u32 st = *step;
-    if (U) write_inputs_row(q, r, st, seed, U);
-    const uint4 s0 = philox_key(seed, (u32)r, st, 0u, TAG_DATA_INIT);
+    constexpr int W = (int)(sizeof(SysRec) / 4);
+    for (int e = tid; e < (last - first + 1) * W; e += blockDim.x) {
+        const int q = e / W, w = e % W;
+        reinterpret_cast<u32*>(&s_sys[q])[w] = reinterpret_cast<const u32*>(&a.sys[s_sel[q]])[w];
+    }
+    __syncthreads();
+    const int r = me;
+    if (r >= a.rows) return;
+    const SysRec& q = s_sys[r / a.N - first];
+    reinterpret_cast<float2*>(a.dY)[r] = make_float2(0.0f, 0.0f);
+    write_inputs_row(q, r, st, a.rk, a.U);
+    // last word of each map but the last (T - 1); thresholds of 0 are below
+    // every word, those past n_cmp above
+    u32 lastw[MAX_SYS_MAPS - 1];
+    int k0 = 0;
+#pragma unroll
+    for (int j = 0; j < MAX_SYS_MAPS - 1; ++j) {
+        const u32 t = q.T[j];
+        const bool zero = j < q.n_cmp && t == 0u;
+        k0 += zero ? 1 : 0;
+        lastw[j] = j < q.n_cmp && !zero ? t - 1u : 0xFFFFFFFFu;
+    }
+    const uint4 s0 = cfs_philox_rk(a.rk, (u32)r, st, 0u, TAG_DATA_INIT);
     float x = (float)(s0.x >> 8) * CFS_INV_2_24, y = (float)(s0.y >> 8) * CFS_INV_2_24;
-    for (int n = 0; n < steps; n += 4) {
-        const uint4 w = philox_key(seed, (u32)r, st, (u32)(n >> 2), TAG_DATA);
+    for (int n = 0; n < a.steps; n += 4) {
+        const uint4 w = cfs_philox_rk(a.rk, (u32)r, st, (u32)(n >> 2), TAG_DATA);
         const u32 ws[4] = {w.x, w.y, w.z, w.w};
-        for (int h = 0; h < 4 && n + h < steps; ++h) {
-            int k = 0;
-            for (int j = 0; j < q.n_cmp; ++j) k += ws[h] >= q.T[j] ? 1 : 0;
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            if (n + h >= a.steps) break;
+            int k = k0;
+#pragma unroll
+            for (int j = 0; j < MAX_SYS_MAPS - 1; ++j) k += ws[h] > lastw[j] ? 1 : 0;
             const float* m = q.prm[k];
             const float nx = fmaf(m[0], x, fmaf(m[1], y, m[4]));
             const float ny = fmaf(m[2], x, fmaf(m[3], y, m[5]));
@@ -1624,18 +1660,7 @@ __global__ void __launch_bounds__(256) data_kernel(const SysRec* __restrict__ sy
             y = ny;
         }
     }
-    out[2 * r] = x;
-    out[2 * r + 1] = y;
-}
-
-__global__ void step_inc_kernel(u32* step) { *step += 1u; }
-
-// loss of the current step into the run's history (index: step - first)
-__global__ void gather_loss_kernel(const float* loss, const u32* step, u32 first, float* hist,
-                                   u32 cap)
-{
-    const u32 s = *step - first;
-    if (s < cap) hist[s] = *loss;
+    reinterpret_cast<float2*>(a.T)[r] = make_float2(x, y);
 }
 
 
@@ -2402,8 +2427,9 @@ cfs_status tc_dw(cfs_sampler* s, const bf16r* U, int B, float* grads, cudaStream
 }
 
 // backward of sum(dY * Y) after forward(): adds into grads [N_PARAMS]
+// (part_clear: the gradient copies are zero already)
 cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, float* grads,
-                    cudaStream_t st)
+                    cudaStream_t st, bool part_clear = false)
 {
     const bf16r* wb = s->wb;
     // fewer rows than one tile: the register-staged GEMMs, whose weight
@@ -2411,7 +2437,7 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     const bool small = !rows_on_tma(B);
     // gradient sums of the output layer and of the biases gather in copies
     // (bias_part) first: fewer atomics on the same address
-    cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
+    if (!part_clear) cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
     out_backward_kernel<<<(B + OB_ROWS - 1) / OB_ROWS, OB_THREADS, 0, st>>>(
         dY, wb, s->H3, s->Z3, B, s->dZ3, small ? s->dZ3T : nullptr, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
     // dZ2 = (dZ3 W3) * silu'(Z2): the K-major B operand is W3^T
@@ -2711,7 +2737,7 @@ cfs_status cfs_sampler_adam(cfs_sampler* s, const float* grads, uint32_t t, floa
     if (!s || !grads || t == 0) return fail(CFS_ERR_INVALID_ARG, "bad arguments");
     adam_kernel<<<(N_PARAMS + 255) / 256, 256, 0, (cudaStream_t)stream>>>(
         s->w, s->m, s->v, grads, s->wb, s->wbT, N_PARAMS, nullptr, t, lr, lr, 0u, 0u, 0.9f,
-        0.999f, 1e-8f);
+        0.999f, 1e-8f, nullptr, nullptr);
     return check_cuda(cudaGetLastError(), "adam launch");
 }
 
@@ -2761,9 +2787,9 @@ cfs_status cfs_sampler_train_ex(cfs_sampler* s, const cfs_system* const* systems
     // device workspace of the run
     std::vector<SysRec> recs(n_systems);
     for (int i = 0; i < n_systems; ++i) pack_system(systems[i], t_values[i], &recs[i]);
-    const size_t bytes = sizeof(SysRec) * n_systems + 4 * 1024 + 4 * 1024 +
+    const size_t bytes = sizeof(SysRec) * n_systems + 4 * 1024 +
                          sizeof(float) * (size_t)B * 2 * 2 + sizeof(bf16r) * (size_t)B * D_IN +
-                         sizeof(float) * N_PARAMS + 256 + sizeof(float) * (steps + 1) + 8 * 256;
+                         sizeof(float) * (N_PARAMS + 1) + sizeof(float) * (steps + 1) + 8 * 256;
     unsigned char* ws = nullptr;
     st = check_cuda(cudaMalloc(&ws, bytes), "cudaMalloc(training workspace)");
     if (st != CFS_OK) return st;
@@ -2774,13 +2800,12 @@ cfs_status cfs_sampler_train_ex(cfs_sampler* s, const cfs_system* const* systems
         return r;
     };
     SysRec* d_sys = (SysRec*)take(sizeof(SysRec) * n_systems);
-    u32* d_sel = (u32*)take(4 * 1024);
     float* d_phi = (float*)take(4 * 1024);
     float* d_T = (float*)take(sizeof(float) * (size_t)B * 2);
     float* d_dY = (float*)take(sizeof(float) * (size_t)B * 2);
     bf16r* d_U = (bf16r*)take(sizeof(bf16r) * (size_t)B * D_IN);
-    float* d_g = (float*)take(sizeof(float) * N_PARAMS);
-    float* d_loss = (float*)take(256);
+    float* d_g = (float*)take(sizeof(float) * (N_PARAMS + 1));
+    float* d_loss = d_g + N_PARAMS;
     float* d_hist = (float*)take(sizeof(float) * (steps + 1));
     u32 step0 = 0;
     cudaStream_t cap = nullptr;
@@ -2794,22 +2819,24 @@ cfs_status cfs_sampler_train_ex(cfs_sampler* s, const cfs_system* const* systems
     // one training step, captured once and replayed
     if (st == CFS_OK) st = check_cuda(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal), "capture");
     if (st == CFS_OK) {
-        cudaMemsetAsync(d_g, 0, sizeof(float) * N_PARAMS, cap);
-        cudaMemsetAsync(d_dY, 0, sizeof(float) * (size_t)B * 2, cap);
-        cudaMemsetAsync(d_loss, 0, 4, cap);
-        prep_kernel<<<1, 1024, 0, cap>>>(s->d_step, seed, n_systems, S, d_sel, d_phi, (int)n_proj);
-        data_kernel<<<(B + 255) / 256, 256, 0, cap>>>(d_sys, d_sel, s->d_step, seed, N, B, 40, d_T,
-                                                      d_U);
+        DataArgs da;
+        std::memset(&da, 0, sizeof(da));
+        philox_round_keys(seed, da.rk);
+        da.sys = d_sys; da.n_sys = n_systems; da.step = s->d_step;
+        da.N = N; da.rows = B; da.steps = 40; da.P = (int)n_proj;
+        da.T = d_T; da.U = d_U; da.phi = d_phi;
+        da.zero_a = d_g; da.n_a = N_PARAMS + 1;          // and the loss behind them
+        da.zero_b = s->bias_part; da.n_b = PART_FLOATS;
+        da.dY = d_dY;
+        data_kernel<<<(B + 255) / 256, 256, 0, cap>>>(da);
         cfs_status fst = forward(s, d_U, B, cap);
         sw_launch(s->Y, d_T, d_phi, (int)n_proj, N, S, 1.0f / ((float)S * (float)n_proj),
                   d_loss, d_dY, cap);
-        gather_loss_kernel<<<1, 1, 0, cap>>>(d_loss, s->d_step, step0, d_hist, steps);
-        if (fst == CFS_OK) fst = backward(s, d_U, B, d_dY, d_g, cap);
+        if (fst == CFS_OK) fst = backward(s, d_U, B, d_dY, d_g, cap, true);
         adam_kernel<<<(N_PARAMS + 255) / 256, 256, 0, cap>>>(s->w, s->m, s->v, d_g, s->wb, s->wbT,
                                                              N_PARAMS, s->d_step, 0u, lr,
                                                              lr_final, step0, steps, 0.9f,
-                                                             0.999f, 1e-8f);
-        step_inc_kernel<<<1, 1, 0, cap>>>(s->d_step);
+                                                             0.999f, 1e-8f, d_loss, d_hist);
         cudaError_t e = cudaGetLastError();
         cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
         st = check_cuda(e != cudaSuccess ? e : e2, "training step capture");
