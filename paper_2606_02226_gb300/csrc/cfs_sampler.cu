@@ -1010,8 +1010,8 @@ __global__ void __launch_bounds__(256) transpose_in_kernel(const bf16r* __restri
 // output layer backward: dH3 = dY W4 (N = 2, not a tensor-core shape), dZ3 =
 // dH3 * silu'(Z3) written as dZ3 and its transpose dZ3^T; dW4 = dY^T H3,
 // db3 = sum dZ3, db4 = sum dY.  A block takes OB_ROWS rows, a warp one row
-// at a time, lane l the four units 4l .. 4l+3 (16-byte loads of Z3, 8-byte
-// loads of H3); with dZ3T (batches of fewer than 128 rows) the block's dZ3
+// at a time, lane l the four units 4l .. 4l+3 (16-byte loads of Z3, from which
+// H3 is formed again); with dZ3T (batches of fewer than 128 rows) the block's dZ3
 // tile is transposed in shared memory; its sums combine across warps there before one atomic per value into copy
 // blockIdx.x % TC_COPIES of `part`.
 constexpr int OB_ROWS = 64;
@@ -1019,7 +1019,6 @@ constexpr int OB_THREADS = 256;
 
 __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* __restrict__ dY,
                                                                   const bf16r* __restrict__ wb,
-                                                                  const bf16r* __restrict__ H3,
                                                                   const float* __restrict__ Z3,
                                                                   int B, bf16r* dZ3, bf16r* dZ3T,
                                                                   int ldt, float* part)
@@ -1044,20 +1043,19 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
         if (r >= B) break;
         const float y0 = dY[2 * r], y1 = dY[2 * r + 1];
         const float4 z = *reinterpret_cast<const float4*>(Z3 + (size_t)r * HID + c);
-        const uint2 hv = *reinterpret_cast<const uint2*>(H3 + (size_t)r * HID + c);
         const float zz[4] = {z.x, z.y, z.z, z.w};
-        const float h[4] = {__uint_as_float(hv.x << 16), __uint_as_float(hv.x & 0xFFFF0000u),
-                            __uint_as_float(hv.y << 16), __uint_as_float(hv.y & 0xFFFF0000u)};
         bf16r db[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const float dh = fmaf(y0, w0[j], y1 * w1[j]);
             const float d = dh * silu_grad_f(zz[j]);
+            // H3 again, the forward's bits (the two share their sigmoid)
+            const float h = from_bf16(to_bf16(silu_f(zz[j])));
             db[j] = to_bf16(d);
             if (dZ3T) tT[c + j][k] = db[j];
             ab[j] += d;
-            a0[j] = fmaf(y0, h[j], a0[j]);
-            a1[j] = fmaf(y1, h[j], a1[j]);
+            a0[j] = fmaf(y0, h, a0[j]);
+            a1[j] = fmaf(y1, h, a1[j]);
         }
         *reinterpret_cast<uint2*>(dZ3 + (size_t)r * HID + c) =
             make_uint2((u32)db[0] | ((u32)db[1] << 16), (u32)db[2] | ((u32)db[3] << 16));
@@ -1741,14 +1739,18 @@ __device__ __forceinline__ void it_st16(u32 addr, u32 a, u32 b, u32 c, u32 d)
 }
 
 // a [128][K] BF16 weight matrix (16-byte aligned) into a K-major tile (K
-// groups 2048 B apart), 16 bytes = 8 columns of one row at a time: a warp's
-// lanes take 32 consecutive rows of one K group, whose shared-memory places
-// are consecutive (element by element the loop was 15 us of every launch)
+// groups 2048 B apart), 16 bytes = 8 columns of one row at a time.  A warp's
+// lanes take 8 rows x 4 K groups: 64-byte runs in global memory and no bank
+// conflicts in shared memory (a row per lane was 32 lines an instruction, and
+// element by element the loop took 15 us of every launch)
 template <int K, int THREADS>
 __device__ __forceinline__ void it_stage_weights(u32 dst, const bf16r* __restrict__ w)
 {
+    constexpr int KG4 = K / 32;                 // runs of 4 K groups
+#pragma unroll
     for (int e = threadIdx.x; e < 128 * (K / 8); e += THREADS) {
-        const int n = e & 127, kg = e >> 7;
+        const int l = e & 31, run = e >> 5;
+        const int n = (run / KG4) * 8 + (l & 7), kg = (run % KG4) * 4 + (l >> 3);
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(w + (size_t)n * K + 8 * kg));
         it_st16(dst + (u32)kg * 2048u + (u32)n * 16u, v.x, v.y, v.z, v.w);
     }
@@ -1990,7 +1992,7 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
 // group's A tile; layer 1 (K = 64), layer 2 and layer 3 run as tcgen05.mma
 // chains into the group's TMEM columns, each epilogue adding the bias,
 // applying SiLU and writing the next A tile in place.  What the backward
-// pass reads is written on the way, row-major: H1, H2, H3 and Z3; the output
+// pass reads is written on the way, row-major: H1, H2 and Z3; the output
 // layer itself (N = 2) runs on the CUDA cores in the layer-3 epilogue.
 // ---------------------------------------------------------------------------
 constexpr int TF_GROUPS = 4;
@@ -2001,7 +2003,7 @@ constexpr int TF_SMEM = 1024 + TF_W1 + 2 * IT_W + TF_GROUPS * IT_A + 256;
 struct TrainFwdArgs {
     const bf16r* U;                // [B][D_IN]
     int B;
-    bf16r *H1, *H2, *H3;           // [B][HID]
+    bf16r *H1, *H2;                // [B][HID]
     float *Z3, *Y;                 // Z3 [B][HID], Y [B][2]
 };
 
@@ -2101,22 +2103,25 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
             it_st16(sA + it_off(r, c0 + 8, 2048u), q[4], q[5], q[6], q[7]);
         });
     };
-    // the group's A tile to rows row0 .. of H, while the MMAs read it too: a
-    // warp's lanes take 8 rows x 4 K groups, which leave shared memory
-    // without conflicts and arrive in 64-byte runs (a row per lane, straight
-    // from the epilogue, was 32 lines an instruction)
-    auto store_tile = [&](bf16r* H, int row0) {
-        const int rr = lane & 7, kq = lane >> 3;
-#pragma unroll 4
+    // the group's A tile -- 16 groups of 16 bytes a row, 2048 B apart -- to 256
+    // bytes of each of the rows row0 .. at `out`, `pitch` bytes apart, while
+    // the MMAs may read it too.  A warp's lanes take 4 rows x 8 groups: whole
+    // 128-byte lines leave, at two lanes a bank (a row per lane, straight from
+    // the epilogue, was 32 lines an instruction, and 8 rows x 4 groups, 64-byte
+    // runs, 9.7 thousand cycles a tile)
+    auto store_tile = [&](void* out, size_t pitch, int row0) {
+        const int rr = lane & 3, kq = lane >> 2;
+#pragma unroll 8
         for (int e = 0; e < 16; ++e) {
-            const int rt = wq * 32 + (e >> 2) * 8 + rr, kg = (e & 3) * 4 + kq;
+            const int rt = wq * 32 + (e >> 1) * 4 + rr, kg = (e & 1) * 8 + kq;
             u32 v[4];
             asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
                          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                         : "r"(sA + it_off(rt, 8 * kg, 2048u))
+                         : "r"(sA + (u32)kg * 2048u + (u32)rt * 16u)
                          : "memory");
             if (row0 + rt < g.B)
-                *reinterpret_cast<uint4*>(H + (size_t)(row0 + rt) * HID + 8 * kg) =
+                *reinterpret_cast<uint4*>(static_cast<unsigned char*>(out) +
+                                          (size_t)(row0 + rt) * pitch + 16 * kg) =
                     make_uint4(v[0], v[1], v[2], v[3]);
         }
     };
@@ -2125,54 +2130,79 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
     for (int tile = blockIdx.x * TF_GROUPS + gi; tile < n_tiles; tile += gridDim.x * TF_GROUPS) {
         const int row = tile * 128 + r;
         const bool in = row < g.B;
-        // the tile's inputs: row r's 64 BF16 values into K groups 0..7
+        // the tile's inputs, 64 BF16 values a row, into K groups 0..7 (8 rows x 4
+        // groups a warp instruction, as the weights)
         {
-            const uint4* src = reinterpret_cast<const uint4*>(g.U + (size_t)row * D_IN);
+            uint4 v[8];
 #pragma unroll
-            for (int kq = 0; kq < D_IN / 8; ++kq) {
-                const uint4 v = in ? __ldg(src + kq) : make_uint4(0u, 0u, 0u, 0u);
-                it_st16(sA + it_off(r, 8 * kq, 2048u), v.x, v.y, v.z, v.w);
+            for (int e = 0; e < 8; ++e) {
+                const int rt = tile * 128 + wq * 32 + (e >> 1) * 8 + (lane & 7);
+                const int kg = (e & 1) * 4 + (lane >> 3);
+                v[e] = rt < g.B ? __ldg(reinterpret_cast<const uint4*>(g.U + (size_t)rt * D_IN) + kg)
+                                : make_uint4(0u, 0u, 0u, 0u);
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int rt = wq * 32 + (e >> 1) * 8 + (lane & 7), kg = (e & 1) * 4 + (lane >> 3);
+                it_st16(sA + (u32)kg * 2048u + (u32)rt * 16u, v[e].x, v[e].y, v[e].z, v[e].w);
             }
         }
         mma_layer(sW1, D_IN);
         if (!(ok = wait_layer())) break;
         hidden_epilogue(s_b1);
         mma_layer(sW2, HID);
-        store_tile(g.H1, tile * 128);
+        store_tile(g.H1, HID * 2, tile * 128);
         if (!(ok = wait_layer())) break;
         hidden_epilogue(s_b2);
         mma_layer(sW3, HID);
-        store_tile(g.H2, tile * 128);
+        store_tile(g.H2, HID * 2, tile * 128);
         if (!(ok = wait_layer())) break;
-        // layer 3: Z3 (FP32) and H3 (BF16) out, then the output layer on
-        // the BF16 activations, columns in order
+        // layer 3: Z3 (FP32) out, and the output layer on the BF16 activations
+        // (which the backward pass forms again from Z3), columns in order.
+        // The A tile holds 64 FP32 columns, so Z3 leaves in two halves
         float y0 = 0.0f, y1 = 0.0f;
-        tc_for_columns(tlane, [&](int c0, const u32 (&v)[16]) {
-            float z[16];
-            u32 q[8];
+        auto output_half = [&](int c_half) {
+            u32 a[16], b[16];
+            auto work = [&](int c0, const u32 (&v)[16]) {
+                const float4* b4 = reinterpret_cast<const float4*>(s_b3 + c0);
+                const float4* p0 = reinterpret_cast<const float4*>(&s_w4[0][c0]);
+                const float4* p1 = reinterpret_cast<const float4*>(&s_w4[1][c0]);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = __uint_as_float(v[j]) + s_b3[c0 + j];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) q[j] = pack_bf16x2(silu_f(z[2 * j]), silu_f(z[2 * j + 1]));
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                const float x = __uint_as_float((q[j >> 1] >> (16 * (j & 1))) << 16);
-                y0 = fmaf(x, s_w4[0][c0 + j], y0);
-                y1 = fmaf(x, s_w4[1][c0 + j], y1);
+                for (int j = 0; j < 4; ++j) {
+                    const float4 bb = b4[j], w0 = p0[j], w1 = p1[j];
+                    const float z[4] = {
+                        __uint_as_float(v[4 * j]) + bb.x, __uint_as_float(v[4 * j + 1]) + bb.y,
+                        __uint_as_float(v[4 * j + 2]) + bb.z, __uint_as_float(v[4 * j + 3]) + bb.w};
+                    const u32 q0 = pack_bf16x2(silu_f(z[0]), silu_f(z[1]));
+                    const u32 q1 = pack_bf16x2(silu_f(z[2]), silu_f(z[3]));
+                    const float h[4] = {__uint_as_float(q0 << 16), __uint_as_float(q0 & 0xFFFF0000u),
+                                        __uint_as_float(q1 << 16), __uint_as_float(q1 & 0xFFFF0000u)};
+                    y0 = fmaf(h[0], w0.x, y0); y1 = fmaf(h[0], w1.x, y1);
+                    y0 = fmaf(h[1], w0.y, y0); y1 = fmaf(h[1], w1.y, y1);
+                    y0 = fmaf(h[2], w0.z, y0); y1 = fmaf(h[2], w1.z, y1);
+                    y0 = fmaf(h[3], w0.w, y0); y1 = fmaf(h[3], w1.w, y1);
+                    it_st16(sA + (u32)((c0 - c_half) / 4 + j) * 2048u + (u32)r * 16u,
+                            __float_as_uint(z[0]), __float_as_uint(z[1]), __float_as_uint(z[2]),
+                            __float_as_uint(z[3]));
+                }
+            };
+            tc_ld16_nowait(tlane + (u32)c_half, a);
+#pragma unroll 1
+            for (int c0 = c_half; c0 < c_half + 64; c0 += 32) {
+                tc_wait_ld(a);
+                tc_ld16_nowait(tlane + (u32)(c0 + 16), b);
+                work(c0, a);
+                tc_wait_ld(b);
+                if (c0 + 32 < c_half + 64) tc_ld16_nowait(tlane + (u32)(c0 + 32), a);
+                work(c0 + 16, b);
             }
-            if (in) {
-                float4* zp = reinterpret_cast<float4*>(g.Z3 + (size_t)row * HID + c0);
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    zp[j] = make_float4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
-            }
-            it_st16(sA + it_off(r, c0, 2048u), q[0], q[1], q[2], q[3]);
-            it_st16(sA + it_off(r, c0 + 8, 2048u), q[4], q[5], q[6], q[7]);
-        });
-        tc_fence_before();          // TMEM read: the next tile's MMAs may overwrite it
-        it_group_sync(gi);
-        store_tile(g.H3, tile * 128);
-        it_group_sync(gi);          // the next tile's inputs go into the A tile
+            if (c_half) tc_fence_before();   // TMEM read: the next tile's MMAs may overwrite it
+            it_group_sync(gi);
+            store_tile(reinterpret_cast<float*>(g.Z3) + c_half, HID * 4, tile * 128);
+            it_group_sync(gi);               // the A tile is free again
+        };
+        output_half(0);
+        output_half(64);
         if (in) {
             g.Y[2 * (size_t)row] = y0 + s_b4[0];
             g.Y[2 * (size_t)row + 1] = y1 + s_b4[1];
@@ -2367,7 +2397,7 @@ cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
         }
         TrainFwdArgs a;
         a.U = U; a.B = B;
-        a.H1 = s->H1; a.H2 = s->H2; a.H3 = s->H3;
+        a.H1 = s->H1; a.H2 = s->H2;
         a.Z3 = s->Z3; a.Y = s->Y;
         const int tiles = (B + 127) / 128;
         const int grid = std::max(1, std::min(device_sm_count(), (tiles + TF_GROUPS - 1) / TF_GROUPS));
@@ -2439,7 +2469,7 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     // (bias_part) first: fewer atomics on the same address
     if (!part_clear) cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
     out_backward_kernel<<<(B + OB_ROWS - 1) / OB_ROWS, OB_THREADS, 0, st>>>(
-        dY, wb, s->H3, s->Z3, B, s->dZ3, small ? s->dZ3T : nullptr, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
+        dY, wb, s->Z3, B, s->dZ3, small ? s->dZ3T : nullptr, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
     // dZ2 = (dZ3 W3) * silu'(Z2): the K-major B operand is W3^T
     // (on tc_rows_kernel the pre-activations Z2 = H1 W2^T + b2 and Z1 = U W1^T
     // + b1 are recomputed, bit for bit, instead of read)
