@@ -124,7 +124,7 @@ struct TcArgs {
     const float* Zin; int ldz;   // SILU_GRAD: pre-activation of the layer
     float* colsum;               // SILU_GRAD: bias gradient partials, [TC_COPIES][N]; CTA b
                                  // adds its column sums into copy b % TC_COPIES
-    int K2;                      // tc_rows_kernel<true>: K of the recomputed pre-activation
+    int K2;                      // tc_rows_kernel: K of the recomputed pre-activation
 };
 
 __device__ __forceinline__ u32 smem_addr(const void* p)
@@ -504,14 +504,12 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
 }
 
 // ---------------------------------------------------------------------------
-// The row GEMMs of training and inference, D[rows][128] = A[rows][K] W^T
-// (K = 64 or 128) with the SILU / SILU_GRAD epilogues, as one persistent
-// warp-specialized kernel per GEMM (one CTA per SM, row tiles of 128 strided
-// over the CTAs):
-//   warp 0  -- TMA: the weights once, then each tile's A into a ring of
-//              TrCfg::STAGES shared-memory slots (2D tensor maps, boxes of 128
-//              rows x 8 K elements, i.e. one 16-byte column of core
-//              matrices: K-adjacent cores 2048 B apart, 8-row groups 128 B);
+// The input-gradient GEMMs of training, D[rows][128] = A[rows][128] W^T with
+// the SILU_GRAD epilogue, as one persistent warp-specialized kernel per GEMM
+// (one CTA per SM, row tiles of 128 strided over the CTAs):
+//   warp 0  -- TMA: the weights once, then each tile's operands into a ring of
+//              TR_STAGES shared-memory slots (2D tensor maps, boxes of 128
+//              rows x 64 K elements in the 128-byte swizzle);
 //   warp 1  -- TMEM owner; one thread issues the tile's tcgen05.mma into one
 //              of two accumulator buffers and commits it to the slot's
 //              "empty" barrier and the accumulator's "full" barrier;
@@ -520,26 +518,33 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
 //              i + 1 is loaded and multiplied; each warp arrives on the
 //              accumulator's "empty" barrier as soon as its columns are in
 //              registers.
-// tc_rows_kernel<true> (SILU_GRAD of the input gradients) also loads the
-// layer below's activations A2 and weights W2 and multiplies them into a
-// second accumulator: its pre-activation Z = A2 W2^T + b, the same MMAs the
-// forward ran, so the SiLU derivative needs no stored Z.
+// The epilogue needs the pre-activation of the layer below for the SiLU
+// derivative: its activations A2 and weights W2 are loaded too and multiplied
+// into a second accumulator, Z = A2 W2^T + b, the same MMAs the forward ran,
+// so no Z has to be stored.
+// Boxes of 8 K elements (16-byte rows, the no-swizzle layout) kept the TMA
+// unit busy with 4096 rows a tile: 25 us a GEMM of 65536 rows.
 // Every wait is bounded; a time-out sets g_tc_error and the role stops.
 // ---------------------------------------------------------------------------
 constexpr int TR_EPI_WARPS = 16;
 constexpr int TR_THREADS = 32 * (2 + TR_EPI_WARPS);
 constexpr int TR_TILE = 128 * 128 * 2;   // one A tile or the weights at K = 128
 
-// shapes of the two variants: RC also recomputes the pre-activation Z of
-// the layer below (second operand pair, second accumulator)
-template <bool RC>
-struct TrCfg {
-    static constexpr int STAGES = RC ? 2 : 3;
-    static constexpr int SLOT = RC ? 2 * TR_TILE : TR_TILE;      // A (and A2) of a tile
-    static constexpr int WEIGHTS = RC ? 2 * TR_TILE : TR_TILE;   // W (and W2)
-    static constexpr int SMEM = 1024 + WEIGHTS + STAGES * SLOT + 256 + 4 * 128;
-    static constexpr int ACC = RC ? 256 : 128;                   // TMEM columns per buffer
-};
+constexpr int TR_KB = 128 * 128;         // a box: 128 rows x 64 K elements
+constexpr int TR_STAGES = 2;
+constexpr int TR_SLOT = 2 * TR_TILE;     // A and A2 of a tile
+constexpr int TR_WEIGHTS = 2 * TR_TILE;  // W and W2
+constexpr int TR_SMEM = 1024 + TR_WEIGHTS + TR_STAGES * TR_SLOT + 256 + 4 * 128;
+constexpr int TR_ACC = 256;              // TMEM columns per accumulator buffer
+
+// K-major operand in the 128-byte swizzle: 8 rows of 64 K elements are one
+// 1024-byte atom (stride offset between 8-row groups); within it a step of 16
+// K elements is 32 bytes of the start address
+__device__ __forceinline__ u64 tc_desc_ksw(u32 saddr)
+{
+    return (u64)((saddr >> 4) & 0x3FFFu) | ((u64)1 << 16) | ((u64)(1024u >> 4) << 32) |
+           ((u64)1 << 46) | ((u64)2 << 61);
+}
 
 __device__ __forceinline__ u64 tc_desc_kn(u32 saddr, u32 lbo, u32 sbo)
 {
@@ -568,20 +573,18 @@ __device__ __forceinline__ void tma_load_2d(u32 dst, const CUtensorMap* map, int
         : "memory");
 }
 
-template <bool RC>
 __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
     const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
     const __grid_constant__ CUtensorMap tmA2, const __grid_constant__ CUtensorMap tmB2,
     const __grid_constant__ TcArgs g)
 {
-    using Cf = TrCfg<RC>;
-    constexpr int ST = Cf::STAGES;
+    constexpr int ST = TR_STAGES;
     extern __shared__ unsigned char tr_smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(tr_smem_raw) + 1023) & ~(uintptr_t)1023);
     // W at sm (W2 after it), then ST slots of A (A2 after it in the slot)
-    const u32 sB = smem_addr(sm), sB2 = sB + TR_TILE, sA = sB + Cf::WEIGHTS;
-    u64* bars = reinterpret_cast<u64*>(sm + Cf::WEIGHTS + ST * Cf::SLOT);
+    const u32 sB = smem_addr(sm), sB2 = sB + TR_TILE, sA = sB + TR_WEIGHTS;
+    u64* bars = reinterpret_cast<u64*>(sm + TR_WEIGHTS + ST * TR_SLOT);
     // barriers: full[s], empty[s] (s < ST), wfull, tfull[2], tempty[2]
     auto full = [&](int s) { return smem_addr(&bars[s]); };
     auto empty = [&](int s) { return smem_addr(&bars[ST + s]); };
@@ -591,24 +594,24 @@ __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
     u32* s_tmem = reinterpret_cast<u32*>(bars + 16);
     __shared__ int s_err;
     float* s_col = reinterpret_cast<float*>(bars + 32);   // [128]
-    // SILU: the layer's bias; RC: the bias of the recomputed pre-activation
+    // the bias of the recomputed pre-activation
     __shared__ float s_bias[128];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_tiles = (g.M + TC_M - 1) / TC_M;
-    const int kch = g.K / 8, kch2 = RC ? g.K2 / 8 : 0;   // 16-byte K columns
-    const u32 tile_bytes = (u32)(TC_M * (g.K + (RC ? g.K2 : 0)) * 2);
+    const int kb = g.K / 64, kb2 = g.K2 / 64;           // boxes of each operand
+    const u32 tile_bytes = (u32)(TC_M * (g.K + g.K2) * 2);
     const u32 w_bytes = tile_bytes;                     // W rows = tile rows = 128
 
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      :
-                     : "r"(smem_addr(s_tmem)), "r"(2u * (u32)Cf::ACC)
+                     : "r"(smem_addr(s_tmem)), "r"(2u * (u32)TR_ACC)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     if (threadIdx.x < 128) {
         s_col[threadIdx.x] = 0.0f;
-        s_bias[threadIdx.x] = (g.mode == EPI_SILU || RC) ? g.bias[threadIdx.x] : 0.0f;
+        s_bias[threadIdx.x] = g.bias[threadIdx.x];
     }
     if (threadIdx.x == 0) {
         s_err = 0;
@@ -631,8 +634,8 @@ __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
     if (warp == 0) {
         if (lane == 0) {
             mbar_expect_tx(wfull, w_bytes);
-            for (int kc = 0; kc < kch; ++kc) tma_load_2d(sB + kc * 2048, &tmB, kc * 8, 0, wfull);
-            for (int kc = 0; kc < kch2; ++kc) tma_load_2d(sB2 + kc * 2048, &tmB2, kc * 8, 0, wfull);
+            for (int c = 0; c < kb; ++c) tma_load_2d(sB + c * TR_KB, &tmB, c * 64, 0, wfull);
+            for (int c = 0; c < kb2; ++c) tma_load_2d(sB2 + c * TR_KB, &tmB2, c * 64, 0, wfull);
             int i = 0, issued = 0;
             for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++i) {
                 const int s = i % ST;
@@ -641,11 +644,11 @@ __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
                     break;
                 }
                 mbar_expect_tx(full(s), tile_bytes);
-                const u32 a = sA + (u32)(s * Cf::SLOT);
-                for (int kc = 0; kc < kch; ++kc)
-                    tma_load_2d(a + kc * 2048, &tmA, kc * 8, tile * TC_M, full(s));
-                for (int kc = 0; kc < kch2; ++kc)
-                    tma_load_2d(a + TR_TILE + kc * 2048, &tmA2, kc * 8, tile * TC_M, full(s));
+                const u32 a = sA + (u32)(s * TR_SLOT);
+                for (int c = 0; c < kb; ++c)
+                    tma_load_2d(a + c * TR_KB, &tmA, c * 64, tile * TC_M, full(s));
+                for (int c = 0; c < kb2; ++c)
+                    tma_load_2d(a + TR_TILE + c * TR_KB, &tmA2, c * 64, tile * TC_M, full(s));
                 issued = i + 1;
             }
             // every load issued has landed before the CTA may leave
@@ -663,15 +666,16 @@ __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
                 if (!mbar_wait(full(s), (u32)(i / ST) & 1u)) { ok = false; break; }
                 if (i >= 2 && !mbar_wait(tempty(b), (u32)(i / 2 - 1) & 1u)) { ok = false; break; }
                 tc_fence_after();
-                const u32 a = sA + (u32)(s * Cf::SLOT), d = tmem + (u32)(b * Cf::ACC);
-                for (int kk = 0; kk < g.K / 16; ++kk)
-                    tc_mma(d, tc_desc_kn(a + kk * 4096, 2048u, 128u),
-                           tc_desc_kn(sB + kk * 4096, 2048u, 128u), idesc, kk > 0 ? 1u : 0u);
+                const u32 a = sA + (u32)(s * TR_SLOT), d = tmem + (u32)(b * TR_ACC);
+                auto at = [](int kk) { return (u32)((kk >> 2) * TR_KB + (kk & 3) * 32); };
+                for (int kk = 0; kk < 4 * kb; ++kk)
+                    tc_mma(d, tc_desc_ksw(a + at(kk)), tc_desc_ksw(sB + at(kk)), idesc,
+                           kk > 0 ? 1u : 0u);
                 // the layer below's pre-activation: the forward's MMAs on the
                 // same operands in the same order, so the same bits
-                for (int kk = 0; kk < kch2 / 2; ++kk)
-                    tc_mma(d + 128u, tc_desc_kn(a + TR_TILE + kk * 4096, 2048u, 128u),
-                           tc_desc_kn(sB2 + kk * 4096, 2048u, 128u), idesc, kk > 0 ? 1u : 0u);
+                for (int kk = 0; kk < 4 * kb2; ++kk)
+                    tc_mma(d + 128u, tc_desc_ksw(a + TR_TILE + at(kk)),
+                           tc_desc_ksw(sB2 + at(kk)), idesc, kk > 0 ? 1u : 0u);
                 tc_commit(empty(s));
                 tc_commit(tfull(b));
                 committed = i + 1;
@@ -690,75 +694,44 @@ __global__ void __launch_bounds__(TR_THREADS, 1) tc_rows_kernel(
         for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++i) {
             const int b = i & 1;
             const int row = tile * TC_M + quad * 32 + lane;
-            float z_next[16];
-            if (!RC) tc_load_z(g, row, c_begin, z_next);   // overlaps the wait
             if (!mbar_wait(tfull(b), (u32)(i / 2) & 1u)) {
                 atomicExch(&s_err, 1);
                 break;
             }
             tc_fence_after();
-            const u32 base = tmem + ((u32)(quad * 32) << 16) + (u32)(b * Cf::ACC);
-            if constexpr (RC) {
-                // per 16 columns: the product and the recomputed pre-activation
+            const u32 base = tmem + ((u32)(quad * 32) << 16) + (u32)(b * TR_ACC);
+            // per 16 columns: the product and the recomputed pre-activation
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int c0 = c_begin + 16 * h;
-                    u32 r[16], q[16];
-                    tc_ld16_nowait(base + (u32)c0, r);
-                    tc_ld16_nowait(base + 128u + (u32)c0, q);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                    if (h == 1) {   // the accumulators are read: release them
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(tempty(b));
-                    }
-                    float v[16], z[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        v[j] = __uint_as_float(r[j]);
-                        z[j] = __uint_as_float(q[j]) + s_bias[c0 + j];
-                    }
-                    tc_epilogue(g, row, c0, v, z, s_col, s_bias);
-                }
-            } else {
-                // both 16-column loads in flight before the one wait
-                u32 r0[16], r1[16];
-                tc_ld16_nowait(base + (u32)c_begin, r0);
-                tc_ld16_nowait(base + (u32)(c_begin + 16), r1);
+            for (int h = 0; h < 2; ++h) {
+                const int c0 = c_begin + 16 * h;
+                u32 r[16], q[16];
+                tc_ld16_nowait(base + (u32)c0, r);
+                tc_ld16_nowait(base + 128u + (u32)c0, q);
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-                // the accumulator is read: release it to the MMA thread before
-                // the arithmetic and the stores
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(tempty(b));
-                {
-                    float v[16], z[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        v[j] = __uint_as_float(r0[j]);
-                        z[j] = z_next[j];
-                    }
-                    tc_load_z(g, row, c_begin + 16, z_next);
-                    tc_epilogue(g, row, c_begin, v, z, s_col, s_bias);
+                if (h == 1) {   // the accumulators are read: release them
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tempty(b));
                 }
-                {
-                    float v[16];
+                float v[16], z[16];
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r1[j]);
-                    tc_epilogue(g, row, c_begin + 16, v, z_next, s_col, s_bias);
+                for (int j = 0; j < 16; ++j) {
+                    v[j] = __uint_as_float(r[j]);
+                    z[j] = __uint_as_float(q[j]) + s_bias[c0 + j];
                 }
+                tc_epilogue(g, row, c0, v, z, s_col, s_bias);
             }
         }
     }
     tc_fence_before();
     __syncthreads();
-    if (g.mode == EPI_SILU_GRAD && !s_err && threadIdx.x < 128 && s_col[threadIdx.x] != 0.0f)
+    if (!s_err && threadIdx.x < 128 && s_col[threadIdx.x] != 0.0f)
         atomicAdd(g.colsum + (blockIdx.x % TC_COPIES) * 128 + threadIdx.x, s_col[threadIdx.x]);
     if (threadIdx.x == 0 && s_err) atomicOr(&g_tc_error, (unsigned)CFS_DEVICE_ERR_TC_TIMEOUT);
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                     "r"(2u * (u32)Cf::ACC)
+                     "r"(2u * (u32)TR_ACC)
                      : "memory");
     }
 }
@@ -2322,61 +2295,34 @@ cfs_status tc_gemm(cudaStream_t st, int M, int N, int K, const bf16r* A, int lda
     return CFS_OK;
 }
 
-// row GEMM D[M][128] = A[M][K] W^T (K = 64 or 128) with the SILU or
-// SILU_GRAD epilogue on the persistent TMA kernel (tc_gemm_kernel for
-// fewer rows than one tile)
-
-// whether row GEMMs of M rows run on tc_rows_kernel: then the backward
-// recomputes the pre-activations Z1 and Z2 and the forward need not store them
+// whether a batch of M rows runs on the fused forward, tc_rows_kernel and
+// tc_dw_kernel; smaller ones use the register-staged tc_gemm_kernel (no tensor
+// map with an extent below its box)
 bool rows_on_tma(int M) { return M >= TC_M; }
 
-// A2, W2 (K2 = 64 or 128), bias2: SILU_GRAD with the pre-activation of the
-// layer below recomputed as A2 W2^T + bias2 instead of read from Zin (only
-// where rows_on_tma(M); elsewhere Zin is read)
-cfs_status tc_rows(cudaStream_t st, int M, int K, const bf16r* A, int lda, const bf16r* W, int ldw,
-                   int mode, const float* bias, float* C, int ldc, bf16r* H, int ldh, bf16r* HT,
-                   int ldt, const float* Zin, int ldz, float* colsum,
-                   const bf16r* A2 = nullptr, int lda2 = 0, const bf16r* W2 = nullptr,
-                   int ldw2 = 0, int K2 = 0, const float* bias2 = nullptr)
+// dZ[M][128] = (A[M][128] W^T) silu'(A2 W2^T + bias2) (K2 = 64 or 128 columns
+// of A2), its column sums into colsum; M >= 128, rows without gaps
+cfs_status tc_rows(cudaStream_t st, int M, const bf16r* A, const bf16r* W, bf16r* dZ, float* colsum,
+                   const bf16r* A2, const bf16r* W2, int K2, const float* bias2)
 {
-    // fewer rows than one tile: the register-staged kernel (no tensor map with
-    // an extent below its box)
-    if (!rows_on_tma(M))
-        return tc_gemm(st, M, HID, K, A, lda, W, ldw, mode, bias, C, ldc, H, ldh, HT, ldt, Zin,
-                       ldz, colsum);
-    const bool rc = A2 != nullptr;
-    const bool aligned =
-        (K == 64 || K == 128) && lda % 8 == 0 && ldw % 8 == 0 &&
-        (!C || ((uintptr_t)C % 16 == 0 && ldc % 4 == 0)) &&
-        (!H || ((uintptr_t)H % 16 == 0 && ldh % 8 == 0)) &&
-        (!Zin || ((uintptr_t)Zin % 16 == 0 && ldz % 4 == 0)) &&
-        (!rc || ((K2 == 64 || K2 == 128) && lda2 % 8 == 0 && ldw2 % 8 == 0 && W2 && bias2 &&
-                 mode == EPI_SILU_GRAD));
-    if (!aligned) return fail(CFS_ERR_INVALID_ARG, "row GEMM operands not aligned");
     CUtensorMap ta, tb, ta2, tb2;
-    cfs_status r = make_tmap_2d_bf16(&ta, A, (uint64_t)K, (uint64_t)M, (uint64_t)lda, 8u, 128u);
-    if (r == CFS_OK) r = make_tmap_2d_bf16(&tb, W, (uint64_t)K, 128u, (uint64_t)ldw, 8u, 128u);
-    if (r == CFS_OK && rc)
-        r = make_tmap_2d_bf16(&ta2, A2, (uint64_t)K2, (uint64_t)M, (uint64_t)lda2, 8u, 128u);
-    if (r == CFS_OK && rc)
-        r = make_tmap_2d_bf16(&tb2, W2, (uint64_t)K2, 128u, (uint64_t)ldw2, 8u, 128u);
+    auto map = [](CUtensorMap* m, const bf16r* p, int rows, int cols) {
+        return make_tmap_2d_bf16(m, p, (uint64_t)cols, (uint64_t)rows, (uint64_t)cols, 64u, 128u,
+                                 true);
+    };
+    cfs_status r = map(&ta, A, M, HID);
+    if (r == CFS_OK) r = map(&tb, W, 128, HID);
+    if (r == CFS_OK) r = map(&ta2, A2, M, K2);
+    if (r == CFS_OK) r = map(&tb2, W2, 128, K2);
     if (r != CFS_OK) return r;
-    if (!rc) { ta2 = ta; tb2 = tb; }   // unused
     TcArgs g;
     std::memset(&g, 0, sizeof(g));
-    g.M = M; g.N = HID; g.K = K;
-    g.A = A; g.lda = lda; g.B = W; g.ldb = ldw;
-    g.k_split = K;
-    g.mode = mode; g.bias = rc ? bias2 : bias; g.C = C; g.ldc = ldc; g.H = H; g.ldh = ldh;
-    g.HT = HT; g.ldt = ldt; g.Zin = rc ? nullptr : Zin; g.ldz = ldz; g.colsum = colsum;
-    g.K2 = rc ? K2 : 0;
+    g.M = M; g.N = HID; g.K = HID; g.K2 = K2;
+    g.mode = EPI_SILU_GRAD; g.bias = bias2; g.H = dZ; g.ldh = HID; g.colsum = colsum;
     const int tiles = (M + TC_M - 1) / TC_M;
     const int grid = std::min(tiles, std::max(1, device_sm_count()));
-    if (rc)
-        tc_rows_kernel<true><<<grid, TR_THREADS, TrCfg<true>::SMEM, st>>>(ta, tb, ta2, tb2, g);
-    else
-        tc_rows_kernel<false><<<grid, TR_THREADS, TrCfg<false>::SMEM, st>>>(ta, tb, ta2, tb2, g);
-    return CFS_OK;
+    tc_rows_kernel<<<grid, TR_THREADS, TR_SMEM, st>>>(ta, tb, ta2, tb2, g);
+    return check_cuda(cudaGetLastError(), "tc_rows_kernel launch");
 }
 
 // forward of B rows of U: H1..H3 (bf16), Z3 (fp32), Y (fp32 [B][2]); with fewer
@@ -2384,7 +2330,9 @@ cfs_status tc_rows(cudaStream_t st, int M, int K, const bf16r* A, int lda, const
 cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
 {
     const bf16r* wb = s->wb;
-    if (rows_on_tma(B) && (uintptr_t)U % 16 == 0) {
+    if ((uintptr_t)U % 16)
+        return fail(CFS_ERR_INVALID_ARG, "sampler inputs must be 16-byte aligned");
+    if (rows_on_tma(B)) {
         // the fused pass (one launch): what the backward reads, and Y
         static int smem_dev = -1;
         if (smem_dev != s->device) {
@@ -2404,18 +2352,15 @@ cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
         train_fwd_kernel<<<grid, TF_THREADS, TF_SMEM, st>>>(wb, s->w, a);
         return check_cuda(cudaGetLastError(), "train_fwd_kernel launch");
     }
-    // Z1, Z2 and the transposed copies only where the backward reads them
-    const bool small = !rows_on_tma(B);
-    cfs_status r = tc_rows(st, B, D_IN, U, D_IN, wb + OFF_W1, D_IN, EPI_SILU, s->w + OFF_B1,
-                           small ? s->Z1 : nullptr, HID, s->H1, HID, small ? s->H1T : nullptr,
-                           s->ldt, nullptr, 0, nullptr);
-    if (r == CFS_OK)
-        r = tc_rows(st, B, HID, s->H1, HID, wb + OFF_W2, HID, EPI_SILU, s->w + OFF_B2,
-                    small ? s->Z2 : nullptr, HID, s->H2, HID, small ? s->H2T : nullptr, s->ldt,
-                    nullptr, 0, nullptr);
-    if (r == CFS_OK)
-        r = tc_rows(st, B, HID, s->H2, HID, wb + OFF_W3, HID, EPI_SILU, s->w + OFF_B3, s->Z3, HID,
-                    s->H3, HID, nullptr, 0, nullptr, 0, nullptr);
+    // with Z1, Z2 and the transposed copies, which the backward of so few rows
+    // reads
+    auto layer = [&](int K, const bf16r* A, int off_w, int off_b, float* Z, bf16r* H, bf16r* HT) {
+        return tc_gemm(st, B, HID, K, A, K, wb + off_w, K, EPI_SILU, s->w + off_b, Z, HID, H, HID,
+                       HT, s->ldt, nullptr, 0, nullptr);
+    };
+    cfs_status r = layer(D_IN, U, OFF_W1, OFF_B1, s->Z1, s->H1, s->H1T);
+    if (r == CFS_OK) r = layer(HID, s->H1, OFF_W2, OFF_B2, s->Z2, s->H2, s->H2T);
+    if (r == CFS_OK) r = layer(HID, s->H2, OFF_W3, OFF_B3, s->Z3, s->H3, nullptr);
     if (r != CFS_OK) return r;
     out_forward_kernel<<<(B + 255) / 256, 256, 0, st>>>(s->H3, wb, s->w, B, s->Y);
     return CFS_OK;
@@ -2470,20 +2415,26 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     if (!part_clear) cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
     out_backward_kernel<<<(B + OB_ROWS - 1) / OB_ROWS, OB_THREADS, 0, st>>>(
         dY, wb, s->Z3, B, s->dZ3, small ? s->dZ3T : nullptr, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
-    // dZ2 = (dZ3 W3) * silu'(Z2): the K-major B operand is W3^T
-    // (on tc_rows_kernel the pre-activations Z2 = H1 W2^T + b2 and Z1 = U W1^T
-    // + b1 are recomputed, bit for bit, instead of read)
-    cfs_status r = tc_rows(st, B, HID, s->dZ3, HID, s->wbT + HID * HID, HID, EPI_SILU_GRAD,
-                           nullptr, nullptr, 0, s->dZ2, HID, small ? s->dZ2T : nullptr, s->ldt,
-                           s->Z2, HID,
-                           s->bias_part, s->H1, HID, wb + OFF_W2, HID, HID, s->w + OFF_B2);
-    if (r == CFS_OK)
-        r = tc_rows(st, B, HID, s->dZ2, HID, s->wbT, HID, EPI_SILU_GRAD, nullptr, nullptr, 0,
-                    small ? nullptr : s->dZ1, HID, small ? s->dZ1T : nullptr, s->ldt, s->Z1, HID,
-                    s->bias_part + TC_COPIES * HID, U,
-                    D_IN, wb + OFF_W1, D_IN, D_IN, s->w + OFF_B1);
+    // dZ2 = (dZ3 W3) * silu'(Z2): the K-major B operand is W3^T; then dZ1
+    // (tc_rows_kernel recomputes the pre-activations Z2 = H1 W2^T + b2 and Z1 =
+    // U W1^T + b1, bit for bit)
+    float *col2 = s->bias_part, *col1 = s->bias_part + TC_COPIES * HID;
+    cfs_status r;
+    if (!small) {
+        r = tc_rows(st, B, s->dZ3, s->wbT + HID * HID, s->dZ2, col2, s->H1, wb + OFF_W2, HID,
+                    s->w + OFF_B2);
+        if (r == CFS_OK)
+            r = tc_rows(st, B, s->dZ2, s->wbT, s->dZ1, col1, U, wb + OFF_W1, D_IN, s->w + OFF_B1);
+        return r == CFS_OK ? tc_dw(s, U, B, grads, st) : r;
+    }
+    auto rows = [&](const bf16r* A, const bf16r* W, bf16r* dZ, bf16r* dZT, const float* Z,
+                    float* col) {
+        return tc_gemm(st, B, HID, HID, A, HID, W, HID, EPI_SILU_GRAD, nullptr, nullptr, 0, dZ, HID,
+                       dZT, s->ldt, Z, HID, col);
+    };
+    r = rows(s->dZ3, s->wbT + HID * HID, s->dZ2, s->dZ2T, s->Z2, col2);
+    if (r == CFS_OK) r = rows(s->dZ2, s->wbT, nullptr, s->dZ1T, s->Z1, col1);
     if (r != CFS_OK) return r;
-    if (rows_on_tma(B)) return tc_dw(s, U, B, grads, st);
     part_reduce_kernel<<<1, 512, 0, st>>>(s->bias_part, grads);
     transpose_in_kernel<<<(B + 31) / 32, 256, 0, st>>>(U, B, s->UT, s->ldt);
     // weight gradients dW = dZ^T A from the transposed copies: K = the rows
@@ -2631,14 +2582,8 @@ cfs_status cfs_sampler_create(const float* params, uint64_t seed, cfs_sampler** 
                                              tc_smem_bytes<2>()),
                         "cudaFuncSetAttribute(tc_gemm_kernel)");
     if (st == CFS_OK)
-        st = check_cuda(cudaFuncSetAttribute(tc_rows_kernel<false>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             TrCfg<false>::SMEM),
-                        "cudaFuncSetAttribute(tc_rows_kernel)");
-    if (st == CFS_OK)
-        st = check_cuda(cudaFuncSetAttribute(tc_rows_kernel<true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             TrCfg<true>::SMEM),
+        st = check_cuda(cudaFuncSetAttribute(tc_rows_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, TR_SMEM),
                         "cudaFuncSetAttribute(tc_rows_kernel)");
     if (st == CFS_OK)
         st = check_cuda(cudaFuncSetAttribute(tc_dw_kernel,
