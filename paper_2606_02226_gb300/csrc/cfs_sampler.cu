@@ -981,23 +981,26 @@ __global__ void __launch_bounds__(256) transpose_in_kernel(const bf16r* __restri
 }
 
 // output layer backward: dH3 = dY W4 (N = 2, not a tensor-core shape), dZ3 =
-// dH3 * silu'(Z3) written as dZ3 and its transpose dZ3^T; dW4 = dY^T H3,
-// db3 = sum dZ3, db4 = sum dY.  A block takes OB_ROWS rows, a warp one row
-// at a time, lane l the four units 4l .. 4l+3 (16-byte loads of Z3, from which
-// H3 is formed again); with dZ3T (batches of fewer than 128 rows) the block's dZ3
-// tile is transposed in shared memory; its sums combine across warps there before one atomic per value into copy
-// blockIdx.x % TC_COPIES of `part`.
+// dH3 * silu'(Z3); dW4 = dY^T H3, db3 = sum dZ3, db4 = sum dY.  Lane l of a
+// warp takes the units 4l .. 4l+3 of a row (16-byte loads of Z3, from which H3
+// is formed again); blocks stride over runs of OB_ROWS rows, and their sums
+// combine across warps in shared memory before one atomic per value into copy
+// blockIdx.x % TC_COPIES of `part`.  SMALL (batches of fewer than 128 rows, a
+// run per block) also writes the transpose dZ3^T.
 constexpr int OB_ROWS = 64;
 constexpr int OB_THREADS = 256;
 
+template <bool SMALL>
 __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* __restrict__ dY,
                                                                   const bf16r* __restrict__ wb,
                                                                   const float* __restrict__ Z3,
                                                                   int B, bf16r* dZ3, bf16r* dZ3T,
                                                                   int ldt, float* part)
 {
-    __shared__ bf16r tT[HID][OB_ROWS + 1];   // the block's dZ3 tile, transposed
+    // the block's dZ3 tile, transposed
+    __shared__ bf16r tT[SMALL ? HID : 1][SMALL ? OB_ROWS + 1 : 1];
     __shared__ float s_sum[3 * HID + 2];     // W4 rows 0 and 1, b3, b4
+    constexpr int WARPS = OB_THREADS / 32, RUN = OB_ROWS / WARPS;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = 4 * lane;
     float w0[4], w1[4], a0[4], a1[4], ab[4];
@@ -1009,31 +1012,44 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
     }
     float b40 = 0.0f, b41 = 0.0f;
     for (int e = threadIdx.x; e < 3 * HID + 2; e += OB_THREADS) s_sum[e] = 0.0f;
-    const int r0 = blockIdx.x * OB_ROWS;
-#pragma unroll 2
-    for (int k = warp; k < OB_ROWS; k += OB_THREADS / 32) {
-        const int r = r0 + k;
-        if (r >= B) break;
-        const float y0 = dY[2 * r], y1 = dY[2 * r + 1];
-        const float4 z = *reinterpret_cast<const float4*>(Z3 + (size_t)r * HID + c);
-        const float zz[4] = {z.x, z.y, z.z, z.w};
-        bf16r db[4];
+    // a warp's RUN consecutive rows, four of them in flight
+    for (int r0 = blockIdx.x * OB_ROWS; r0 < B; r0 += gridDim.x * OB_ROWS) {
+#pragma unroll 1
+        for (int k = 0; k < RUN; k += 4) {
+            const int r = r0 + warp * RUN + k;
+            float4 z[4];
+            float2 y[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float dh = fmaf(y0, w0[j], y1 * w1[j]);
-            const float d = dh * silu_grad_f(zz[j]);
-            // H3 again, the forward's bits (the two share their sigmoid)
-            const float h = from_bf16(to_bf16(silu_f(zz[j])));
-            db[j] = to_bf16(d);
-            if (dZ3T) tT[c + j][k] = db[j];
-            ab[j] += d;
-            a0[j] = fmaf(y0, h, a0[j]);
-            a1[j] = fmaf(y1, h, a1[j]);
+            for (int q = 0; q < 4; ++q) {
+                const bool in = r + q < B;
+                y[q] = in ? __ldg(reinterpret_cast<const float2*>(dY) + r + q)
+                          : make_float2(0.0f, 0.0f);
+                z[q] = in ? __ldcs(reinterpret_cast<const float4*>(Z3 + (size_t)(r + q) * HID + c))
+                          : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (r + q >= B) break;
+                const float zz[4] = {z[q].x, z[q].y, z[q].z, z[q].w};
+                bf16r db[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float dh = fmaf(y[q].x, w0[j], y[q].y * w1[j]);
+                    const float d = dh * silu_grad_f(zz[j]);
+                    // H3 again, the forward's bits (the two share their sigmoid)
+                    const float h = from_bf16(to_bf16(silu_f(zz[j])));
+                    db[j] = to_bf16(d);
+                    if constexpr (SMALL) tT[c + j][warp * RUN + k + q] = db[j];
+                    ab[j] += d;
+                    a0[j] = fmaf(y[q].x, h, a0[j]);
+                    a1[j] = fmaf(y[q].y, h, a1[j]);
+                }
+                *reinterpret_cast<uint2*>(dZ3 + (size_t)(r + q) * HID + c) =
+                    make_uint2((u32)db[0] | ((u32)db[1] << 16), (u32)db[2] | ((u32)db[3] << 16));
+                b40 += y[q].x;
+                b41 += y[q].y;
+            }
         }
-        *reinterpret_cast<uint2*>(dZ3 + (size_t)r * HID + c) =
-            make_uint2((u32)db[0] | ((u32)db[1] << 16), (u32)db[2] | ((u32)db[3] << 16));
-        b40 += y0;
-        b41 += y1;
     }
     __syncthreads();   // tT complete, s_sum zeroed
 #pragma unroll
@@ -1046,15 +1062,19 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
         atomicAdd(&s_sum[3 * HID], b40);
         atomicAdd(&s_sum[3 * HID + 1], b41);
     }
-    // dZ3^T rows: a warp writes 64 consecutive rows of one unit as 32 words
-    for (int e = threadIdx.x; dZ3T && e < HID * (OB_ROWS / 2); e += OB_THREADS) {
-        const int u = e / (OB_ROWS / 2), jp = 2 * (e % (OB_ROWS / 2));
-        const int r = r0 + jp;
-        if (r + 1 < B) {
-            *reinterpret_cast<u32*>(dZ3T + (size_t)u * ldt + r) =
-                (u32)tT[u][jp] | ((u32)tT[u][jp + 1] << 16);
-        } else if (r < B) {
-            dZ3T[(size_t)u * ldt + r] = tT[u][jp];
+    if constexpr (SMALL) {
+        // dZ3^T rows (one run of rows per block): a warp writes 64 consecutive
+        // rows of one unit as 32 words
+        const int r0 = blockIdx.x * OB_ROWS;
+        for (int e = threadIdx.x; e < HID * (OB_ROWS / 2); e += OB_THREADS) {
+            const int u = e / (OB_ROWS / 2), jp = 2 * (e % (OB_ROWS / 2));
+            const int r = r0 + jp;
+            if (r + 1 < B) {
+                *reinterpret_cast<u32*>(dZ3T + (size_t)u * ldt + r) =
+                    (u32)tT[u][jp] | ((u32)tT[u][jp + 1] << 16);
+            } else if (r < B) {
+                dZ3T[(size_t)u * ldt + r] = tT[u][jp];
+            }
         }
     }
     __syncthreads();   // s_sum complete
@@ -1064,8 +1084,8 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
 }
 
 // ---------------------------------------------------------------------------
-// sliced-Wasserstein loss and gradient.  A CTA takes one system and a run of
-// its projections; a group of G = N / 8 threads sorts one projection at a
+// sliced-Wasserstein loss and gradient.  A CTA takes an equal run of the
+// (system, projection) pairs; a group of G = N / 8 threads sorts one projection at a
 // time, each thread holding 8 projected predicted keys (x) and 8 projected
 // target keys (y).
 //
@@ -1076,7 +1096,9 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
 // stage on a bit of the window is a min/max of two slots of one thread.
 // When the next stage's bit lies outside the window, the group moves its
 // keys through shared memory into the window that holds it (19 moves for
-// N = 1024, each one barrier of the group's threads; two buffers alternate).  Blocks that a merge
+// N = 1024, each one barrier of the group's threads; two buffers alternate;
+// windows of 4 bits with 16 keys a thread take 14 moves, but leave 16 warps on
+// an SM instead of 24: 67.4 us against 67.9, no reason to).  Blocks that a merge
 // sorts descending hold their keys negated, so every stage puts the smaller
 // key at the lower position and a merge boundary only flips signs.  The
 // shared-memory slots are XOR-swizzled so that the 16 lanes of a half-warp
@@ -1090,7 +1112,8 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
 // belongs to one thread of the group), then over the groups, then added to
 // dX with one atomic per coordinate and CTA.  Keys must be finite.
 // ---------------------------------------------------------------------------
-constexpr int SW_E = 8;            // keys per thread and set
+constexpr int SW_LG = 3;           // register bits of a window
+constexpr int SW_E = 1 << SW_LG;   // keys per thread and set
 constexpr int SW_THREADS = 256;    // threads per CTA at most
 
 __device__ __forceinline__ float sw_key(float u0, float u1, float c, float sn)
@@ -1107,7 +1130,7 @@ __host__ __device__ constexpr int sw_swz(int p)
 // position bits of thread t in window a (slot bits left zero)
 __device__ __forceinline__ int sw_tpos(int a, int t)
 {
-    return (t & ((1 << a) - 1)) | ((t >> a) << (a + 3));
+    return (t & ((1 << a) - 1)) | ((t >> a) << (a + SW_LG));
 }
 
 // compare-exchange of the slot pairs that differ in register bit M
@@ -1170,7 +1193,7 @@ template <int N, int K, int HI, int CUR>
 __device__ __forceinline__ void sw_windows(float (&x)[SW_E], float (&y)[SW_E], int t, int g,
                                            float2* base, int& par)
 {
-    constexpr int A = HI >= 2 ? HI - 2 : 0;
+    constexpr int A = HI >= SW_LG - 1 ? HI - (SW_LG - 1) : 0;
     if constexpr (A != CUR) sw_move<N, CUR, A>(x, y, t, g, base, par);
     if constexpr (HI - A >= 2) sw_reg_stage<2>(x, y);
     if constexpr (HI - A >= 1) sw_reg_stage<1>(x, y);
@@ -1192,13 +1215,13 @@ __device__ __forceinline__ void sw_merges(float (&x)[SW_E], float (&y)[SW_E], in
 {
     sw_windows<N, K, K - 1, 0>(x, y, t, g, base, par);
     if constexpr ((1 << K) < N) {
-        // window 0 holds position (t << 3) | e: flip where merge K and K + 1
+        // window 0 holds position (t << SW_LG) | e: flip where merge K and K + 1
         // disagree on the sign (t opaque again, as in the moves)
         int tv;
         asm volatile("mov.b32 %0, %1;" : "=r"(tv) : "r"(t));
 #pragma unroll
         for (int e = 0; e < SW_E; ++e) {
-            const int p = (tv << 3) | e;
+            const int p = (tv << SW_LG) | e;
             const bool f = sw_neg<N, K>(p) != sw_neg<N, K + 1>(p);
             const float sg = f ? -1.0f : 1.0f;
             x[e] *= sg;
@@ -1212,7 +1235,7 @@ template <int N>
 __global__ void __launch_bounds__(SW_THREADS, 3) sw_kernel(const float* __restrict__ X,
                                                           const float* __restrict__ T,
                                                           const float* __restrict__ phi, int P,
-                                                          int pc, float scale, float* loss,
+                                                          u64 n_sorts, float scale, float* loss,
                                                           float* dX)
 {
     constexpr int G = N / SW_E;
@@ -1223,99 +1246,111 @@ __global__ void __launch_bounds__(SW_THREADS, 3) sw_kernel(const float* __restri
     float2* bufs = gacc + (size_t)groups * N;          // [groups][2][N]
     __shared__ float red[SW_THREADS / 32];
     const int g = threadIdx.x / G, t = threadIdx.x % G;
-    const int cps = (P + pc - 1) / pc;
-    const int s = blockIdx.x / cps, j0 = (blockIdx.x % cps) * pc, j1 = min(P, j0 + pc);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        const size_t r = ((size_t)s * N + i) * 2;
-        pts[(i & (SW_E - 1)) * G + (i >> 3)] = make_float4(X[r], X[r + 1], T[r], T[r + 1]);
-    }
-    for (int i = threadIdx.x; i < groups * N; i += blockDim.x) gacc[i] = make_float2(0.0f, 0.0f);
-    __syncthreads();
-    float lacc = 0.0f;
-    // each group takes every groups-th projection of the CTA's run; from here
-    // to the final sums a group synchronizes only its own threads
-    for (int j = j0 + g; j < j1; j += groups) {
-        float sn, c;
-        sincosf(phi[j], &sn, &c);
-        // every address below derives from t and g: recomputing them per
-        // projection costs a few integer operations, keeping all of them live
-        // across the loop would cost registers
-        int tt, gg;
-        asm volatile("mov.b32 %0, %1;" : "=r"(tt) : "r"(t));
-        asm volatile("mov.b32 %0, %1;" : "=r"(gg) : "r"(g));
-        float x[SW_E], y[SW_E];
-#pragma unroll
-        for (int e = 0; e < SW_E; ++e) {
-            const float4 q = pts[e * G + tt];
-            // merge 1 starts with the blocks where position bit 1 is set negated
-            const float sg = sw_neg<N, 1>(e) ? -1.0f : 1.0f;
-            x[e] = sg * sw_key(q.x, q.y, c, sn);
-            y[e] = sg * sw_key(q.z, q.w, c, sn);
+    // the sorts (system s, projection j) are numbered s P + j; this CTA takes an
+    // equal run of them, one system of the run after the other
+    const u64 q1 = n_sorts / gridDim.x * (blockIdx.x + 1) +
+                   min((u64)blockIdx.x + 1, n_sorts % gridDim.x);
+    for (u64 q0 = n_sorts / gridDim.x * blockIdx.x + min((u64)blockIdx.x, n_sorts % gridDim.x);
+         q0 < q1;) {
+        const u32 s = (u32)(q0 / (u32)P);
+        const int j0 = (int)(q0 - (u64)s * (u32)P);
+        const int j1 = (int)min((u64)P, (u64)j0 + (q1 - q0));
+        q0 += (u64)(j1 - j0);
+        for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            const size_t r = ((size_t)s * N + i) * 2;
+            pts[(i & (SW_E - 1)) * G + (i >> SW_LG)] = make_float4(X[r], X[r + 1], T[r], T[r + 1]);
         }
-        // the moves alternate between the group's two buffers, starting from
-        // the first in every projection (the barrier after the previous
-        // projection's search makes that safe), so every choice is static
-        int par = 0;
-        sw_merges<N, 1>(x, y, tt, gg, bufs + (size_t)gg * 2 * N, par);
-        // ranks 8t .. 8t+7: squared differences; each rank's gradient
-        // (linear order) and the sorted keys go to the buffer the last move
-        // did not read.  The keys are stored as the binary search visits
-        // them (breadth-first, Eytzinger order: the pivot of rank r = (2m +
-        // 1) h - 1 at node N / 2h + m, node 1 the root), so the first six
-        // levels of every search read at most 32 consecutive words: no bank
-        // conflicts there, where the sorted order put every pivot of a level
-        // in one bank
-        float* sk = reinterpret_cast<float*>(bufs + ((size_t)gg * 2 + par) * N);
-        float* sgr = sk + N;
-        float d[SW_E];
+        for (int i = threadIdx.x; i < groups * N; i += blockDim.x) gacc[i] = make_float2(0.0f, 0.0f);
+        __syncthreads();
+        float lacc = 0.0f;
+        // each group takes every groups-th projection of the CTA's run; from here
+        // to the final sums a group synchronizes only its own threads
+        for (int j = j0 + g; j < j1; j += groups) {
+            float sn, c;
+            sincosf(phi[j], &sn, &c);
+            // every address below derives from t and g: recomputing them per
+            // projection costs a few integer operations, keeping all of them live
+            // across the loop would cost registers
+            int tt, gg;
+            asm volatile("mov.b32 %0, %1;" : "=r"(tt) : "r"(t));
+            asm volatile("mov.b32 %0, %1;" : "=r"(gg) : "r"(g));
+            float x[SW_E], y[SW_E];
 #pragma unroll
-        for (int e = 0; e < SW_E; ++e) {
-            d[e] = x[e] - y[e];
-            lacc = fmaf(d[e], d[e], lacc);
-            d[e] = 2.0f * d[e] / (float)N;
-            const int q = tt * SW_E + e + 1;            // rank + 1
-            if (q < N) {
-                const int tz = __ffs(q) - 1;             // h = 2^tz
-                sk[((N / 2) >> tz) + ((q >> tz) >> 1)] = x[e];
+            for (int e = 0; e < SW_E; ++e) {
+                const float4 q = pts[e * G + tt];
+                // merge 1 starts with the blocks where position bit 1 is set negated
+                const float sg = sw_neg<N, 1>(e) ? -1.0f : 1.0f;
+                x[e] = sg * sw_key(q.x, q.y, c, sn);
+                y[e] = sg * sw_key(q.z, q.w, c, sn);
             }
-        }
-        reinterpret_cast<float4*>(sgr)[2 * tt] = make_float4(d[0], d[1], d[2], d[3]);
-        reinterpret_cast<float4*>(sgr)[2 * tt + 1] = make_float4(d[4], d[5], d[6], d[7]);
-        sw_group_sync<G>(gg);
-#pragma unroll 2
-        for (int e = 0; e < SW_E; ++e) {
-            const int i = tt * SW_E + e;
-            const float4 q = pts[e * G + tt];
-            const float kx = sw_key(q.x, q.y, c, sn);
-            int k = 1;
+            // the moves alternate between the group's two buffers, starting from
+            // the first in every projection (the barrier after the previous
+            // projection's search makes that safe), so every choice is static
+            int par = 0;
+            sw_merges<N, 1>(x, y, tt, gg, bufs + (size_t)gg * 2 * N, par);
+            // ranks 8t .. 8t+7: squared differences; each rank's gradient
+            // (linear order) and the sorted keys go to the buffer the last move
+            // did not read.  The keys are stored as the binary search visits
+            // them (breadth-first, Eytzinger order: the pivot of rank r = (2m +
+            // 1) h - 1 at node N / 2h + m, node 1 the root), so the first six
+            // levels of every search read at most 32 consecutive words: no bank
+            // conflicts there, where the sorted order put every pivot of a level
+            // in one bank
+            float* sk = reinterpret_cast<float*>(bufs + ((size_t)gg * 2 + par) * N);
+            float* sgr = sk + N;
+            float d[SW_E];
 #pragma unroll
-            for (int h = N / 2; h >= 1; h >>= 1) k = 2 * k + (sk[k] < kx ? 1 : 0);
-            const float gv = sgr[k - N];
-            float2 a = gacc[(size_t)gg * N + sw_swz(i)];
-            a.x = fmaf(gv, c, a.x);
-            a.y = fmaf(gv, sn, a.y);
-            gacc[(size_t)gg * N + sw_swz(i)] = a;
+            for (int e = 0; e < SW_E; ++e) {
+                d[e] = x[e] - y[e];
+                lacc = fmaf(d[e], d[e], lacc);
+                d[e] = 2.0f * d[e] / (float)N;
+                const int q = tt * SW_E + e + 1;            // rank + 1
+                if (q < N) {
+                    const int tz = __ffs(q) - 1;             // h = 2^tz
+                    sk[((N / 2) >> tz) + ((q >> tz) >> 1)] = x[e];
+                }
+            }
+#pragma unroll
+            for (int e = 0; e < SW_E; e += 4)
+                reinterpret_cast<float4*>(sgr)[(tt * SW_E + e) / 4] =
+                    make_float4(d[e], d[e + 1], d[e + 2], d[e + 3]);
+            sw_group_sync<G>(gg);
+#pragma unroll 2
+            for (int e = 0; e < SW_E; ++e) {
+                const int i = tt * SW_E + e;
+                const float4 q = pts[e * G + tt];
+                const float kx = sw_key(q.x, q.y, c, sn);
+                int k = 1;
+#pragma unroll
+                for (int h = N / 2; h >= 1; h >>= 1) k = 2 * k + (sk[k] < kx ? 1 : 0);
+                const float gv = sgr[k - N];
+                float2 a = gacc[(size_t)gg * N + sw_swz(i)];
+                a.x = fmaf(gv, c, a.x);
+                a.y = fmaf(gv, sn, a.y);
+                gacc[(size_t)gg * N + sw_swz(i)] = a;
+            }
+            sw_group_sync<G>(gg);
         }
-        sw_group_sync<G>(gg);
-    }
-    float v = lacc;
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-        float ax = 0.0f, ay = 0.0f;
-        for (int q = 0; q < groups; ++q) {
-            const float2 a = gacc[(size_t)q * N + sw_swz(i)];
-            ax += a.x;
-            ay += a.y;
+        float v = lacc;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+        __syncthreads();
+        for (int i = threadIdx.x; i < N; i += blockDim.x) {
+            float ax = 0.0f, ay = 0.0f;
+            for (int q = 0; q < groups; ++q) {
+                const float2 a = gacc[(size_t)q * N + sw_swz(i)];
+                ax += a.x;
+                ay += a.y;
+            }
+            atomicAdd(dX + ((size_t)s * N + i) * 2, ax * scale);
+            atomicAdd(dX + ((size_t)s * N + i) * 2 + 1, ay * scale);
         }
-        atomicAdd(dX + ((size_t)s * N + i) * 2, ax * scale);
-        atomicAdd(dX + ((size_t)s * N + i) * 2 + 1, ay * scale);
-    }
-    if (threadIdx.x == 0) {
-        float tot = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-        atomicAdd(loss, tot * scale / (float)N);
+        if (threadIdx.x == 0) {
+            float tot = 0.0f;
+            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
+            atomicAdd(loss, tot * scale / (float)N);
+        }
+        __syncthreads();                // pts, gacc and red serve the next system
     }
 }
 
@@ -1399,29 +1434,21 @@ void sw_launch(const float* X, const float* T, const float* phi, int P, int N, i
     int groups = std::min(SW_THREADS / G, P);
     const int per_warp = std::max(1, 32 / G);
     groups = std::min(SW_THREADS / G, (groups + per_warp - 1) / per_warp * per_warp);
-    // sorts per group: shortest makespan over the resident CTAs, a CTA
-    // costing its sorts plus about 0.3 of a sort for staging the points and
-    // adding its gradient sums to dX
-    const long slots = (long)std::max(1, d.sms) * std::max(1, d.ctas[sw_log2(N) - 5]);
-    int best_pg = 1;
-    double best = -1.0;
-    for (int pg = 1; pg <= 16; ++pg) {
-        const long ctas = (long)n_sys * ((P + groups * pg - 1) / (groups * pg));
-        const double span = (double)((ctas + slots - 1) / slots) * (pg + 0.3);
-        if (best < 0.0 || span < best) { best = span; best_pg = pg; }
-        if (groups * pg >= P) break;
-    }
-    const int pc = groups * best_pg;
-    const unsigned grid = (unsigned)n_sys * (unsigned)((P + pc - 1) / pc);
+    // as many CTAs as fit, each an equal share of the sorts (whole projections
+    // runs per CTA left 104 SMs with 32 of the 4096 sorts of 64 x 64 and 48
+    // with 16; 27 each now)
+    const u64 slots = (u64)std::max(1, d.sms) * (u64)std::max(1, d.ctas[sw_log2(N) - 5]);
+    const u64 n_sorts = (u64)(u32)n_sys * (u64)P;
+    const unsigned grid = (unsigned)std::min<u64>(slots, (n_sorts - 1) / (u64)groups + 1);
     const unsigned threads = (unsigned)(groups * G);
     const size_t bytes = sw_smem_bytes(N, groups);
     switch (N) {
-    case 32: sw_kernel<32><<<grid, threads, bytes, st>>>(X, T, phi, P, pc, scale, loss, dX); break;
-    case 64: sw_kernel<64><<<grid, threads, bytes, st>>>(X, T, phi, P, pc, scale, loss, dX); break;
-    case 128: sw_kernel<128><<<grid, threads, bytes, st>>>(X, T, phi, P, pc, scale, loss, dX); break;
-    case 256: sw_kernel<256><<<grid, threads, bytes, st>>>(X, T, phi, P, pc, scale, loss, dX); break;
-    case 512: sw_kernel<512><<<grid, threads, bytes, st>>>(X, T, phi, P, pc, scale, loss, dX); break;
-    default: sw_kernel<1024><<<grid, threads, bytes, st>>>(X, T, phi, P, pc, scale, loss, dX); break;
+    case 32: sw_kernel<32><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 64: sw_kernel<64><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 128: sw_kernel<128><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 256: sw_kernel<256><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 512: sw_kernel<512><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    default: sw_kernel<1024><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
     }
 }
 
@@ -2413,8 +2440,14 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     // gradient sums of the output layer and of the biases gather in copies
     // (bias_part) first: fewer atomics on the same address
     if (!part_clear) cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
-    out_backward_kernel<<<(B + OB_ROWS - 1) / OB_ROWS, OB_THREADS, 0, st>>>(
-        dY, wb, s->Z3, B, s->dZ3, small ? s->dZ3T : nullptr, s->ldt, s->bias_part + 2 * TC_COPIES * HID);
+    float* ob = s->bias_part + 2 * TC_COPIES * HID;
+    const int runs = (B + OB_ROWS - 1) / OB_ROWS;
+    if (small)
+        out_backward_kernel<true><<<runs, OB_THREADS, 0, st>>>(dY, wb, s->Z3, B, s->dZ3, s->dZ3T,
+                                                               s->ldt, ob);
+    else
+        out_backward_kernel<false><<<std::min(runs, 4 * std::max(1, device_sm_count())), OB_THREADS,
+                                     0, st>>>(dY, wb, s->Z3, B, s->dZ3, nullptr, 0, ob);
     // dZ2 = (dZ3 W3) * silu'(Z2): the K-major B operand is W3^T; then dZ1
     // (tc_rows_kernel recomputes the pre-activations Z2 = H1 W2^T + b2 and Z1 =
     // U W1^T + b1, bit for bit)
