@@ -1938,7 +1938,10 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
         const float4* c14 = reinterpret_cast<const float4*>(c1);
         const float4* w04 = reinterpret_cast<const float4*>(s_w10);
         const float4* w14 = reinterpret_cast<const float4*>(s_w11);
-#pragma unroll 1
+        // (unrolled: the loads of one group of columns hide behind the others'
+        // tanh; one group at a time took a fifth of the kernel, 206 us for 256 x
+        // 4096 samples against 167)
+#pragma unroll 8
         for (int c0 = 0; c0 < HID; c0 += 8) {
             u32 q[4];
 #pragma unroll
