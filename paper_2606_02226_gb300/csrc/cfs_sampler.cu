@@ -1991,45 +1991,75 @@ __global__ void __launch_bounds__(IT_THREADS, 1) infer_tc_kernel(const bf16r* __
 
 // ---------------------------------------------------------------------------
 // The training forward pass fused per 128-row tile (the same structure as
-// infer_tc_kernel): the tile of inputs U goes from global memory into the
-// group's A tile; layer 1 (K = 64), layer 2 and layer 3 run as tcgen05.mma
+// infer_tc_kernel): layer 1 (K = 64), layer 2 and layer 3 run as tcgen05.mma
 // chains into the group's TMEM columns, each epilogue adding the bias,
-// applying SiLU and writing the next A tile in place.  What the backward
-// pass reads is written on the way, row-major: H1, H2 and Z3; the output
-// layer itself (N = 2) runs on the CUDA cores in the layer-3 epilogue.
+// applying SiLU and writing the next A tile in place; the output layer itself
+// (N = 2) runs on the CUDA cores in the layer-3 epilogue.  What the backward
+// pass reads is written on the way, row-major: H1, H2 and Z3.
+// All tiles are in the 128-byte-swizzled K-major layout (128 rows of 128
+// bytes a block), which the MMAs read and TMA moves: the weights and a tile of
+// inputs arrive, and H1 and H2 leave straight from the A tile while the next
+// layer's MMAs read it, with no thread's loads or stores.  The epilogues' two
+// special-function operations an element (13 us at 65536 rows) are the bound
+// left: 27.5 us there.  The same arithmetic took 53 us with a row per lane for
+// every load and store, and 40 through shared memory in whole lines.
 // ---------------------------------------------------------------------------
 constexpr int TF_GROUPS = 4;
 constexpr int TF_THREADS = 128 * TF_GROUPS;
 constexpr int TF_W1 = HID * D_IN * 2;          // 16 KB
+constexpr int TF_BLOCK = 128 * 128;            // 128 rows of 128 bytes
 constexpr int TF_SMEM = 1024 + TF_W1 + 2 * IT_W + TF_GROUPS * IT_A + 256;
 
-struct TrainFwdArgs {
-    const bf16r* U;                // [B][D_IN]
-    int B;
-    bf16r *H1, *H2;                // [B][HID]
-    float *Z3, *Y;                 // Z3 [B][HID], Y [B][2]
+struct TrainFwdMaps {
+    CUtensorMap U, W1, W2, W3;     // boxes of 128 rows x 64 BF16
+    CUtensorMap H1, H2, Z3;        // Z3 as [B][2 * HID] 16-bit words: 32 floats a box
 };
 
-__global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* __restrict__ wb,
-                                                                  const float* __restrict__ w,
-                                                                  const TrainFwdArgs g)
+struct TrainFwdArgs {
+    int B;
+    float* Y;                      // [B][2]
+};
+
+// a box of shared memory to the tensor map's matrix at (x, y); rows and
+// columns outside it are not written
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, u32 src, int x, int y)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                     reinterpret_cast<u64>(map)),
+                 "r"(x), "r"(y), "r"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void tma_store_commit()
+{
+    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
+// all but the newest N of this thread's store groups have read their source
+template <int N>
+__device__ __forceinline__ void tma_store_read_wait()
+{
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
+}
+
+__global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(
+    const __grid_constant__ TrainFwdMaps m, const bf16r* __restrict__ wb,
+    const float* __restrict__ w, const TrainFwdArgs g)
 {
     extern __shared__ unsigned char tf_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(tf_raw) + 1023) & ~(uintptr_t)1023);
     const u32 sW1 = smem_addr(sm), sW2 = sW1 + TF_W1, sW3 = sW2 + IT_W;
     const u32 sA0 = sW3 + IT_W;
+    // barriers: weights, then per group the inputs and the MMAs
     u64* bars = reinterpret_cast<u64*>(sm + TF_W1 + 2 * IT_W + TF_GROUPS * IT_A);
-    u32* s_tmem = reinterpret_cast<u32*>(bars + TF_GROUPS);
+    u32* s_tmem = reinterpret_cast<u32*>(bars + 1 + 2 * TF_GROUPS);
     __shared__ __align__(16) float s_b1[HID], s_b2[HID], s_b3[HID], s_w4[D_OUT][HID];
     __shared__ float s_b4[2];
     __shared__ int s_err;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const u32 wfull = smem_addr(&bars[0]);
 
-    // weights into the B-operand layout (rows = output features, K = inputs)
-    it_stage_weights<D_IN, TF_THREADS>(sW1, wb + OFF_W1);
-    it_stage_weights<HID, TF_THREADS>(sW2, wb + OFF_W2);
-    it_stage_weights<HID, TF_THREADS>(sW3, wb + OFF_W3);
     for (int j = tid; j < HID; j += TF_THREADS) {
         s_b1[j] = w[OFF_B1 + j];
         s_b2[j] = w[OFF_B2 + j];
@@ -2047,40 +2077,59 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
     }
     if (tid == 0) {
         s_err = 0;
-        for (int q = 0; q < TF_GROUPS; ++q) mbar_init(smem_addr(&bars[q]), 1u);
+        for (int q = 0; q < 1 + 2 * TF_GROUPS; ++q) mbar_init(smem_addr(&bars[q]), 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_expect_tx(wfull, (u32)(TF_W1 + 2 * IT_W));
+        tma_load_2d(sW1, &m.W1, 0, 0, wfull);
+        for (int c = 0; c < 2; ++c) {
+            tma_load_2d(sW2 + c * TF_BLOCK, &m.W2, 64 * c, 0, wfull);
+            tma_load_2d(sW3 + c * TF_BLOCK, &m.W3, 64 * c, 0, wfull);
+        }
     }
-    it_fence_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
 
     const int gi = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
     const u32 sA = sA0 + (u32)(gi * IT_A);
-    const u32 bar = smem_addr(&bars[gi]);
+    const u32 ubar = smem_addr(&bars[1 + gi]), bar = smem_addr(&bars[1 + TF_GROUPS + gi]);
     const u32 tcol = *s_tmem + (u32)(gi * 128);
     const u32 tlane = tcol + ((u32)(wq * 32) << 16);
     const bool issuer = wq == 0 && lane == 0;
     const u32 idesc = tc_idesc(128);
-    u32 phase = 0;
+    u32 phase = 0, uphase = 0;
     int pending = 0;
     bool ok = true;
 
-    auto mma_layer = [&](u32 sW, int K) {
+    // 16 bytes of this thread's row: chunk c of the block at `block`
+    auto chunk = [&](u32 block, int c) { return block + (u32)r * 128u + (u32)((c ^ (r & 7)) * 16); };
+    // the issuer's part of a layer: the MMAs of the A tile with sW
+    auto issue = [&](u32 sW, int K) {
+        tc_fence_after();
+        for (int kk = 0; kk < K / 16; ++kk) {
+            const u32 at = (u32)((kk >> 2) * TF_BLOCK + (kk & 3) * 32);
+            tc_mma(tcol, tc_desc_ksw(sA + at), tc_desc_ksw(sW + at), idesc, kk > 0 ? 1u : 0u);
+        }
+        tc_commit(bar);
+        pending = 1;
+    };
+    // layers 2 and 3: the A tile just written, to the MMAs and to H
+    auto mma_layer = [&](u32 sW, const CUtensorMap* H, int row0) {
         it_fence_async_smem();
         tc_fence_before();
         it_group_sync(gi);
         if (issuer) {
-            tc_fence_after();
-            for (int kk = 0; kk < K / 16; ++kk)
-                tc_mma(tcol, tc_desc_kn(sA + (u32)kk * 4096u, 2048u, 128u),
-                       tc_desc_kn(sW + (u32)kk * 4096u, 2048u, 128u), idesc, kk > 0 ? 1u : 0u);
-            tc_commit(bar);
-            pending = 1;
+            issue(sW, HID);
+            tma_store_2d(H, sA, 0, row0);
+            tma_store_2d(H, sA + TF_BLOCK, 64, row0);
+            tma_store_commit();
         }
     };
-    auto wait_layer = [&]() -> bool {
-        const bool done = it_group_all(gi, mbar_wait(bar, phase));
+    // the layer's accumulator is complete, and the A tile has been read
+    auto wait_layer = [&](bool in_ok) -> bool {
+        const bool mine = in_ok && mbar_wait(bar, phase);
+        if (issuer) tma_store_read_wait<0>();
+        const bool done = it_group_all(gi, mine);
         if (done) {
             phase ^= 1u;
             if (issuer) pending = 0;
@@ -2102,70 +2151,42 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
                 q[2 * j + 1] = pack_bf16x2(silu_f(__uint_as_float(acc[4 * j + 2]) + bb.z),
                                            silu_f(__uint_as_float(acc[4 * j + 3]) + bb.w));
             }
-            it_st16(sA + it_off(r, c0, 2048u), q[0], q[1], q[2], q[3]);
-            it_st16(sA + it_off(r, c0 + 8, 2048u), q[4], q[5], q[6], q[7]);
+            const u32 block = sA + (u32)((c0 >> 6) * TF_BLOCK);
+            const int c = (c0 & 63) / 8;
+            it_st16(chunk(block, c), q[0], q[1], q[2], q[3]);
+            it_st16(chunk(block, c + 1), q[4], q[5], q[6], q[7]);
         });
-    };
-    // the group's A tile -- 16 groups of 16 bytes a row, 2048 B apart -- to 256
-    // bytes of each of the rows row0 .. at `out`, `pitch` bytes apart, while
-    // the MMAs may read it too.  A warp's lanes take 4 rows x 8 groups: whole
-    // 128-byte lines leave, at two lanes a bank (a row per lane, straight from
-    // the epilogue, was 32 lines an instruction, and 8 rows x 4 groups, 64-byte
-    // runs, 9.7 thousand cycles a tile)
-    auto store_tile = [&](void* out, size_t pitch, int row0) {
-        const int rr = lane & 3, kq = lane >> 2;
-#pragma unroll 8
-        for (int e = 0; e < 16; ++e) {
-            const int rt = wq * 32 + (e >> 1) * 4 + rr, kg = (e & 1) * 8 + kq;
-            u32 v[4];
-            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                         : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                         : "r"(sA + (u32)kg * 2048u + (u32)rt * 16u)
-                         : "memory");
-            if (row0 + rt < g.B)
-                *reinterpret_cast<uint4*>(static_cast<unsigned char*>(out) +
-                                          (size_t)(row0 + rt) * pitch + 16 * kg) =
-                    make_uint4(v[0], v[1], v[2], v[3]);
-        }
     };
 
     const int n_tiles = (g.B + 127) / 128;
     for (int tile = blockIdx.x * TF_GROUPS + gi; tile < n_tiles; tile += gridDim.x * TF_GROUPS) {
-        const int row = tile * 128 + r;
+        const int row0 = tile * 128, row = row0 + r;
         const bool in = row < g.B;
-        // the tile's inputs, 64 BF16 values a row, into K groups 0..7 (8 rows x 4
-        // groups a warp instruction, as the weights)
-        {
-            uint4 v[8];
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int rt = tile * 128 + wq * 32 + (e >> 1) * 8 + (lane & 7);
-                const int kg = (e & 1) * 4 + (lane >> 3);
-                v[e] = rt < g.B ? __ldg(reinterpret_cast<const uint4*>(g.U + (size_t)rt * D_IN) + kg)
-                                : make_uint4(0u, 0u, 0u, 0u);
-            }
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int rt = wq * 32 + (e >> 1) * 8 + (lane & 7), kg = (e & 1) * 4 + (lane >> 3);
-                it_st16(sA + (u32)kg * 2048u + (u32)rt * 16u, v[e].x, v[e].y, v[e].z, v[e].w);
-            }
+        bool go = true;
+        if (issuer) {
+            // (the A tile is free: the last tile's stores have read it, below)
+            mbar_expect_tx(ubar, (u32)TF_BLOCK);
+            tma_load_2d(sA, &m.U, 0, row0, ubar);
+            go = mbar_wait(ubar, uphase) && mbar_wait(wfull, 0u);
+            if (go) issue(sW1, D_IN);
         }
-        mma_layer(sW1, D_IN);
-        if (!(ok = wait_layer())) break;
+        uphase ^= 1u;
+        if (!(ok = wait_layer(go))) break;
         hidden_epilogue(s_b1);
-        mma_layer(sW2, HID);
-        store_tile(g.H1, HID * 2, tile * 128);
-        if (!(ok = wait_layer())) break;
+        mma_layer(sW2, &m.H1, row0);
+        if (!(ok = wait_layer(true))) break;
         hidden_epilogue(s_b2);
-        mma_layer(sW3, HID);
-        store_tile(g.H2, HID * 2, tile * 128);
-        if (!(ok = wait_layer())) break;
+        mma_layer(sW3, &m.H2, row0);
+        if (!(ok = wait_layer(true))) break;
         // layer 3: Z3 (FP32) out, and the output layer on the BF16 activations
-        // (which the backward pass forms again from Z3), columns in order.
-        // The A tile holds 64 FP32 columns, so Z3 leaves in two halves
+        // (which the backward pass forms again from Z3), columns in order.  Z3
+        // leaves in quarters of 32 columns through the A tile's two blocks
         float y0 = 0.0f, y1 = 0.0f;
-        auto output_half = [&](int c_half) {
-            u32 a[16], b[16];
+        u32 a[16], b[16];
+        tc_ld16_nowait(tlane, a);
+#pragma unroll 1
+        for (int q = 0; q < 4; ++q) {
+            const u32 block = sA + (u32)((q & 1) * TF_BLOCK);
             auto work = [&](int c0, const u32 (&v)[16]) {
                 const float4* b4 = reinterpret_cast<const float4*>(s_b3 + c0);
                 const float4* p0 = reinterpret_cast<const float4*>(&s_w4[0][c0]);
@@ -2184,28 +2205,29 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
                     y0 = fmaf(h[1], w0.y, y0); y1 = fmaf(h[1], w1.y, y1);
                     y0 = fmaf(h[2], w0.z, y0); y1 = fmaf(h[2], w1.z, y1);
                     y0 = fmaf(h[3], w0.w, y0); y1 = fmaf(h[3], w1.w, y1);
-                    it_st16(sA + (u32)((c0 - c_half) / 4 + j) * 2048u + (u32)r * 16u,
-                            __float_as_uint(z[0]), __float_as_uint(z[1]), __float_as_uint(z[2]),
-                            __float_as_uint(z[3]));
+                    it_st16(chunk(block, (c0 & 31) / 4 + j), __float_as_uint(z[0]),
+                            __float_as_uint(z[1]), __float_as_uint(z[2]), __float_as_uint(z[3]));
                 }
             };
-            tc_ld16_nowait(tlane + (u32)c_half, a);
-#pragma unroll 1
-            for (int c0 = c_half; c0 < c_half + 64; c0 += 32) {
-                tc_wait_ld(a);
-                tc_ld16_nowait(tlane + (u32)(c0 + 16), b);
-                work(c0, a);
-                tc_wait_ld(b);
-                if (c0 + 32 < c_half + 64) tc_ld16_nowait(tlane + (u32)(c0 + 32), a);
-                work(c0 + 16, b);
+            if (q >= 2) {       // the block's last quarter has left
+                if (issuer) tma_store_read_wait<1>();
+                it_group_sync(gi);
             }
-            if (c_half) tc_fence_before();   // TMEM read: the next tile's MMAs may overwrite it
+            tc_wait_ld(a);
+            tc_ld16_nowait(tlane + (u32)(32 * q + 16), b);
+            work(32 * q, a);
+            tc_wait_ld(b);
+            if (q < 3) tc_ld16_nowait(tlane + (u32)(32 * q + 32), a);
+            work(32 * q + 16, b);
+            it_fence_async_smem();
+            if (q == 3) tc_fence_before();   // TMEM read: the next tile's MMAs may overwrite it
             it_group_sync(gi);
-            store_tile(reinterpret_cast<float*>(g.Z3) + c_half, HID * 4, tile * 128);
-            it_group_sync(gi);               // the A tile is free again
-        };
-        output_half(0);
-        output_half(64);
+            if (issuer) {
+                tma_store_2d(&m.Z3, block, 64 * q, row0);
+                tma_store_commit();
+                if (q == 3) tma_store_read_wait<0>();
+            }
+        }
         if (in) {
             g.Y[2 * (size_t)row] = y0 + s_b4[0];
             g.Y[2 * (size_t)row + 1] = y1 + s_b4[1];
@@ -2213,8 +2235,16 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(const bf16r* _
     }
     if (!ok) {
         atomicExch(&s_err, 1);
-        if (issuer && pending) mbar_wait(bar, phase);
+        if (issuer) {
+            if (pending) mbar_wait(bar, phase);
+            mbar_wait(ubar, uphase ^ 1u);      // the last tile's inputs
+        }
     }
+    // the copies into and out of this CTA's shared memory are over before it
+    // may leave: the weights (all of them, also where no tile waited for them)
+    // and every group's stores
+    if (tid == 0) mbar_wait(wfull, 0u);
+    if (issuer) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     if (tid == 0 && s_err) atomicOr(&g_tc_error, (unsigned)CFS_DEVICE_ERR_TC_TIMEOUT);
@@ -2373,13 +2403,22 @@ cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
             if (r != CFS_OK) return r;
             smem_dev = s->device;
         }
-        TrainFwdArgs a;
-        a.U = U; a.B = B;
-        a.H1 = s->H1; a.H2 = s->H2;
-        a.Z3 = s->Z3; a.Y = s->Y;
+        TrainFwdMaps m;
+        auto map = [](CUtensorMap* t, const void* p, int rows, int cols) {
+            return make_tmap_2d_bf16(t, p, (uint64_t)cols, (uint64_t)rows, (uint64_t)cols, 64u,
+                                     128u, true);
+        };
+        cfs_status r = map(&m.U, U, B, D_IN);
+        if (r == CFS_OK) r = map(&m.W1, wb + OFF_W1, HID, D_IN);
+        if (r == CFS_OK) r = map(&m.W2, wb + OFF_W2, HID, HID);
+        if (r == CFS_OK) r = map(&m.W3, wb + OFF_W3, HID, HID);
+        if (r == CFS_OK) r = map(&m.H1, s->H1, B, HID);
+        if (r == CFS_OK) r = map(&m.H2, s->H2, B, HID);
+        if (r == CFS_OK) r = map(&m.Z3, s->Z3, B, 2 * HID);
+        if (r != CFS_OK) return r;
         const int tiles = (B + 127) / 128;
         const int grid = std::max(1, std::min(device_sm_count(), (tiles + TF_GROUPS - 1) / TF_GROUPS));
-        train_fwd_kernel<<<grid, TF_THREADS, TF_SMEM, st>>>(wb, s->w, a);
+        train_fwd_kernel<<<grid, TF_THREADS, TF_SMEM, st>>>(m, wb, s->w, TrainFwdArgs{B, s->Y});
         return check_cuda(cudaGetLastError(), "train_fwd_kernel launch");
     }
     // with Z1, Z2 and the transposed copies, which the backward of so few rows
