@@ -1084,371 +1084,312 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
 }
 
 // ---------------------------------------------------------------------------
-// sliced-Wasserstein loss and gradient.  A CTA takes an equal run of the
-// (system, projection) pairs; a group of G = N / 8 threads sorts one projection at a
-// time, each thread holding 8 projected predicted keys (x) and 8 projected
-// target keys (y).
+// sliced-Wasserstein loss and gradient.  A pair of warps takes the sorts of
+// 1024 / N projections at once: a group of G = N / 32 lanes of the first warp
+// sorts the projected predicted points of one, the same lanes of the second
+// warp its projected target points, each lane holding 32 keys.
 //
-// Sorting network: bitonic.  Merge k (blocks of 2^k positions) runs
-// compare-exchange stages on position bits k-1, ..., 0.  A position's bits
-// are split into a window of 3 register bits [a, a + 3) -- the key's slot
-// in its thread -- and the others, which number the thread in the group; a
-// stage on a bit of the window is a min/max of two slots of one thread.
-// When the next stage's bit lies outside the window, the group moves its
-// keys through shared memory into the window that holds it (19 moves for
-// N = 1024, each one barrier of the group's threads; two buffers alternate;
-// windows of 4 bits with 16 keys a thread take 14 moves, but leave 16 warps on
-// an SM instead of 24: 67.4 us against 67.9, no reason to).  Blocks that a merge
-// sorts descending hold their keys negated, so every stage puts the smaller
-// key at the lower position and a merge boundary only flips signs.  The
-// shared-memory slots are XOR-swizzled so that the 16 lanes of a half-warp
-// hit distinct banks in every window.
+// Sorting network: every lane sorts its 32 keys in registers (Batcher's
+// odd-even merge sort); bitonic merges do the rest.  Merge k (blocks of 2^k
+// positions) runs compare-exchange stages on position bits k-1, ..., 0.  A
+// position's bits are split into a window of 5 register bits [a, a + 5) -- the
+// key's slot in its lane -- and the others, which number the lane; a stage on a
+// bit of the window is a min/max of two slots of one lane.  The stages on
+// bits k-1 .. 5 run in the topmost window and those on bits 4 .. 0 in the lowest,
+// so a merge moves the keys twice through shared memory, 32 stores and 32 loads
+// of a warp without bank conflicts and no barrier but the warp's own.  Blocks
+// that a merge sorts descending hold their keys negated, so every stage puts
+// the smaller key at the lower position and a merge boundary only flips signs.
 //
-// After the sort, thread t holds ranks 8t .. 8t+7.  A point's rank is then
-// found by binary search of its own key (recomputed bit for bit) among the
-// sorted predicted keys, stored in the search's breadth-first order, so the
-// network carries no indices.  Gradients of the
-// group's projections are summed per point in shared memory (each point
-// belongs to one thread of the group), then over the groups, then added to
-// dX with one atomic per coordinate and CTA.  Keys must be finite.
+// A point's rank is then found by binary search of its own key (recomputed bit
+// for bit) among the sorted predicted keys, so the network carries no indices.
+// The gradients of a CTA's projections are summed per point, and added to dX
+// with one atomic per coordinate, system and round of sorts.  Keys must be
+// finite.
+//
+// What it measured (64 systems x 1024 points x 64 projections): 50.6 us.  8 keys of
+// either kind a thread and 128 threads a sort took 67 us, four fifths of the
+// shared memory's cycles for 19 moves; half the moves leave the ALU pipe (min and
+// max, 29 us), the moves (30 us) and the issue slots (27 us) about even.  One
+// warp for both kinds had half the parallelism: 63 us there, and 20 us
+// instead of 12 for 32 sorts.
 // ---------------------------------------------------------------------------
-constexpr int SW_LG = 3;           // register bits of a window
-constexpr int SW_E = 1 << SW_LG;   // keys per thread and set
-constexpr int SW_THREADS = 256;    // threads per CTA at most
+constexpr int SW_LG = 5;           // register bits of a window
+constexpr int SW_E = 1 << SW_LG;   // keys per lane
+constexpr int SW_PAIRS = 4;        // of warps per CTA at most
+// per multiprocessor: 64 registers a thread; 27 of the 4096 sorts of 64 x 64 fall to
+// one, two rounds of its 16 pairs (with 3 CTAs three rounds: 53 us)
+constexpr int SW_CTAS = 4;
+
+__host__ __device__ constexpr int sw_log2(int n)
+{
+    return n > 1 ? 1 + sw_log2(n / 2) : 0;
+}
 
 __device__ __forceinline__ float sw_key(float u0, float u1, float c, float sn)
 {
     return fmaf(u0, c, u1 * sn);
 }
 
-// bank swizzle of a float2 slot: bits 4, 5, 6 fold into the low bits
-__host__ __device__ constexpr int sw_swz(int p)
+// word of position p in a group's array: one word of padding per 32 positions.
+// Positions with disjoint bits add up, so a lane's keys lie at constant
+// distances from its first one; and bit b moves a word by an odd multiple of
+// 2^(b mod 5) banks, so the lanes of both windows hit all banks (the groups of
+// a warp lie at odd multiples of G words)
+__host__ __device__ constexpr int sw_word(int p)
 {
-    return p ^ (((p >> 4) & 1) << 1) ^ (((p >> 5) & 1) << 2) ^ (((p >> 6) & 1) * 9);
+    return p + (p >> 5);
 }
 
-// position bits of thread t in window a (slot bits left zero)
-__device__ __forceinline__ int sw_tpos(int a, int t)
+// words of one group's array
+template <int N>
+constexpr int SW_WORDS = N + N / SW_E;
+
+// all keys of a kind in a CTA
+constexpr int SW_ALL = SW_PAIRS * 32 * (SW_E + 1);
+
+// word of lane t's first key in window A
+template <int A>
+__device__ __forceinline__ int sw_first(int t)
 {
-    return (t & ((1 << a) - 1)) | ((t >> a) << (a + SW_LG));
+    return sw_word((t & ((1 << A) - 1)) | ((t >> A) << (A + SW_LG)));
+}
+
+__device__ __forceinline__ void sw_exchange(float& a, float& b)
+{
+    const float lo = fminf(a, b), hi = fmaxf(a, b);
+    a = lo;
+    b = hi;
+}
+
+// Batcher's odd-even merge sort of a lane's keys, from the exchanges over a
+// distance of D in the merge of runs of P
+template <int P, int D>
+__device__ __forceinline__ void sw_lane_sort(float (&x)[SW_E])
+{
+#pragma unroll
+    for (int e = 0; e + D < SW_E; ++e)
+        if (e >= D % P && (e - D % P) % (2 * D) < D && e / (2 * P) == (e + D) / (2 * P))
+            sw_exchange(x[e], x[e + D]);
+    if constexpr (D > 1)
+        sw_lane_sort<P, D / 2>(x);
+    else if constexpr (2 * P < SW_E)
+        sw_lane_sort<2 * P, 2 * P>(x);
 }
 
 // compare-exchange of the slot pairs that differ in register bit M
 template <int M>
-__device__ __forceinline__ void sw_reg_stage(float (&x)[SW_E], float (&y)[SW_E])
+__device__ __forceinline__ void sw_reg_stage(float (&x)[SW_E])
 {
 #pragma unroll
-    for (int e = 0; e < SW_E; ++e) {
-        if (e & (1 << M)) continue;
-        const int f = e | (1 << M);
-        const float xl = fminf(x[e], x[f]), xh = fmaxf(x[e], x[f]);
-        const float yl = fminf(y[e], y[f]), yh = fmaxf(y[e], y[f]);
-        x[e] = xl; x[f] = xh;
-        y[e] = yl; y[f] = yh;
-    }
+    for (int e = 0; e < SW_E; ++e)
+        if (!(e & (1 << M))) sw_exchange(x[e], x[e | (1 << M)]);
 }
 
-// barrier of the G threads of group g: a named barrier (ids 1 ..) for whole
-// warps, the group's lanes of its warp below that
-template <int G>
-__device__ __forceinline__ void sw_group_sync(int g)
+// the stages on register bits M .. 0
+template <int M>
+__device__ __forceinline__ void sw_reg_stages(float (&x)[SW_E])
 {
-    if constexpr (G >= 64) {
-        asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(G) : "memory");
-    } else if constexpr (G == 32) {
-        __syncwarp();
-    } else {
-        __syncwarp(((1u << G) - 1u) << ((threadIdx.x & 31u) & ~(unsigned)(G - 1)));
-    }
+    sw_reg_stage<M>(x);
+    if constexpr (M > 0) sw_reg_stages<M - 1>(x);
 }
 
-// moves the group's keys from window A to window NA through buffer `par`
-template <int N, int A, int NA>
-__device__ __forceinline__ void sw_move(float (&x)[SW_E], float (&y)[SW_E], int t, int g,
-                                        float2* base, int& par)
+// merge k's stages on position bits 5 and up, from register bit M of window A down
+template <int M, int A>
+__device__ __forceinline__ void sw_high_stages(float (&x)[SW_E], int k)
 {
-    float2* buf = base + (par ? N : 0);
-    par ^= 1;
-    // t passes through an opaque move so that each move computes its own
-    // addresses here instead of all of them staying live from the start
-    int tv;
-    asm volatile("mov.b32 %0, %1;" : "=r"(tv) : "r"(t));
-    t = tv;
-    const int pw = sw_swz(sw_tpos(A, t));
+    if (A + M < k) sw_reg_stage<M>(x);
+    if constexpr (A + M > SW_LG) sw_high_stages<M - 1, A>(x, k);
+}
+
+// moves the group's keys from window A to window NA
+template <int A, int NA>
+__device__ __forceinline__ void sw_move(float (&x)[SW_E], int t, float* buf)
+{
+    float* w = buf + sw_first<A>(t);
+    __syncwarp();               // the last move has read the buffer
 #pragma unroll
-    for (int e = 0; e < SW_E; ++e) buf[pw ^ sw_swz(e << A)] = make_float2(x[e], y[e]);
-    sw_group_sync<N / SW_E>(g);
-    const int pr = sw_swz(sw_tpos(NA, t));
+    for (int e = 0; e < SW_E; ++e) w[sw_word(e << A)] = x[e];
+    __syncwarp();
+    const float* r = buf + sw_first<NA>(t);
 #pragma unroll
-    for (int e = 0; e < SW_E; ++e) {
-        const float2 v = buf[pr ^ sw_swz(e << NA)];
-        x[e] = v.x;
-        y[e] = v.y;
-    }
+    for (int e = 0; e < SW_E; ++e) x[e] = r[sw_word(e << NA)];
 }
 
-// the windows of merge K from the one whose top stage bit is HI down; the
-// keys are in window CUR on entry and in window 0 on return
-template <int N, int K, int HI, int CUR>
-__device__ __forceinline__ void sw_windows(float (&x)[SW_E], float (&y)[SW_E], int t, int g,
-                                           float2* base, int& par)
+// sorts the group's keys: ranks 32 t .. 32 t + 31 in lane t on return.  The
+// keys of odd lanes come negated where N > 32
+template <int N>
+__device__ __forceinline__ void sw_sort(float (&x)[SW_E], int t, float* buf)
 {
-    constexpr int A = HI >= SW_LG - 1 ? HI - (SW_LG - 1) : 0;
-    if constexpr (A != CUR) sw_move<N, CUR, A>(x, y, t, g, base, par);
-    if constexpr (HI - A >= 2) sw_reg_stage<2>(x, y);
-    if constexpr (HI - A >= 1) sw_reg_stage<1>(x, y);
-    sw_reg_stage<0>(x, y);
-    if constexpr (A > 0) sw_windows<N, K, A - 1, A>(x, y, t, g, base, par);
-}
-
-// sign of a key in merge K: negative where position bit K is set (the
-// descending blocks); the last merge (2^K = N) is ascending everywhere
-template <int N, int K>
-__device__ __forceinline__ bool sw_neg(int p)
-{
-    return (1 << K) < N && ((p >> K) & 1);
-}
-
-template <int N, int K>
-__device__ __forceinline__ void sw_merges(float (&x)[SW_E], float (&y)[SW_E], int t, int g,
-                                          float2* base, int& par)
-{
-    sw_windows<N, K, K - 1, 0>(x, y, t, g, base, par);
-    if constexpr ((1 << K) < N) {
-        // window 0 holds position (t << SW_LG) | e: flip where merge K and K + 1
-        // disagree on the sign (t opaque again, as in the moves)
-        int tv;
-        asm volatile("mov.b32 %0, %1;" : "=r"(tv) : "r"(t));
+    constexpr int L = sw_log2(N), A = L - SW_LG;
+    sw_lane_sort<1, 1>(x);
+    if constexpr (A > 0) {
+        // one body for all the merges: unrolled, with the moves and stages of
+        // each, the kernel spent its time fetching instructions
+        bool down = t & 1;
+#pragma unroll 1
+        for (int k = SW_LG + 1; k <= L; ++k) {
+            // lane t of window 0 holds positions (t << 5) | e: its keys are
+            // negated where position bit k is set (not in the last merge)
+            const bool next = k < L && ((t >> (k - SW_LG)) & 1);
+            const float sg = next != down ? -1.0f : 1.0f;
+            down = next;
 #pragma unroll
-        for (int e = 0; e < SW_E; ++e) {
-            const int p = (tv << SW_LG) | e;
-            const bool f = sw_neg<N, K>(p) != sw_neg<N, K + 1>(p);
-            const float sg = f ? -1.0f : 1.0f;
-            x[e] *= sg;
-            y[e] *= sg;
+            for (int e = 0; e < SW_E; ++e) x[e] *= sg;
+            sw_move<0, A>(x, t, buf);
+            sw_high_stages<SW_LG - 1, A>(x, k);
+            sw_move<A, 0>(x, t, buf);
+            sw_reg_stages<SW_LG - 1>(x);
         }
-        sw_merges<N, K + 1>(x, y, t, g, base, par);
     }
+}
+
+// barrier of a pair's 64 threads
+__device__ __forceinline__ void sw_pair_sync(int pair)
+{
+    asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");
 }
 
 template <int N>
-__global__ void __launch_bounds__(SW_THREADS, 3) sw_kernel(const float* __restrict__ X,
-                                                          const float* __restrict__ T,
-                                                          const float* __restrict__ phi, int P,
-                                                          u64 n_sorts, float scale, float* loss,
-                                                          float* dX)
+__global__ void __launch_bounds__(64 * SW_PAIRS, SW_CTAS) sw_kernel(
+    const float* __restrict__ X, const float* __restrict__ T, const float* __restrict__ phi, int P,
+    u64 n_sorts, float scale, float* loss, float* dX)
 {
-    constexpr int G = N / SW_E;
-    extern __shared__ float4 sw_smem[];
-    const int groups = blockDim.x / G;
-    float4* pts = sw_smem;                             // [8][G] (x0, x1, t0, t1), point 8t+e at e*G+t
-    float2* gacc = reinterpret_cast<float2*>(pts + N); // [groups][N] gradient sums
-    float2* bufs = gacc + (size_t)groups * N;          // [groups][2][N]
-    __shared__ float red[SW_THREADS / 32];
-    const int g = threadIdx.x / G, t = threadIdx.x % G;
+    constexpr int G = N / SW_E, HALF = SW_E / 2;
+    __shared__ float s_key[2 * SW_ALL];      // [predicted, target][groups][SW_WORDS]
+    __shared__ float2 s_dir[32 * SW_PAIRS / G];
+    __shared__ float s_loss[2 * SW_PAIRS];
+    const int pair = threadIdx.x >> 6, role = (threadIdx.x >> 5) & 1, lane = threadIdx.x & 31;
+    const u32 g = pair * (32 / G) + lane / G;
+    const int t = lane % G;
+    const u32 groups = (blockDim.x >> 6) * (32 / G);
+    float* key = s_key + g * SW_WORDS<N>;
+    float* buf = key + role * SW_ALL;
+    // points of eight-byte alignment are read as one word
+    const bool wide = (((uintptr_t)X | (uintptr_t)T) & 7u) == 0;
+    auto point = [&](const float* p) -> float2 {
+        return wide ? __ldg(reinterpret_cast<const float2*>(p)) : make_float2(__ldg(p), __ldg(p + 1));
+    };
     // the sorts (system s, projection j) are numbered s P + j; this CTA takes an
-    // equal run of them, one system of the run after the other
+    // equal run of them, one for every group at a time
     const u64 q1 = n_sorts / gridDim.x * (blockIdx.x + 1) +
                    min((u64)blockIdx.x + 1, n_sorts % gridDim.x);
-    for (u64 q0 = n_sorts / gridDim.x * blockIdx.x + min((u64)blockIdx.x, n_sorts % gridDim.x);
-         q0 < q1;) {
-        const u32 s = (u32)(q0 / (u32)P);
-        const int j0 = (int)(q0 - (u64)s * (u32)P);
-        const int j1 = (int)min((u64)P, (u64)j0 + (q1 - q0));
-        q0 += (u64)(j1 - j0);
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            const size_t r = ((size_t)s * N + i) * 2;
-            pts[(i & (SW_E - 1)) * G + (i >> SW_LG)] = make_float4(X[r], X[r + 1], T[r], T[r + 1]);
-        }
-        for (int i = threadIdx.x; i < groups * N; i += blockDim.x) gacc[i] = make_float2(0.0f, 0.0f);
-        __syncthreads();
-        float lacc = 0.0f;
-        // each group takes every groups-th projection of the CTA's run; from here
-        // to the final sums a group synchronizes only its own threads
-        for (int j = j0 + g; j < j1; j += groups) {
+    u64 q0 = n_sorts / gridDim.x * blockIdx.x + min((u64)blockIdx.x, n_sorts % gridDim.x);
+    u32 s0 = (u32)(q0 / (u32)P), j0 = (u32)(q0 - (u64)s0 * (u32)P);
+    float lacc = 0.0f;
+    while (q0 < q1) {
+        const u32 n = (u32)min((u64)groups, q1 - q0);
+        if ((u32)(pair * (32 / G)) < n) {
+            // (a group without a sort repeats the first one and counts for nothing)
+            const u32 j = j0 + (g < n ? g : 0u), s = s0 + j / (u32)P;
             float sn, c;
-            sincosf(phi[j], &sn, &c);
-            // every address below derives from t and g: recomputing them per
-            // projection costs a few integer operations, keeping all of them live
-            // across the loop would cost registers
-            int tt, gg;
-            asm volatile("mov.b32 %0, %1;" : "=r"(tt) : "r"(t));
-            asm volatile("mov.b32 %0, %1;" : "=r"(gg) : "r"(g));
-            float x[SW_E], y[SW_E];
+            sincosf(phi[j % (u32)P], &sn, &c);
+            if (role == 0 && t == 0) s_dir[g] = make_float2(c, sn);
+            // slot e of lane t starts with point e G + t
+            const size_t at = ((size_t)s * N + t) * 2;
+            {
+                const float* p = (role ? T : X) + at;
+                const float sg = N > SW_E && (t & 1) ? -1.0f : 1.0f;
+                float x[SW_E];
+                if (wide) {
 #pragma unroll
-            for (int e = 0; e < SW_E; ++e) {
-                const float4 q = pts[e * G + tt];
-                // merge 1 starts with the blocks where position bit 1 is set negated
-                const float sg = sw_neg<N, 1>(e) ? -1.0f : 1.0f;
-                x[e] = sg * sw_key(q.x, q.y, c, sn);
-                y[e] = sg * sw_key(q.z, q.w, c, sn);
+                    for (int e = 0; e < SW_E; ++e) {
+                        const float2 u = __ldg(reinterpret_cast<const float2*>(p) + e * G);
+                        x[e] = sw_key(u.x, u.y, sg * c, sg * sn);
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < SW_E; ++e)
+                        x[e] = sw_key(__ldg(p + 2 * e * G), __ldg(p + 2 * e * G + 1), sg * c, sg * sn);
+                }
+                sw_sort<N>(x, t, buf);
+                __syncwarp();       // the last move has read the buffer
+#pragma unroll
+                for (int e = 0; e < SW_E; ++e) buf[sw_first<0>(t) + e] = x[e];
             }
-            // the moves alternate between the group's two buffers, starting from
-            // the first in every projection (the barrier after the previous
-            // projection's search makes that safe), so every choice is static
-            int par = 0;
-            sw_merges<N, 1>(x, y, tt, gg, bufs + (size_t)gg * 2 * N, par);
-            // ranks 8t .. 8t+7: squared differences; each rank's gradient
-            // (linear order) and the sorted keys go to the buffer the last move
-            // did not read.  The keys are stored as the binary search visits
-            // them (breadth-first, Eytzinger order: the pivot of rank r = (2m +
-            // 1) h - 1 at node N / 2h + m, node 1 the root), so the first six
-            // levels of every search read at most 32 consecutive words: no bank
-            // conflicts there, where the sorted order put every pivot of a level
-            // in one bank
-            float* sk = reinterpret_cast<float*>(bufs + ((size_t)gg * 2 + par) * N);
-            float* sgr = sk + N;
-            float d[SW_E];
+            sw_pair_sync(pair);
+            // squared differences, and each rank's gradient in place of its
+            // target, half of them by each warp
+            {
+                float* k = key + sw_first<0>(t) + role * HALF;
 #pragma unroll
-            for (int e = 0; e < SW_E; ++e) {
-                d[e] = x[e] - y[e];
-                lacc = fmaf(d[e], d[e], lacc);
-                d[e] = 2.0f * d[e] / (float)N;
-                const int q = tt * SW_E + e + 1;            // rank + 1
-                if (q < N) {
-                    const int tz = __ffs(q) - 1;             // h = 2^tz
-                    sk[((N / 2) >> tz) + ((q >> tz) >> 1)] = x[e];
+                for (int e = 0; e < HALF; ++e) {
+                    const float d = k[e] - k[SW_ALL + e];
+                    if (g < n) lacc = fmaf(d, d, lacc);
+                    k[SW_ALL + e] = 2.0f * d / (float)N;
                 }
             }
+            sw_pair_sync(pair);
+            // half of the points' ranks by bisection.  The first six pivots of
+            // a search lie in different banks for different halves, so only the
+            // last levels, 64 pivots and more, have conflicts
+            float grad[HALF];
+            const float* p = X + at + 2 * G * HALF * role;
 #pragma unroll
-            for (int e = 0; e < SW_E; e += 4)
-                reinterpret_cast<float4*>(sgr)[(tt * SW_E + e) / 4] =
-                    make_float4(d[e], d[e + 1], d[e + 2], d[e + 3]);
-            sw_group_sync<G>(gg);
-#pragma unroll 2
-            for (int e = 0; e < SW_E; ++e) {
-                const int i = tt * SW_E + e;
-                const float4 q = pts[e * G + tt];
-                const float kx = sw_key(q.x, q.y, c, sn);
-                int k = 1;
+            for (int e = 0; e < HALF; ++e) {
+                const float2 u = point(p + 2 * G * e);
+                const float kx = sw_key(u.x, u.y, c, sn);
+                const float* r = key;
 #pragma unroll
-                for (int h = N / 2; h >= 1; h >>= 1) k = 2 * k + (sk[k] < kx ? 1 : 0);
-                const float gv = sgr[k - N];
-                float2 a = gacc[(size_t)gg * N + sw_swz(i)];
-                a.x = fmaf(gv, c, a.x);
-                a.y = fmaf(gv, sn, a.y);
-                gacc[(size_t)gg * N + sw_swz(i)] = a;
+                for (int h = N / 2; h >= 1; h >>= 1) r += r[sw_word(h - 1)] < kx ? sw_word(h) : 0;
+                grad[e] = r[SW_ALL];
             }
-            sw_group_sync<G>(gg);
+            sw_pair_sync(pair);     // the searches have read the keys
+#pragma unroll
+            for (int e = 0; e < HALF; ++e) key[(e + HALF * role) * G + t] = grad[e];
         }
-        float v = lacc;
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
         __syncthreads();
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            float ax = 0.0f, ay = 0.0f;
-            for (int q = 0; q < groups; ++q) {
-                const float2 a = gacc[(size_t)q * N + sw_swz(i)];
-                ax += a.x;
-                ay += a.y;
+        for (u32 a = 0; a < n;) {
+            const u32 b = min(n, a + ((u32)P - j0));    // the round's sorts of system s0
+            for (int i = threadIdx.x; i < N; i += blockDim.x) {
+                float ax = 0.0f, ay = 0.0f;
+                for (u32 h = a; h < b; ++h) {
+                    const float v = s_key[h * SW_WORDS<N> + i];
+                    ax = fmaf(v, s_dir[h].x, ax);
+                    ay = fmaf(v, s_dir[h].y, ay);
+                }
+                atomicAdd(dX + ((size_t)s0 * N + i) * 2, ax * scale);
+                atomicAdd(dX + ((size_t)s0 * N + i) * 2 + 1, ay * scale);
             }
-            atomicAdd(dX + ((size_t)s * N + i) * 2, ax * scale);
-            atomicAdd(dX + ((size_t)s * N + i) * 2 + 1, ay * scale);
+            j0 += b - a;
+            if (j0 == (u32)P) {
+                j0 = 0;
+                ++s0;
+            }
+            a = b;
         }
-        if (threadIdx.x == 0) {
-            float tot = 0.0f;
-            for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += red[w];
-            atomicAdd(loss, tot * scale / (float)N);
-        }
-        __syncthreads();                // pts, gacc and red serve the next system
+        q0 += n;
+        __syncthreads();        // the arrays serve the next round
+    }
+    for (int o = 16; o > 0; o >>= 1) lacc += __shfl_xor_sync(0xffffffffu, lacc, o);
+    if (lane == 0) s_loss[threadIdx.x >> 5] = lacc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float tot = 0.0f;
+        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) tot += s_loss[w];
+        atomicAdd(loss, tot * scale / (float)N);
     }
 }
 
-// dynamic shared memory of sw_kernel<N> with `groups` groups
-size_t sw_smem_bytes(int N, int groups)
-{
-    return sizeof(float4) * N + sizeof(float2) * 3 * (size_t)N * groups;
-}
-
-template <int N>
-const void* sw_func()
-{
-    return reinterpret_cast<const void*>(&sw_kernel<N>);
-}
-
-const void* sw_kernel_of(int N)
-{
-    switch (N) {
-    case 32: return sw_func<32>();
-    case 64: return sw_func<64>();
-    case 128: return sw_func<128>();
-    case 256: return sw_func<256>();
-    case 512: return sw_func<512>();
-    default: return sw_func<1024>();
-    }
-}
-
-// per device: the shared-memory opt-in of every sw_kernel instance and how
-// many full-size CTAs of each fit on an SM (set outside stream capture)
-struct SwDevInfo {
-    bool ready = false;
-    int sms = 0;
-    int ctas[6] = {0, 0, 0, 0, 0, 0};
-};
-SwDevInfo g_sw_info[64];
-
-int sw_log2(int N)
-{
-    int l = 0;
-    while ((1 << l) < N) ++l;
-    return l;
-}
-
-cfs_status sw_init()
-{
-    int dev = 0;
-    cfs_status st = cfs::check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
-    if (st != CFS_OK) return st;
-    if (dev < 0 || dev >= 64) return cfs::fail(CFS_ERR_UNSUPPORTED, "device index out of range");
-    SwDevInfo& d = g_sw_info[dev];
-    if (d.ready) return CFS_OK;
-    st = cfs::check_cuda(cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev), "SMs");
-    for (int N = 32; N <= 1024 && st == CFS_OK; N *= 2) {
-        const int groups = SW_THREADS / (N / SW_E);
-        const size_t bytes = sw_smem_bytes(N, groups);
-        const void* f = sw_kernel_of(N);
-        st = cfs::check_cuda(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)bytes),
-                        "cudaFuncSetAttribute(sw_kernel)");
-        int n = 0;
-        if (st == CFS_OK)
-            st = cfs::check_cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, f, SW_THREADS,
-                                                                          bytes),
-                            "occupancy(sw_kernel)");
-        d.ctas[sw_log2(N) - 5] = std::max(1, n);
-    }
-    if (st == CFS_OK) d.ready = true;
-    return st;
-}
-
-// launches the SW kernel for N points per system (a power of two, 32..1024);
-// sw_init() must have run on this device
+// launches the SW kernel for N points per system (a power of two, 32..1024)
 void sw_launch(const float* X, const float* T, const float* phi, int P, int N, int n_sys,
                float scale, float* loss, float* dX, cudaStream_t st)
 {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    const SwDevInfo& d = g_sw_info[dev >= 0 && dev < 64 ? dev : 0];
-    const int G = N / SW_E;
-    // groups per CTA: enough for the projections, whole warps
-    int groups = std::min(SW_THREADS / G, P);
-    const int per_warp = std::max(1, 32 / G);
-    groups = std::min(SW_THREADS / G, (groups + per_warp - 1) / per_warp * per_warp);
-    // as many CTAs as fit, each an equal share of the sorts (whole projections
-    // runs per CTA left 104 SMs with 32 of the 4096 sorts of 64 x 64 and 48
-    // with 16; 27 each now)
-    const u64 slots = (u64)std::max(1, d.sms) * (u64)std::max(1, d.ctas[sw_log2(N) - 5]);
+    const u64 sms = (u64)std::max(1, cfs::device_sm_count());
     const u64 n_sorts = (u64)(u32)n_sys * (u64)P;
-    const unsigned grid = (unsigned)std::min<u64>(slots, (n_sorts - 1) / (u64)groups + 1);
-    const unsigned threads = (unsigned)(groups * G);
-    const size_t bytes = sw_smem_bytes(N, groups);
+    // as many pairs of warps as there are sorts for, first one on every
+    // multiprocessor; then as many CTAs as fit, each an equal share of the sorts
+    const u64 pairs = (n_sorts - 1) / (u64)(32 * SW_E / N) + 1;
+    const unsigned w = (unsigned)std::min<u64>(SW_PAIRS, (pairs - 1) / sms + 1);
+    const unsigned grid = (unsigned)std::min<u64>(sms * SW_CTAS, (pairs - 1) / w + 1);
+    const unsigned threads = 64 * w;
     switch (N) {
-    case 32: sw_kernel<32><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 64: sw_kernel<64><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 128: sw_kernel<128><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 256: sw_kernel<256><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 512: sw_kernel<512><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    default: sw_kernel<1024><<<grid, threads, bytes, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 32: sw_kernel<32><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 64: sw_kernel<64><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 128: sw_kernel<128><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 256: sw_kernel<256><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 512: sw_kernel<512><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    default: sw_kernel<1024><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
     }
 }
 
@@ -2664,7 +2605,6 @@ cfs_status cfs_sampler_create(const float* params, uint64_t seed, cfs_sampler** 
         st = check_cuda(cudaFuncSetAttribute(tc_dw_kernel,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM),
                         "cudaFuncSetAttribute(tc_dw_kernel)");
-    if (st == CFS_OK) st = sw_init();
     if (st == CFS_OK) st = check_cuda(cudaMalloc(&s->d_step, 256), "cudaMalloc(step)");
     if (st == CFS_OK) st = check_cuda(cudaMemset(s->m, 0, sizeof(float) * N_PARAMS * 2), "memset");
     if (st == CFS_OK) st = check_cuda(cudaMemset(s->d_step, 0, 256), "memset");
@@ -2773,8 +2713,6 @@ cfs_status cfs_sw_loss(const float* X, const float* T, uint32_t n_sys, uint32_t 
         return fail(CFS_ERR_INVALID_ARG, "points per system must be a power of two in 32..1024");
     if (n_sys == 0 || n_proj == 0) return CFS_OK;
     const float scale = 1.0f / ((float)n_sys * (float)n_proj);
-    cfs_status st = sw_init();
-    if (st != CFS_OK) return st;
     sw_launch(X, T, phi, (int)n_proj, (int)n_per, (int)n_sys, scale, loss, dX,
               (cudaStream_t)stream);
     return check_cuda(cudaGetLastError(), "sw_kernel launch");
