@@ -126,6 +126,16 @@ struct TcArgs {
                                  // adds its column sums into copy b % TC_COPIES
 };
 
+// Waits for the grid before this one in the stream where this one was launched
+// to start early (launch_after), and lets the next one do so.  In this order:
+// what ran before the previous grid is then complete for the next one's part
+// before its own wait, which loads weights and touches nothing else
+__device__ __forceinline__ void after_previous()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ u32 smem_addr(const void* p)
 {
     return (u32)__cvta_generic_to_shared(p);
@@ -610,6 +620,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) tc_dw_kernel(const __grid_const
 {
     extern __shared__ unsigned char dw_smem_raw[];
     if ((int)blockIdx.x >= g.cta0[3]) {
+        after_previous();
         part_reduce(g.part, g.grads);
         return;
     }
@@ -649,6 +660,7 @@ __global__ void __launch_bounds__(DW_THREADS, 1) tc_dw_kernel(const __grid_const
     __syncthreads();
     tc_fence_after();
     const u32 tmem = *s_tmem;
+    after_previous();
     // slot s: A at s0 + s DW_SLOT (two boxes), B after it (N / 64 boxes)
     if (warp == 0) {
         if (lane == 0) {
@@ -813,6 +825,7 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
         a0[j] = a1[j] = ab[j] = 0.0f;
     }
     float b40 = 0.0f, b41 = 0.0f;
+    after_previous();       // (the weights are older)
     for (int e = threadIdx.x; e < 3 * HID + 2; e += OB_THREADS) s_sum[e] = 0.0f;
     // a warp's RUN consecutive rows, four of them in flight
     for (int r0 = blockIdx.x * OB_ROWS; r0 < B; r0 += gridDim.x * OB_ROWS) {
@@ -1061,6 +1074,7 @@ __global__ void __launch_bounds__(64 * SW_PAIRS, SW_CTAS) sw_kernel(
     __shared__ float s_key[2 * SW_ALL];      // [predicted, target][groups][SW_WORDS]
     __shared__ float2 s_dir[32 * SW_PAIRS / G];
     __shared__ float s_loss[2 * SW_PAIRS];
+    after_previous();
     const int pair = threadIdx.x >> 6, role = (threadIdx.x >> 5) & 1, lane = threadIdx.x & 31;
     const u32 g = pair * (32 / G) + lane / G;
     const int t = lane % G;
@@ -1173,8 +1187,30 @@ __global__ void __launch_bounds__(64 * SW_PAIRS, SW_CTAS) sw_kernel(
     }
 }
 
+// Launches `kernel`, which calls after_previous(); where the stream's previous
+// operation is a kernel of this file that does so too (`after`), it may start
+// while that one's last CTAs run: their tail hides its launch, its TMEM and its
+// weights (loss and gradients of 65536 rows 191 -> 184 us; replayed in a graph,
+// where the launches are cheaper, 1 us a step).
+template <class... Params, class... Args>
+void launch_after(bool after, void (*kernel)(Params...), unsigned grid, unsigned threads,
+                  size_t smem, cudaStream_t st, const Args&... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &attr;
+    c.numAttrs = after ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, Params(args)...);
+}
+
 // launches the SW kernel for N points per system (a power of two, 32..1024)
-void sw_launch(const float* X, const float* T, const float* phi, int P, int N, int n_sys,
+void sw_launch(bool after, const float* X, const float* T, const float* phi, int P, int N, int n_sys,
                float scale, float* loss, float* dX, cudaStream_t st)
 {
     const u64 sms = (u64)std::max(1, cfs::device_sm_count());
@@ -1184,14 +1220,16 @@ void sw_launch(const float* X, const float* T, const float* phi, int P, int N, i
     const u64 pairs = (n_sorts - 1) / (u64)(32 * SW_E / N) + 1;
     const unsigned w = (unsigned)std::min<u64>(SW_PAIRS, (pairs - 1) / sms + 1);
     const unsigned grid = (unsigned)std::min<u64>(sms * SW_CTAS, (pairs - 1) / w + 1);
-    const unsigned threads = 64 * w;
+    auto sw = [&](auto* kernel) {
+        launch_after(after, kernel, grid, 64 * w, 0, st, X, T, phi, P, n_sorts, scale, loss, dX);
+    };
     switch (N) {
-    case 32: sw_kernel<32><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 64: sw_kernel<64><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 128: sw_kernel<128><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 256: sw_kernel<256><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    case 512: sw_kernel<512><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
-    default: sw_kernel<1024><<<grid, threads, 0, st>>>(X, T, phi, P, n_sorts, scale, loss, dX); break;
+    case 32: sw(&sw_kernel<32>); break;
+    case 64: sw(&sw_kernel<64>); break;
+    case 128: sw(&sw_kernel<128>); break;
+    case 256: sw(&sw_kernel<256>); break;
+    case 512: sw(&sw_kernel<512>); break;
+    default: sw(&sw_kernel<1024>); break;
     }
 }
 
@@ -1231,6 +1269,7 @@ __global__ void __launch_bounds__(256) adam_kernel(float* w, float* m, float* v,
                                                    float b1, float b2, float eps,
                                                    const float* loss, float* hist)
 {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
         const u32 t = step ? (*step + 1u) : t_explicit;
@@ -1344,6 +1383,7 @@ __global__ void __launch_bounds__(256) data_kernel(const __grid_constant__ DataA
 {
     __shared__ SysRec s_sys[256 / 32];   // rows of a block: at most 8 systems (N >= 32)
     __shared__ u32 s_sel[256 / 32];
+    after_previous();
     const u32 st = *a.step;
     const int r0 = blockIdx.x * blockDim.x;
     const int first = r0 / a.N, last = min(r0 + (int)blockDim.x - 1, a.rows - 1) / a.N;
@@ -1835,6 +1875,8 @@ __global__ void __launch_bounds__(TF_THREADS, 1) train_fwd_kernel(
     __syncthreads();
     tc_fence_after();
 
+    after_previous();       // (the weights are older)
+
     const int gi = warp >> 2, wq = warp & 3, r = wq * 32 + lane;
     const u32 sA = sA0 + (u32)(gi * IT_A);
     const u32 ubar = smem_addr(&bars[1 + gi]), bar = smem_addr(&bars[1 + TF_GROUPS + gi]);
@@ -2077,6 +2119,8 @@ __global__ void __launch_bounds__(BR_THREADS, 1) back_rows_kernel(
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+
+    after_previous();       // (the weights are older)
 
     const int gi = tid / BR_GT, quad = warp & 3, half = (warp >> 2) & 1;
     const int r = quad * 32 + lane;
@@ -2371,7 +2415,8 @@ cfs_status box_map(CUtensorMap* t, const void* p, int rows, int cols)
 
 // forward of B rows of U: H1..H3 (bf16), Z3 (fp32), Y (fp32 [B][2]); with fewer
 // rows than one tile also Z1, Z2, H1^T, H2^T
-cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
+// (after: as for launch_after)
+cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st, bool after = false)
 {
     const bf16r* wb = s->wb;
     if ((uintptr_t)U % 16)
@@ -2398,7 +2443,8 @@ cfs_status forward(cfs_sampler* s, const bf16r* U, int B, cudaStream_t st)
         if (r != CFS_OK) return r;
         const int tiles = (B + 127) / 128;
         const int grid = std::max(1, std::min(device_sm_count(), (tiles + TF_GROUPS - 1) / TF_GROUPS));
-        train_fwd_kernel<<<grid, TF_THREADS, TF_SMEM, st>>>(m, wb, s->w, TrainFwdArgs{B, s->Y});
+        launch_after(after, train_fwd_kernel, grid, TF_THREADS, TF_SMEM, st, m, wb, s->w,
+                     TrainFwdArgs{B, s->Y});
         return check_cuda(cudaGetLastError(), "train_fwd_kernel launch");
     }
     // with Z1, Z2 and the transposed copies, which the backward of so few rows
@@ -2432,8 +2478,8 @@ cfs_status back_rows(cfs_sampler* s, const bf16r* U, int B, float* col2, float* 
     if (r != CFS_OK) return r;
     const int tiles = (B + 127) / 128;
     const int grid = std::max(1, std::min(device_sm_count(), (tiles + BR_GROUPS - 1) / BR_GROUPS));
-    back_rows_kernel<<<grid, BR_THREADS, BR_SMEM, st>>>(
-        m, BackRowsArgs{B, s->w + OFF_B2, s->w + OFF_B1, col2, col1});
+    launch_after(true, back_rows_kernel, grid, BR_THREADS, BR_SMEM, st, m,
+                 BackRowsArgs{B, s->w + OFF_B2, s->w + OFF_B1, col2, col1});
     return check_cuda(cudaGetLastError(), "back_rows_kernel launch");
 }
 
@@ -2468,14 +2514,14 @@ cfs_status tc_dw(cfs_sampler* s, const bf16r* U, int B, float* grads, cudaStream
     }
     if ((uintptr_t)grads % 16)
         return fail(CFS_ERR_INVALID_ARG, "weight-gradient GEMM operands not aligned");
-    tc_dw_kernel<<<g.cta0[3] + 1, DW_THREADS, DW_SMEM, st>>>(m, g);
+    launch_after(true, tc_dw_kernel, g.cta0[3] + 1, DW_THREADS, DW_SMEM, st, m, g);
     return check_cuda(cudaGetLastError(), "tc_dw_kernel launch");
 }
 
-// backward of sum(dY * Y) after forward(): adds into grads [N_PARAMS]
-// (part_clear: the gradient copies are zero already)
+// backward of sum(dY * Y), after a kernel of this file; forward() has run and
+// bias_part is zero: adds into grads [N_PARAMS]
 cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, float* grads,
-                    cudaStream_t st, bool part_clear = false)
+                    cudaStream_t st)
 {
     const bf16r* wb = s->wb;
     // fewer rows than one tile: the register-staged GEMMs, whose weight
@@ -2483,15 +2529,15 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     const bool small = !rows_on_tma(B);
     // gradient sums of the output layer and of the biases gather in copies
     // (bias_part) first: fewer atomics on the same address
-    if (!part_clear) cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, st);
     float* ob = s->bias_part + 2 * TC_COPIES * HID;
     const int runs = (B + OB_ROWS - 1) / OB_ROWS;
     if (small)
-        out_backward_kernel<true><<<runs, OB_THREADS, 0, st>>>(dY, wb, s->Z3, B, s->dZ3, s->dZ3T,
-                                                               s->ldt, ob);
+        launch_after(true, &out_backward_kernel<true>, runs, OB_THREADS, 0, st, dY, wb, s->Z3, B,
+                     s->dZ3, s->dZ3T, s->ldt, ob);
     else
-        out_backward_kernel<false><<<std::min(runs, 4 * std::max(1, device_sm_count())), OB_THREADS,
-                                     0, st>>>(dY, wb, s->Z3, B, s->dZ3, nullptr, 0, ob);
+        launch_after(true, &out_backward_kernel<false>,
+                     std::min(runs, 4 * std::max(1, device_sm_count())), OB_THREADS, 0, st, dY, wb,
+                     s->Z3, B, s->dZ3, nullptr, 0, ob);
     // dZ2 = (dZ3 W3) * silu'(Z2), then dZ1
     float *col2 = s->bias_part, *col1 = s->bias_part + TC_COPIES * HID;
     cfs_status r;
@@ -2755,6 +2801,7 @@ cfs_status cfs_sampler_backward(cfs_sampler* s, const void* U, uint32_t B, const
     cfs_status st = ensure_rows(s, (int)B);
     if (st != CFS_OK) return st;
     cudaStream_t sm = (cudaStream_t)stream;
+    cudaMemsetAsync(s->bias_part, 0, sizeof(float) * PART_FLOATS, sm);
     st = forward(s, (const bf16r*)U, (int)B, sm);
     if (st == CFS_OK) st = backward(s, (const bf16r*)U, (int)B, dY, grads, sm);
     if (st != CFS_OK) return st;
@@ -2770,7 +2817,7 @@ cfs_status cfs_sw_loss(const float* X, const float* T, uint32_t n_sys, uint32_t 
         return fail(CFS_ERR_INVALID_ARG, "points per system must be a power of two in 32..1024");
     if (n_sys == 0 || n_proj == 0) return CFS_OK;
     const float scale = 1.0f / ((float)n_sys * (float)n_proj);
-    sw_launch(X, T, phi, (int)n_proj, (int)n_per, (int)n_sys, scale, loss, dX,
+    sw_launch(false, X, T, phi, (int)n_proj, (int)n_per, (int)n_sys, scale, loss, dX,
               (cudaStream_t)stream);
     return check_cuda(cudaGetLastError(), "sw_kernel launch");
 }
@@ -2874,14 +2921,13 @@ cfs_status cfs_sampler_train_ex(cfs_sampler* s, const cfs_system* const* systems
         da.zero_b = s->bias_part; da.n_b = PART_FLOATS;
         da.dY = d_dY;
         data_kernel<<<(B + 255) / 256, 256, 0, cap>>>(da);
-        cfs_status fst = forward(s, d_U, B, cap);
-        sw_launch(s->Y, d_T, d_phi, (int)n_proj, N, S, 1.0f / ((float)S * (float)n_proj),
+        cfs_status fst = forward(s, d_U, B, cap, true);
+        sw_launch(true, s->Y, d_T, d_phi, (int)n_proj, N, S, 1.0f / ((float)S * (float)n_proj),
                   d_loss, d_dY, cap);
-        if (fst == CFS_OK) fst = backward(s, d_U, B, d_dY, d_g, cap, true);
-        adam_kernel<<<(N_PARAMS + 255) / 256, 256, 0, cap>>>(s->w, s->m, s->v, d_g, s->wb, s->wbT,
-                                                             N_PARAMS, s->d_step, 0u, lr,
-                                                             lr_final, step0, steps, 0.9f,
-                                                             0.999f, 1e-8f, d_loss, d_hist);
+        if (fst == CFS_OK) fst = backward(s, d_U, B, d_dY, d_g, cap);
+        launch_after(true, adam_kernel, (N_PARAMS + 255) / 256, 256, 0, cap, s->w, s->m, s->v, d_g,
+                     s->wb, s->wbT, N_PARAMS, s->d_step, 0u, lr, lr_final, step0, steps, 0.9f,
+                     0.999f, 1e-8f, d_loss, d_hist);
         cudaError_t e = cudaGetLastError();
         cudaError_t e2 = cudaStreamEndCapture(cap, &graph);
         st = check_cuda(e != cudaSuccess ? e : e2, "training step capture");
