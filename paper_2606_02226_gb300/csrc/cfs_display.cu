@@ -35,6 +35,7 @@ struct DispArgs {
     float* a_max;                 // device [n_layers]
     int n_layers;
     u32 n_items;
+    u32 parts_log2;               // an item's pixels are dealt to 2^parts_log2 CTAs
     float inv_gamma, brightness, a_max_fixed;
     u32 background;
 };
@@ -119,16 +120,32 @@ __device__ __forceinline__ float block_max(float m, float* red)
     return m;
 }
 
+__device__ __forceinline__ u32 item_of(const DispArgs& a, u32 v)
+{
+    return v >> a.parts_log2;
+}
+
+// the pixels [p0, p1) of part v of the launch (p0 >= p1 where the layer ends
+// before them)
+__device__ __forceinline__ void part_of(const DispArgs& a, u32 v, const DisplayLayer& L, u32& p0,
+                                        u32& p1)
+{
+    const u32 px = kDisplayPxPerItem >> a.parts_log2;
+    p0 = (item_of(a, v) - L.item_begin) * kDisplayPxPerItem +
+         (v & ((1u << a.parts_log2) - 1u)) * px;
+    p1 = min(L.n_px, p0 + px);
+}
+
 __global__ void __launch_bounds__(kThreads) density_max_kernel(const __grid_constant__ DispArgs a)
 {
     __shared__ __align__(16) DisplayLayer sL;
     __shared__ float red[kThreads / 32];
-    for (u32 item = blockIdx.x; item < a.n_items; item += gridDim.x) {
-        const int li = load_layer(a, item, sL);
+    for (u32 v = blockIdx.x; item_of(a, v) < a.n_items; v += gridDim.x) {
+        const int li = load_layer(a, item_of(a, v), sL);
         float m = 0.0f;
         if (sL.kind != CFS_TARGET_DEPTH_U64) {
-            const u32 p0 = (item - sL.item_begin) * kDisplayPxPerItem;
-            const u32 p1 = min(sL.n_px, p0 + kDisplayPxPerItem);
+            u32 p0, p1;
+            part_of(a, v, sL, p0, p1);
             const bool planes_ok = sL.kind != CFS_TARGET_HIST_U32 || (sL.n_px & 3u) == 0;
             for (u32 p = p0 + 4 * threadIdx.x; p < p1; p += 4 * kThreads) {
                 float4 s[4];
@@ -167,10 +184,10 @@ __device__ __forceinline__ u32 map_pixel(const float4 s, float l_max, const Disp
 __global__ void __launch_bounds__(kThreads, 4) display_map_kernel(const __grid_constant__ DispArgs a)
 {
     __shared__ __align__(16) DisplayLayer sL;
-    for (u32 item = blockIdx.x; item < a.n_items; item += gridDim.x) {
-        const int li = load_layer(a, item, sL);
-        const u32 p0 = (item - sL.item_begin) * kDisplayPxPerItem;
-        const u32 p1 = min(sL.n_px, p0 + kDisplayPxPerItem);
+    for (u32 v = blockIdx.x; item_of(a, v) < a.n_items; v += gridDim.x) {
+        const int li = load_layer(a, item_of(a, v), sL);
+        u32 p0, p1;
+        part_of(a, v, sL, p0, p1);
         u32* out = reinterpret_cast<u32*>(sL.out);
         if (sL.kind == CFS_TARGET_DEPTH_U64) {
             const u64* keys = reinterpret_cast<const u64*>(sL.data);
@@ -321,8 +338,13 @@ cfs_status display_enqueue(const DisplayLayer* one, const DisplayLayer* layers, 
     a.brightness = p.brightness;
     a.a_max_fixed = p.a_max > 0.0f ? p.a_max : 0.0f;
     a.background = p.background;
-    const int sms = device_sm_count();
-    const unsigned grid = (unsigned)std::min<uint64_t>(n_items, (uint64_t)std::max(1, sms) * 8);
+    // one CTA an item, 8 per multiprocessor at most; where there are fewer items
+    // than that, each goes to 2, 4 or 8 CTAs, which still have a load of four
+    // pixels for every thread (a 320 x 240 layer of 4 channels, 10 items: 16 + 33 us
+    // for both passes on 10 CTAs, 4.5 + 7.8 on 80; 1920 x 1080: 6.6 us a pass)
+    const uint64_t most = (uint64_t)std::max(1, device_sm_count()) * 8;
+    while (a.parts_log2 < 3 && ((uint64_t)n_items << (a.parts_log2 + 1)) <= most) ++a.parts_log2;
+    const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)n_items << a.parts_log2, most);
     if (any_density && !(p.a_max > 0.0f)) {
         cfs_status st = check_cuda(cudaMemsetAsync(a_max, 0, sizeof(float) * (size_t)n_layers,
                                                    stream), "cudaMemsetAsync(a_max)");
