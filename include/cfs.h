@@ -352,8 +352,10 @@ cfs_status cfs_batch_windows(cfs_batch* batch, int32_t* out);
  * four fields shape the compiled program; chunk is the default work-item
  * size of every frame.  cfs_batch_create starts from the measured default
  * plan (ilp 2, window on when the chain splats once into a histogram, 53248
- * words, warp aggregation off, 4096 points per item); a batch as created whose
- * items of 4096 points would leave CTAs without work has smaller ones. */
+ * words, warp aggregation off, 4096 points per item); the items of a batch as
+ * created are of its own sizes instead, up to 65536 points in large batches
+ * and fewer towards the end, below 4096 where those would leave CTAs without
+ * work. */
 typedef struct {
     int ilp;                /* trajectories stepped together per thread: 1 or 2 */
     int window;             /* privatized shared-memory window for the chain's histogram
@@ -381,7 +383,8 @@ cfs_status cfs_batch_set_plan(cfs_batch* batch, const cfs_batch_plan* plan);
  *     to even: 2^16-2^17, 2^18-2^19, ...) and target size (width x height of
  *     target 0) -- the item size and whether the frame uses the window, timed
  *     on that class's frames alone; the classes' choices are then kept only
- *     if the whole batch runs faster with them than under stage 1's plan
+ *     if the whole batch runs faster with them than under stage 1's plan,
+ *     and the sizes of the batch as created if it runs faster still with those
  *     (batches of more than 32 classes skip this stage).
  * The choices are kept in the library's tuning cache under keys made of the
  * device (name, SM count), the program's structure and the classes; a later
