@@ -10,10 +10,9 @@
 //
 // Network: u (64) -> 128 -> 128 -> 128 -> 2, SiLU after the first three
 // layers; BF16 weights and activations, FP32 accumulation on the tensor
-// cores, FP32 master weights and Adam state.  Training runs its GEMMs on the
-// fifth-generation tensor cores (tcgen05.mma, accumulators in tensor
-// memory); the fused inference kernel keeps its small per-point products in
-// registers (mma.sync m16n8k16 bf16).
+// cores, FP32 master weights and Adam state.  Training and inference run their
+// products on the fifth-generation tensor cores (tcgen05.mma, accumulators in
+// tensor memory).
 //
 // Parameter vector (FP32, this order): W1 [128][64], b1 [128], W2 [128][128],
 // b2, W3 [128][128], b3, W4 [2][128], b4 [2] -- 41602 floats.
@@ -80,11 +79,10 @@ __device__ __forceinline__ float silu_grad_f(float z)
 // CTA tile: 128 rows x the whole width N (64 or 128).  K runs in chunks of
 // 64, staged by the CTA's 128 threads into shared memory in the no-swizzle
 // K-major layout of 8-row x 16-byte core matrices (K-adjacent cores 128 B
-// apart, 8-row groups 1024 B apart).  Two stages: while the tensor core
-// multiplies chunk c, the threads stage chunk c + 1.  Thread 0 issues the
-// four tcgen05.mma of a chunk (M = 128, N, K = 16 each) and commits them to
-// the stage's mbarrier; the stage is refilled only after that barrier
-// completes.  The epilogue reads the accumulator with tcgen05.ld: warp w
+// apart, 8-row groups 1024 B apart).  Thread 0 issues the four tcgen05.mma of
+// a chunk (M = 128, N, K = 16 each) and commits them to an mbarrier; the chunk's
+// place is refilled only after that barrier completes.  It serves batches of
+// fewer than 128 rows: K is at most 128, two chunks.  The epilogue reads the accumulator with tcgen05.ld: warp w
 // owns TMEM lanes 32w..32w+31, so every thread holds one output row.
 // Every wait is bounded: on a time-out the CTA records it in g_tc_error,
 // skips its epilogue, frees its TMEM and returns.
@@ -94,28 +92,18 @@ enum Epi { EPI_SILU = 1, EPI_SILU_GRAD = 2, EPI_ATOMIC = 3 };
 constexpr int TC_M = 128, TC_K = 64, TC_THREADS = 256;
 constexpr int TC_NV = 128 * 8 / TC_THREADS;   // 16-byte vectors per thread per operand tile
 constexpr int TC_TILE_BYTES = 128 * TC_K * 2;             // 16 KB: 128 rows x 64 K
-// dynamic shared memory of the kernel with ST stages of (A, B) chunks, plus
-// barriers and alignment; one stage is padded to 50 KB so that at most four
-// CTAs share an SM (four times 128 TMEM columns fill its 512)
-template <int ST>
-constexpr int tc_smem_bytes()
-{
-    return ST == 1 ? 50 * 1024 : 2 * ST * TC_TILE_BYTES + 1024 + 1024;
-}
+// dynamic shared memory: a chunk of A and B, barrier and alignment, padded so that
+// at most four CTAs share an SM (four times 128 TMEM columns fill its 512)
+constexpr int TC_SMEM = 50 * 1024;
 constexpr u32 TC_WAIT_LIMIT = 1u << 24;
 constexpr int TC_COPIES = 16;   // copies of the bias-gradient sums (spread the atomics)
 
 __device__ unsigned int g_tc_error = 0;
-// chunk stages of the register-staged GEMM kernel: by the chunks a CTA runs
-// (one stage for at most two: four CTAs per SM then take all row tiles of a
-// GEMM in one wave; two stages for K-split weight gradients, whose CTAs run
-// four chunks).
 
 struct TcArgs {
     int M, N, K;                 // N in {64, 128}
     const bf16r* A; int lda;     // [M][lda], K contiguous
     const bf16r* B; int ldb;     // [N][ldb], K contiguous
-    int k_split;                 // K per blockIdx.z, a multiple of TC_K
     int mode;
     const float* bias;           // SILU: [N]
     float* C; int ldc;           // SILU: pre-activation Z out; ATOMIC: C += D
@@ -398,26 +386,20 @@ __device__ __forceinline__ void tc_epilogue(const TcArgs& g, int row, int c0, co
     }
 }
 
-template <int ST>
 __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_constant__ TcArgs g)
 {
     extern __shared__ unsigned char tc_smem_raw[];
     unsigned char* sm = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(tc_smem_raw) + 1023) & ~(uintptr_t)1023);
-    // stage s: A at sm + 2 s TILE, B right after it
-    u64* bars = reinterpret_cast<u64*>(sm + 2 * ST * TC_TILE_BYTES);
-    u32* s_tmem = reinterpret_cast<u32*>(sm + 2 * ST * TC_TILE_BYTES + 64);
-    float* s_col = reinterpret_cast<float*>(sm + 2 * ST * TC_TILE_BYTES + 128);   // [128]
+    // A at sm, B right after it
+    const u32 sA = smem_addr(sm), sB = sA + TC_TILE_BYTES;
+    const u32 bar = smem_addr(sm + 2 * TC_TILE_BYTES);
+    u32* s_tmem = reinterpret_cast<u32*>(sm + 2 * TC_TILE_BYTES + 64);
+    float* s_col = reinterpret_cast<float*>(sm + 2 * TC_TILE_BYTES + 128);   // [128]
     const int tid = threadIdx.x, warp = tid >> 5;
     const int m0 = blockIdx.x * TC_M;
-    const int kb = blockIdx.z * g.k_split;
-    const int ke = min(g.K, kb + g.k_split);
-    const int n_chunks = ke > kb ? (ke - kb + TC_K - 1) / TC_K : 0;
+    const int n_chunks = (g.K + TC_K - 1) / TC_K;
     const u32 ncols = g.N <= 64 ? 64u : 128u;
-    // stage s's barrier completes once per chunk c = s, s + ST, ...: chunk c
-    // is its (c / ST)-th phase
-    auto bar = [&](int c) { return smem_addr(&bars[c % ST]); };
-    auto phase = [](int c) { return (u32)(c / ST) & 1u; };
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -428,8 +410,7 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
     }
     if (tid < 128) s_col[tid] = 0.0f;
     if (tid == 0) {
-#pragma unroll
-        for (int q = 0; q < ST; ++q) mbar_init(smem_addr(&bars[q]), 1u);
+        mbar_init(bar, 1u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     tc_fence_before();
@@ -440,16 +421,15 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
 
     bool ok = true;
     for (int c = 0; c < n_chunks; ++c) {
-        const int s = c % ST;
-        // the stage's previous chunk (c - ST) must have left the tensor core
-        if (c >= ST) ok = mbar_wait(bar(c - ST), phase(c - ST));
+        // (the barrier completes once per chunk: the previous one must have left
+        // the tensor core)
+        if (c > 0) ok = mbar_wait(bar, (u32)(c - 1) & 1u);
         if (!__syncthreads_and(ok)) { ok = false; break; }
-        const int k0 = kb + c * TC_K;
-        const u32 sA = smem_addr(sm + 2 * s * TC_TILE_BYTES), sB = sA + TC_TILE_BYTES;
+        const int k0 = c * TC_K;
         {
             uint4 va[TC_NV], vb[TC_NV];
-            tc_stage_load(va, g.A, g.lda, g.M, m0, TC_M, k0, ke);
-            tc_stage_load(vb, g.B, g.ldb, g.N, 0, g.N, k0, ke);
+            tc_stage_load(va, g.A, g.lda, g.M, m0, TC_M, k0, g.K);
+            tc_stage_load(vb, g.B, g.ldb, g.N, 0, g.N, k0, g.K);
             tc_stage_store(sA, va, TC_M);
             tc_stage_store(sB, vb, g.N);
         }
@@ -462,7 +442,7 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
             for (int kk = 0; kk < TC_K / 16; ++kk)
                 tc_mma(tmem, tc_desc(sA + kk * 256), tc_desc(sB + kk * 256), idesc,
                        (c > 0 || kk > 0) ? 1u : 0u);
-            tc_commit(bar(c));
+            tc_commit(bar);
         }
     }
     // epilogue split: warp w reads TMEM lanes 32 (w % 4) .. + 31 (its rows)
@@ -472,10 +452,7 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
     const int c_begin = half * (g.N / 2), c_end = c_begin + g.N / 2;
     float z_next[16];
     tc_load_z(g, row, c_begin, z_next);   // independent of the MMAs: overlaps them
-    if (ok && n_chunks > 0) {
-        const int last = n_chunks - 1;
-        ok = mbar_wait(bar(last), phase(last));
-    }
+    if (ok && n_chunks > 0) ok = mbar_wait(bar, (u32)(n_chunks - 1) & 1u);
     ok = __syncthreads_and(ok) != 0;
     tc_fence_after();
     if (ok && n_chunks > 0) {
@@ -492,10 +469,7 @@ __global__ void __launch_bounds__(TC_THREADS) tc_gemm_kernel(const __grid_consta
     } else if (!ok && tid == 0) {
         atomicOr(&g_tc_error, (unsigned)CFS_DEVICE_ERR_TC_TIMEOUT);
         // give in-flight MMAs a bounded chance to drain before TMEM is freed
-        if (n_chunks > 0) {
-            const int last = n_chunks - 1;
-            mbar_wait(bar(last), phase(last));
-        }
+        if (n_chunks > 0) mbar_wait(bar, (u32)(n_chunks - 1) & 1u);
     }
     tc_fence_before();
     __syncthreads();
@@ -2369,11 +2343,10 @@ cfs_status ensure_rows(cfs_sampler* s, int B)
     return CFS_OK;
 }
 
-// D = A B^T on the tensor cores (both operands K-major), split over K into
-// `splits` CTA ranges (ATOMIC adds the partial products)
+// D = A B^T on the tensor cores (both operands K-major; ATOMIC adds it to C)
 cfs_status tc_gemm(cudaStream_t st, int M, int N, int K, const bf16r* A, int lda, const bf16r* B,
              int ldb, int mode, const float* bias, float* C, int ldc, bf16r* H, int ldh,
-             bf16r* HT, int ldt, const float* Zin, int ldz, float* colsum, int splits = 1)
+             bf16r* HT, int ldt, const float* Zin, int ldz, float* colsum)
 {
     // the staging reads 16-byte vectors, the epilogue writes them: every
     // operand and output of this library is laid out for that; anything
@@ -2389,16 +2362,9 @@ cfs_status tc_gemm(cudaStream_t st, int M, int N, int K, const bf16r* A, int lda
     g.M = M; g.N = N; g.K = K;
     g.A = A; g.lda = lda;
     g.B = B; g.ldb = ldb;
-    const int per = (K + splits - 1) / splits;
-    g.k_split = (per + TC_K - 1) / TC_K * TC_K;
     g.mode = mode; g.bias = bias; g.C = C; g.ldc = ldc; g.H = H; g.ldh = ldh;
     g.HT = HT; g.ldt = ldt; g.Zin = Zin; g.ldz = ldz; g.colsum = colsum;
-    dim3 grid((M + TC_M - 1) / TC_M, 1, (K + g.k_split - 1) / g.k_split);
-    const int stages = g.k_split / TC_K <= 2 ? 1 : 2;
-    if (stages == 1)
-        tc_gemm_kernel<1><<<grid, TC_THREADS, tc_smem_bytes<1>(), st>>>(g);
-    else
-        tc_gemm_kernel<2><<<grid, TC_THREADS, tc_smem_bytes<2>(), st>>>(g);
+    tc_gemm_kernel<<<(M + TC_M - 1) / TC_M, TC_THREADS, TC_SMEM, st>>>(g);
     return CFS_OK;
 }
 
@@ -2691,14 +2657,8 @@ cfs_status cfs_sampler_create(const float* params, uint64_t seed, cfs_sampler** 
     s->bias_part = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(s->w) + off_part);
     // the tensor-core GEMM stages its chunk pairs in dynamic shared memory
     if (st == CFS_OK)
-        st = check_cuda(cudaFuncSetAttribute(tc_gemm_kernel<1>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             tc_smem_bytes<1>()),
-                        "cudaFuncSetAttribute(tc_gemm_kernel)");
-    if (st == CFS_OK)
-        st = check_cuda(cudaFuncSetAttribute(tc_gemm_kernel<2>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             tc_smem_bytes<2>()),
+        st = check_cuda(cudaFuncSetAttribute(tc_gemm_kernel,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM),
                         "cudaFuncSetAttribute(tc_gemm_kernel)");
     if (st == CFS_OK)
         st = check_cuda(cudaFuncSetAttribute(back_rows_kernel,
