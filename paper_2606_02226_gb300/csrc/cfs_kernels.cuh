@@ -578,10 +578,8 @@ cfs_bbox_kernel(const __grid_constant__ cfs_launch_args a)
 /* The batched renderer (many frames of different systems, one launch): a
  * persistent grid whose CTAs take work items -- a chunk of one frame's
  * points -- from a global counter (one atomicAdd per item; no CTA ever waits
- * for another).  Items are numbered frame by frame and every frame has at
- * least as many items as the grid has CTAs (small frames get small items),
- * so the whole grid works on one or two frames at a time and their layers
- * stay in L2.  A CTA loads a frame's thresholds, maps, palettes and target
+ * for another).  Items are numbered frame by frame, so the grid works on a
+ * few frames at a time and their layers stay in L2.  A CTA loads a frame's thresholds, maps, palettes and target
  * geometry into shared memory when its next item belongs to another frame.
  * With CFS_TILE the first splat goes to a privatized shared-memory window
  * of the frame's histogram, one per channel, placed by the pre-pass
