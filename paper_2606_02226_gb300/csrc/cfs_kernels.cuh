@@ -702,8 +702,7 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
                 z = CFS_DIM == 3 ? (float)(r.z >> 8) * CFS_INV_2_24 : 0.0f;
             }
         };
-        /* (two copies of the step code: the frames whose buckets all hold at
-         * most one threshold, and the others) */
+        /* (a copy of the step code for each kind of choice) */
         auto run_item = [&](const auto& choose) {
 #if CFS_ILP == 2
             /* two trajectories per thread, stepped in lockstep: their
@@ -729,7 +728,8 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
             }
 #endif
         };
-        if (s_kt.more <= 1) run_item(CfsChooseKtab<false>{s_kt, 1});
+        if (s_kt.more5 <= 1) run_item(CfsChooseOne{s_kt});
+        else if (s_kt.more <= 1) run_item(CfsChooseKtab<false>{s_kt, 1});
         else run_item(CfsChooseKtab<true>{s_kt, s_kt.more});
         __syncthreads();
     }

@@ -8,21 +8,36 @@
 #define CFS_WINDOW_CUH
 
 /* ---- map choice of a frame ------------------------------------------------
- * k = #{ j < n_cmp : w >= T_j } through a bucket table: the top 7 bits of the
- * word pick one of 128 buckets (128 bytes: every bank holds one word of them,
- * so a warp's lookups never conflict), whose entry is 16 times the count at
- * the bucket's start; the word is then compared with the thresholds the
- * bucket may hold.  `more` is the largest number of thresholds in one bucket
- * (1 for most systems), the same for the whole frame; the loop for more of
- * them, compiled into a copy of its own, cost 5% of the animation's time when
- * every step tested for it.  A finer table with a fallback (12 bits, one
- * lookup) took 3.4 shared-memory cycles per warp instead of 2 and a divergent
- * branch. */
+ * k = #{ j < n_cmp : w >= T_j } through a bucket table.  Where no bucket of the
+ * word's top 5 bits holds more than one threshold (`more5`, most systems), one
+ * lookup does: bucket b's entry has the other 27 bits of the threshold's
+ * predecessor, the last word of the bucket that stays, above the count k at
+ * the bucket's start (32 words, one a bank: no conflicts).  That is one
+ * shared-memory cycle a warp instead of two, of 14.7 a step in a kernel that
+ * they bound: 142.0 -> 136.8 ms for the 256 animation frames.
+ * In other frames the top 7 bits of the word pick one of 128 buckets (128
+ * bytes: every bank holds one word of them, so a warp's lookups never
+ * conflict), whose entry is 16 times the count at the bucket's start; the word
+ * is then compared with the thresholds the bucket may hold.  `more` is the
+ * largest number of thresholds in one of these; the loop for more than one,
+ * compiled into a copy of its own, cost 5% of the animation's time when every
+ * step tested for it.  A finer table with a fallback (12 bits, one lookup) took
+ * 3.4 shared-memory cycles per warp instead of 2 and a divergent branch. */
 #define CFS_KTAB_BITS 7
 struct CfsKtab {
     unsigned char k16[1 << CFS_KTAB_BITS];
     u32 last[CFS_A_MAX_MAPS][4];    /* [k][0]: T_k - 1, the last word that stays at k */
-    int more;
+    u32 one[32];                    /* [bucket]: (T_k - 1) << 5 | k */
+    int more, more5;
+};
+
+struct CfsChooseOne {
+    const CfsKtab& t;               /* shared memory */
+    __device__ __forceinline__ int operator()(u32 w) const
+    {
+        const u32 e = t.one[w >> 27];
+        return (int)((e & 31u) + (w << 5 > e ? 1u : 0u));
+    }
 };
 
 template <bool MORE>
@@ -62,7 +77,19 @@ __device__ __forceinline__ void cfs_build_ktab(const u32* T, int n_cmp, CfsKtab&
             more = max(more, k1 - k0);
         }
         more = __reduce_max_sync(0xffffffffu, more);
-        if (threadIdx.x == 0) t.more = more;
+        const u32 w0 = threadIdx.x << 27, w1 = w0 | 0x07FFFFFFu;
+        int k0 = 0, k1 = 0;
+        for (int j = 0; j < n_cmp; ++j) {
+            k0 += w0 >= T[j] ? 1 : 0;
+            k1 += w1 >= T[j] ? 1 : 0;
+        }
+        /* (no threshold: no word passes 27 ones) */
+        t.one[threadIdx.x] = (k1 > k0 ? (T[k0] - 1u) << 5 : 0xFFFFFFE0u) | (u32)k0;
+        const int more5 = __reduce_max_sync(0xffffffffu, k1 - k0);
+        if (threadIdx.x == 0) {
+            t.more = more;
+            t.more5 = more5;
+        }
     }
 }
 
