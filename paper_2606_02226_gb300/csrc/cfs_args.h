@@ -17,7 +17,8 @@ typedef struct {
     int W, H, C, kind;
     float x0, x1, y0, y1;
     float sx, sy;                       /* W / (x1 - x0), H / (y1 - y0) in FP32 */
-    int pad0, pad1;
+    int blind;                          /* stored clouds: depth splats do not read first */
+    int pad1;
     float palette[CFS_A_MAX_MAPS][4];
     unsigned int palette8[CFS_A_MAX_MAPS];
 } cfs_dev_target;

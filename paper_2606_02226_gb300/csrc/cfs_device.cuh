@@ -522,7 +522,8 @@ __device__ __forceinline__ void cfs_splat_rgba(const cfs_dev_target& t, float x,
 /* u64 depth+colour [H][W]: min= (bits(z) << 32) | rgba8.  With
  * CFS_DEPTH_TEST the current value is read first (a strong relaxed load) and
  * the reduction is skipped when it could not lower it: keys only decrease,
- * so a key not below an observed value is not below the final one either. */
+ * so a key not below an observed value is not below the final one either.
+ * (Stored clouds read or not by the target's `blind`.) */
 __device__ __forceinline__ void cfs_splat_depth(const cfs_dev_target& t, float x, float y,
                                                 float z, bool alive, u32 rgba8, u32& disc)
 {
@@ -533,7 +534,9 @@ __device__ __forceinline__ void cfs_splat_depth(const cfs_dev_target& t, float x
         u64* base = reinterpret_cast<u64*>(t.data);
         u64* p = base + ((size_t)iy * (size_t)t.W + (size_t)ix);
         const u64 key = ((u64)__float_as_uint(z) << 32) | (u64)rgba8;
-#if CFS_DEPTH_TEST
+#if CFS_DEPTH_TEST && CFS_POINTS
+        if (t.blind || key < cfs_ld_relaxed_u64(p)) cfs_red_min_u64(p, key);
+#elif CFS_DEPTH_TEST
         if (key < cfs_ld_relaxed_u64(p)) cfs_red_min_u64(p, key);
 #else
         cfs_red_min_u64(p, key);

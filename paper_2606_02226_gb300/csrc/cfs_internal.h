@@ -101,6 +101,7 @@ cfs_status launch(const Kernel& k, unsigned grid, const void* args, size_t args_
                   cudaStream_t stream);
 cfs_status check_cuda(cudaError_t e, const char* what);
 int device_sm_count();
+uint64_t device_l2_bytes();     // of the current device, 0 if unknown
 // 2D tensor map (TMA) of a BF16 matrix [rows][cols], row stride ld elements,
 // box_rows x box_cols boxes, no swizzle, zeros outside (cfs_runtime.cpp)
 cfs_status make_tmap_2d_bf16(CUtensorMap* map, const void* base, uint64_t cols, uint64_t rows,

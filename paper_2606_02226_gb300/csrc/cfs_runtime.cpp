@@ -225,6 +225,14 @@ int device_sm_count()
     return n;
 }
 
+uint64_t device_l2_bytes()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrL2CacheSize, dev) != cudaSuccess) return 0;
+    return n > 0 ? (uint64_t)n : 0;
+}
+
 cfs_status get_kernel(const ProgramSpec& spec, const char* name, Kernel* out)
 {
     Driver& d = driver();
