@@ -166,8 +166,12 @@ __global__ void __launch_bounds__(kBlock) noalloc_place_kernel(const __grid_cons
     __shared__ NaTables tab;
     __shared__ cfs_dev_target tg;
     __shared__ CfsPlace place;
+    __shared__ CfsKtab kt;
     load_tables(a.ws->frames[blockIdx.x], tab, tg);
     __syncthreads();
+    cfs_build_ktab(tab.T, tab.n_cmp, kt);
+    __syncthreads();
+    const CfsChooseKtab<true> choose{kt, kt.more};
     const int C = tg.C;
     cfs_place_windows(tg, C, kCounters, place, s_samples,
                       reinterpret_cast<unsigned char*>(s_samples + CFS_WIN_SAMPLES * blockDim.x),
@@ -186,8 +190,7 @@ __global__ void __launch_bounds__(kBlock) noalloc_place_kernel(const __grid_cons
             uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
 #pragma unroll 1
             for (u32 n = 4u * nb; n < min(n1, 4u * nb + 4u); ++n) {
-                int k = 0;
-                for (int q = 0; q < tab.n_cmp; ++q) k += r.x >= tab.T[q] ? 1 : 0;
+                const int k = choose(r.x);
                 r = make_uint4(r.y, r.z, r.w, 0u);
                 apply_map(tab, k, x, y);
                 if (n < a.burn_in) continue;
