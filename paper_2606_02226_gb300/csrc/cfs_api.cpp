@@ -775,12 +775,16 @@ cfs_status cfs_render_points(const cfs_chain* chain, const float* xyz, const uin
     // larger one makes each point wait for DRAM, and with no more points than
     // pixels few of them lose.  2^26 points into 8192^2 (512 MB, four times the L2):
     // 562 us with the read, 488 without; 2^22: 64 and 46; into 4096^2 (128 MB) 526
-    // and 630; 2^24 into 1024^2 156 and 250.  The line is twice the L2.
+    // and 630; 2^24 into 1024^2 156 and 250.  The line is twice the L2.  With
+    // hardware trigonometry a point's arithmetic is shorter, so that the reductions
+    // themselves bound large clouds, the more so in Morton order, whose reads hit
+    // (2^26 points 339 us with the read, 382 without; 2^24 109 and 113; 2^23 68 and
+    // 66, in generation order 100 and 68): an eighth of the pixels at most there.
     const uint64_t l2 = device_l2_bytes();
     for (int t = 0; t < n_targets; ++t) {
         const uint64_t pixels = (uint64_t)targets[t].width * (uint64_t)targets[t].height;
         a.tg[t].blind = targets[t].kind == CFS_TARGET_DEPTH_U64 && l2 > 0 && 8 * pixels > 2 * l2 &&
-                        n <= pixels;
+                        (uint64_t)n * (sp.fast_trig ? 8 : 1) <= pixels;
     }
     a.cloud_xyz = (unsigned long long)(uintptr_t)xyz;
     a.cloud_fn = (unsigned long long)(uintptr_t)fn;
