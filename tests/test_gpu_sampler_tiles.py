@@ -25,3 +25,29 @@ def test_a_row_does_not_depend_on_its_place(torch_cuda, B, rows):  # noqa: F811
         big, small = torch.zeros((B, 2), device="cuda"), torch.zeros((128, 2), device="cuda")
         big[r] = small[77] = torch.tensor([0.75, -1.25], device="cuda")
         assert np.array_equal(s.backward(Ut, big).cpu().numpy(), s.backward(few, small).cpu().numpy())
+
+
+@pytest.mark.parametrize("B", [100, 4096])
+def test_captured_step_replays_the_same(torch_cuda, B):  # noqa: F811
+    # the backward's kernels start under each other's tails: their order holds in
+    # a graph of the caller's too
+    torch = torch_cuda
+    cfs, s, _, _, Ut = _setup(torch, B)
+    dY = torch.linspace(-1, 1, 2 * B, device="cuda").view(B, 2)
+    Y, g = s.forward(Ut).clone(), s.backward(Ut, dY).clone()
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        graph.capture_begin()
+        Yc = s.forward(Ut, stream=stream)
+        gc = s.backward(Ut, dY, stream=stream)
+        graph.capture_end()
+    for _ in range(3):
+        gc.zero_()
+        Yc.zero_()
+        torch.cuda.synchronize()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(Yc, Y)
+        assert float((gc - g).norm() / g.norm()) < 1e-5
