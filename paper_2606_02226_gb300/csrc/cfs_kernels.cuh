@@ -675,8 +675,10 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
             cur = f;
         }
         const u32 sid = s_sid, pbeg = s_pbeg;
+        /* (no sum of a point number and a size: with almost 2^32 points it would
+         * wrap, and the last item be lost or its loop never end) */
         const u32 j0 = (item - s_ibeg) * s_chunk;
-        const u32 j1 = min(j0 + s_chunk, s_npts);
+        const u32 mine = min(s_chunk, s_npts - j0);
         const float* st = s_start;
         const u32 sc = s_scount;
         const u32 npts = s_npts;
@@ -701,11 +703,11 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
 #if CFS_ILP == 2
             /* two trajectories per thread, stepped in lockstep: their
              * independent dependency chains hide each other's latency */
-            for (u32 j = j0 + threadIdx.x; j < j1; j += 2 * blockDim.x) {
-                const u32 j2 = j + blockDim.x;
+            for (u32 t = threadIdx.x; t < mine; t += 2 * blockDim.x) {
+                const u32 j = j0 + t, j2 = j + blockDim.x;
                 float x, y, z;
                 start_of(j, x, y, z);
-                if (j2 < j1) {
+                if (t + blockDim.x < mine) {
                     float x2, y2, z2;
                     start_of(j2, x2, y2, z2);
                     cfs_run_point2(a, choose, CFS_BATCH_TG, sm, pbeg + j, pbeg + j2, sid, x, y, z, x2, y2,
@@ -715,7 +717,8 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
                 }
             }
 #else
-            for (u32 j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
+            for (u32 t = threadIdx.x; t < mine; t += blockDim.x) {
+                const u32 j = j0 + t;
                 float x, y, z;
                 start_of(j, x, y, z);
                 cfs_run_point(a, choose, CFS_BATCH_TG, sm, pbeg + j, sid, x, y, z, disc, tile);
