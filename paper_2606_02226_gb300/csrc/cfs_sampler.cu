@@ -799,6 +799,8 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
         a0[j] = a1[j] = ab[j] = 0.0f;
     }
     float b40 = 0.0f, b41 = 0.0f;
+    // rows of dY on eight-byte boundaries are read as one word
+    const bool wide = ((uintptr_t)dY & 7u) == 0;
     after_previous();       // (the weights are older)
     for (int e = threadIdx.x; e < 3 * HID + 2; e += OB_THREADS) s_sum[e] = 0.0f;
     // a warp's RUN consecutive rows, four of them in flight
@@ -811,8 +813,10 @@ __global__ void __launch_bounds__(OB_THREADS) out_backward_kernel(const float* _
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const bool in = r + q < B;
-                y[q] = in ? __ldg(reinterpret_cast<const float2*>(dY) + r + q)
-                          : make_float2(0.0f, 0.0f);
+                const float* p = dY + 2 * (size_t)(r + q);
+                y[q] = !in ? make_float2(0.0f, 0.0f)
+                           : (wide ? __ldg(reinterpret_cast<const float2*>(p))
+                                   : make_float2(__ldg(p), __ldg(p + 1)));
                 z[q] = in ? __ldcs(reinterpret_cast<const float4*>(Z3 + (size_t)(r + q) * HID + c))
                           : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             }
