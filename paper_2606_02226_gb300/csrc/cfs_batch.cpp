@@ -939,12 +939,12 @@ cfs_status cfs_batch_tune(cfs_batch* b, uint32_t trial_iters, uint32_t flags, vo
     // (only for a batch of at most kMaxTunedClasses classes: each class costs
     // up to eight trials)
     int n_win = b->spec.tile ? (int)counts.size() : 0;
-    bool use_classes = false;
-    if (st == CFS_OK && (int)counts.size() <= kMaxTunedClasses) {
+    cfs_batch_plan prog = b->plan;
+    prog.chunk = 0;                     // the program's knobs only
+    const std::string pkey = format_plan(prog);
+    const bool by_class = (int)counts.size() <= kMaxTunedClasses;
+    if (st == CFS_OK && by_class) {
         n_win = 0;
-        cfs_batch_plan prog = b->plan;
-        prog.chunk = 0;                 // the program's knobs only
-        const std::string pkey = format_plan(prog);
         std::vector<uint8_t> active(b->n_frames);
         for (const auto& kv : counts) {
             if (st != CFS_OK) break;
@@ -974,41 +974,46 @@ cfs_status cfs_batch_tune(cfs_batch* b, uint32_t trial_iters, uint32_t flags, vo
                 if (cls[f] == kv.first) { b->chunks[f] = c_best; b->nowin[f] = nw_best; }
             if (!nw_best && b->spec.tile) ++n_win;
         }
-        // a class timed alone is not the class inside the batch (frames of
-        // other classes share the CTAs and the L2): the classes' choices are
-        // kept only when the whole batch runs faster with them than with the
-        // program's plan alone ("1" in the cache, "0" if not); and both give
-        // way to the sizes of the batch as created if it runs faster with
-        // those ("2")
-        if (st == CFS_OK) {
-            const std::string ukey = "classes|" + devkey + "|" + skey + "|" + pkey + "|" +
-                                     mix.str();
-            std::string v;
-            bool use_created = false;
-            if (!retune && cache_get(ukey, &v) && (v == "0" || v == "1" || v == "2")) {
-                use_classes = v == "1";
-                use_created = v == "2";
-            } else {
-                all_cached = false;
-                const std::vector<uint32_t> ch = b->chunks;
-                const std::vector<uint8_t> nw = b->nowin;
-                float with_ms = 0.0f, without_ms = 0.0f, created_ms = 0.0f;
-                st = trial(nullptr, &with_ms);
-                set_all(b->plan.chunk, 0);
-                if (st == CFS_OK) st = trial(nullptr, &without_ms);
-                b->chunks = b->created;
-                if (st == CFS_OK) st = trial(nullptr, &created_ms);
-                use_created = created_ms < std::min(with_ms, without_ms);
-                use_classes = !use_created && with_ms < without_ms;
-                b->chunks = ch;
-                b->nowin = nw;
-                if (st == CFS_OK) cache_put(ukey, use_created ? "2" : (use_classes ? "1" : "0"));
-            }
-            if (!use_classes) {
-                set_all(b->plan.chunk, 0);
-                if (use_created) b->chunks = b->created;
-                n_win = b->spec.tile ? (int)counts.size() : 0;
-            }
+    }
+
+    // ---- the item sizes, on the whole batch -------------------------------
+    // A class timed alone is not the class inside the batch (frames of other
+    // classes share the CTAs and the L2): the classes' choices are kept only
+    // when the whole batch runs faster with them than with the program's plan
+    // alone ("1" in the cache, "0" if not); and both give way to the sizes of
+    // the batch as created if it runs faster with those ("2"), which a batch of
+    // any number of classes tries: uniform sizes lose to them in large batches
+    // (256 animation frames: 159 ms with items of 4096 points, 146 of 32768, 142
+    // as created).  (Entries under the older prefix "classes|" were made without
+    // that trial and are not read.)
+    bool use_classes = false;
+    if (st == CFS_OK) {
+        const std::string ukey = "sizes|" + devkey + "|" + skey + "|" + pkey + "|" + mix.str();
+        std::string v;
+        bool use_created = false;
+        if (!retune && cache_get(ukey, &v) && (v == "0" || (v == "1" && by_class) || v == "2")) {
+            use_classes = v == "1";
+            use_created = v == "2";
+        } else {
+            all_cached = false;
+            const std::vector<uint32_t> ch = b->chunks;
+            const std::vector<uint8_t> nw = b->nowin;
+            float with_ms = 1e30f, without_ms = 0.0f, created_ms = 0.0f;
+            if (by_class) st = trial(nullptr, &with_ms);
+            set_all(b->plan.chunk, 0);
+            if (st == CFS_OK) st = trial(nullptr, &without_ms);
+            b->chunks = b->created;
+            if (st == CFS_OK) st = trial(nullptr, &created_ms);
+            use_created = created_ms < std::min(with_ms, without_ms);
+            use_classes = !use_created && with_ms < without_ms;
+            b->chunks = ch;
+            b->nowin = nw;
+            if (st == CFS_OK) cache_put(ukey, use_created ? "2" : (use_classes ? "1" : "0"));
+        }
+        if (!use_classes) {
+            set_all(b->plan.chunk, 0);
+            if (use_created) b->chunks = b->created;
+            n_win = b->spec.tile ? (int)counts.size() : 0;
         }
     }
 
