@@ -339,6 +339,23 @@ _PALETTE_AT = cfs_target.palette.offset
 _PALETTE8_AT = cfs_target.palette8.offset
 
 
+def _palette_bytes(entries, dtype, ndim: int) -> bytes:
+    """The first MAX_MAPS rows of a palette (four columns where it has two
+    dimensions), in the layout of cfs_target; never longer than its field."""
+    p = np.asarray(entries, dtype=dtype)
+    if p.ndim < ndim:
+        if p.shape == (0,):
+            return b""
+        raise IndexError(f"a palette of this kind has {ndim} dimension(s)")
+    if p.shape[0] == 0:
+        return b""
+    if p.ndim > ndim:
+        raise TypeError(f"a palette of this kind has {ndim} dimension(s)")
+    if ndim == 2 and p.shape[1] < 4:
+        raise IndexError("a palette has four columns")
+    return p[:MAX_MAPS].tobytes() if ndim == 1 else p[:MAX_MAPS, :4].tobytes()
+
+
 def make_targets(descs, tensors=None, fake_ptr: bool = False):
     n = len(descs)
     if n > MAX_TARGETS:
@@ -364,17 +381,11 @@ def make_targets(descs, tensors=None, fake_ptr: bool = False):
         # 15 us of every call (17.5 us to describe one target, 3 us this way)
         palette = getattr(d, "palette", None)
         if palette is not None:
-            p = np.asarray(palette, dtype=np.float32)[:MAX_MAPS, :4]
-            if p.shape[1] != 4:
-                raise IndexError("a palette has four columns")
-            raw = p.tobytes()
+            raw = _palette_bytes(palette, np.float32, 2)
             ctypes.memmove(ctypes.addressof(t) + _PALETTE_AT, raw, len(raw))
         palette8 = getattr(d, "palette8", None)
         if palette8 is not None:
-            p8 = np.asarray(palette8, dtype=np.uint32)
-            if p8.ndim != 1:
-                raise TypeError("a packed palette has one dimension")
-            raw = p8[:MAX_MAPS].tobytes()
+            raw = _palette_bytes(palette8, np.uint32, 1)
             ctypes.memmove(ctypes.addressof(t) + _PALETTE8_AT, raw, len(raw))
     return arr, n
 
