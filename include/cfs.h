@@ -351,16 +351,16 @@ cfs_status cfs_batch_windows(cfs_batch* batch, int32_t* out);
  * tile size and atomic strategy, work-item size).  The first
  * four fields shape the compiled program; chunk is the default work-item
  * size of every frame.  cfs_batch_create starts from the measured default
- * plan (ilp 2, window on when the chain splats once into a histogram, 53248
- * words, warp aggregation off, 4096 points per item); the items of a batch as
- * created are of its own sizes instead, up to 65536 points in large batches
- * and fewer towards the end, below 4096 where those would leave CTAs without
- * work. */
+ * plan (ilp 2, window on when the chain splats once, into a histogram that is
+ * target 0, 53248 words, warp aggregation off, 4096 points per item); the
+ * items of a batch as created are of its own sizes instead, up to 65536 points
+ * in large batches and fewer towards the end, below 4096 where those would
+ * leave CTAs without work. */
 typedef struct {
     int ilp;                /* trajectories stepped together per thread: 1 or 2 */
     int window;             /* privatized shared-memory window for the chain's histogram
                                splat: 0 off, 1 on (ignored unless the chain splats once,
-                               into a histogram, and is not a scribble) */
+                               into a histogram that is target 0, and is not a scribble) */
     uint32_t window_words;  /* window capacity in u32 counters: 1024..53248, multiple of 256;
                                the histogram's channels share them in proportion to their
                                sampled splats, one window (pixel box) per channel */

@@ -170,6 +170,15 @@ cfs_status capture(cfs_batch* b, int clear)
 }  // namespace
 
 namespace cfs {
+// Whether the program can have a privatized window: its chain splats once, into
+// a histogram that is target 0.  (The kernel keeps the bin values and the boxes
+// of that target alone; a splat into another one reads past them.)
+static bool window_allowed(const ProgramSpec& sp)
+{
+    return sp.scribble.empty() && sp.splats.size() == 1 && sp.splats[0].slot == 0 &&
+           sp.splats[0].kind == CFS_TARGET_HIST_U32;
+}
+
 // Launch shape of the persistent batch program (also used by the compile-only
 // check): the default plan's program knobs; returns the privatized window's
 // capacity in u32 counters (0 when the chain cannot use one).
@@ -182,9 +191,7 @@ uint32_t batch_spec_defaults(ProgramSpec& sp)
     sp.min_blocks = 2;
     sp.spill_allowance = 64;
     sp.depth_test = 1;
-    // privatized window: when the chain splats once, into a histogram
-    sp.tile = (sp.splats.size() == 1 && sp.splats[0].kind == CFS_TARGET_HIST_U32 &&
-               sp.scribble.empty()) ? 1 : 0;
+    sp.tile = window_allowed(sp) ? 1 : 0;
     // warp-level aggregation of equal window addresses (match.any) measured
     // slower than plain shared atomics on the animation batch: off
     sp.warp_agg = 0;
@@ -276,12 +283,6 @@ cfs_status plan_items(cfs_batch* b, const std::vector<uint8_t>* active = nullptr
 // dynamic shared memory of the window pre-pass: 1024 threads' 32 samples of 5
 // bytes (CFS_WIN_SMEM in cfs_window.cuh)
 constexpr int kWindowSampleBytes = 1024 * 32 * 5;
-
-bool window_allowed(const ProgramSpec& sp)
-{
-    return sp.scribble.empty() && sp.splats.size() == 1 &&
-           sp.splats[0].kind == CFS_TARGET_HIST_U32;
-}
 
 cfs_status check_plan(const cfs_batch_plan& p)
 {
