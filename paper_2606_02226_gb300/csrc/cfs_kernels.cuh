@@ -300,7 +300,9 @@ cfs_cloud_kernel(const __grid_constant__ cfs_launch_args a)
     const u32 n_pts = a.n_points, sid = a.system_id;
     const u32 stride = gridDim.x * blockDim.x;
     auto run = [&](const auto& choose) {
-        for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < n_pts; j += stride) {
+        /* (a step of at most what is left: with almost 2^32 points j + stride
+         * would wrap and the loop start again) */
+        for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < n_pts; j += min(stride, n_pts - j)) {
             const u32 i = a.point_begin + j;
             float x, y, z;
             cfs_start(a, i, sid, j, n_pts, x, y, z);
@@ -418,7 +420,9 @@ cfs_render_kernel(const __grid_constant__ cfs_launch_args a)
     for (int t = 0; t < CFS_NT_ARR; ++t) disc[t] = 0;
     const CfsChooseConst choose{a};
     const u32 stride = gridDim.x * blockDim.x;
-    for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < a.n_points; j += stride) {
+    /* (a step of at most what is left, as in cfs_cloud_kernel) */
+    for (u32 j = blockIdx.x * blockDim.x + threadIdx.x; j < a.n_points;
+         j += min(stride, a.n_points - j)) {
         const u32 i = a.point_begin + j;
         float x, y, z;
         cfs_start(a, i, a.system_id, j, a.n_points, x, y, z);
