@@ -12,6 +12,12 @@
 #define CFS_A_MAX_TARGETS 4
 #define CFS_A_OP_PARAMS 16
 
+/* window pre-pass: threads of its CTA at most, samples of each, and the dynamic
+ * shared bytes that hold them (a 32-bit pixel position and a channel byte) */
+#define CFS_WIN_THREADS 1024
+#define CFS_WIN_SAMPLES 32
+#define CFS_WIN_SMEM (CFS_WIN_THREADS * CFS_WIN_SAMPLES * 5)
+
 typedef struct {
     unsigned long long data;            /* device pointer */
     int W, H, C, kind;

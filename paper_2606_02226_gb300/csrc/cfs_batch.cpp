@@ -280,10 +280,6 @@ cfs_status plan_items(cfs_batch* b, const std::vector<uint8_t>* active = nullptr
     return CFS_OK;
 }
 
-// dynamic shared memory of the window pre-pass: 1024 threads' 32 samples of 5
-// bytes (CFS_WIN_SMEM in cfs_window.cuh)
-constexpr int kWindowSampleBytes = 1024 * 32 * 5;
-
 cfs_status check_plan(const cfs_batch_plan& p)
 {
     if (p.ilp != 1 && p.ilp != 2) return fail(CFS_ERR_INVALID_ARG, "plan: ilp must be 1 or 2");
@@ -322,7 +318,7 @@ cfs_status build_program(cfs_batch* b)
     if (st != CFS_OK) return st;
     if (b->spec.tile) {
         ProgramSpec bs = b->spec;
-        bs.dyn_smem = kWindowSampleBytes;
+        bs.dyn_smem = CFS_WIN_SMEM;
         st = get_kernel(bs, "cfs_bbox_kernel", &b->bbox_kernel);
     }
     b->args.tile_cap = b->tile_cap;

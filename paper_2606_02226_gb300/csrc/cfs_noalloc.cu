@@ -310,7 +310,9 @@ __global__ void __launch_bounds__(kBlock, 1) noalloc_batch_kernel(const __grid_c
                 }
             }
         };
-        // (two copies of the step code, as in the generated batch kernel)
+        // (a copy of the step code for each choice; the generated batch kernel's
+        // third, one lookup, took 242 us here as without it: the table's part for
+        // it is built and not read)
         if (kt.more <= 1) run_item(CfsChooseKtab<false>{kt, 1});
         else run_item(CfsChooseKtab<true>{kt, kt.more});
         __syncthreads();

@@ -246,9 +246,6 @@ __device__ __forceinline__ void cfs_flush_tile(const F& t, u32* cnt, const int4*
  * the 256-frame animation and most of a batch of a few small frames. */
 #define CFS_WG 64                        /* coarse density grid: CFS_WG x CFS_WG cells */
 #define CFS_WIN_SHAPES 5                 /* window aspect ratios 1/4, 1/2, 1, 2, 4 */
-#define CFS_WIN_SAMPLES 32
-#define CFS_WIN_THREADS 1024
-#define CFS_WIN_SMEM (CFS_WIN_THREADS * CFS_WIN_SAMPLES * 5)   /* dynamic shared bytes */
 
 #define CFS_WGP (CFS_WG + 1)             /* row pitch of the grid: a column's cells in 32 banks */
 struct CfsPlace {
