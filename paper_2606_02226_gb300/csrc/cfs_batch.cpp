@@ -224,13 +224,16 @@ namespace {
 // Points per item of each frame of a batch as created.  A CTA that leaves a
 // frame flushes its windows, up to 53248 reductions, so the fewer CTAs a frame
 // is dealt to the better; but the last items should be small, or CTAs wait for
-// them.  So an item is a quarter of an equal share of the points from its frame
-// on, at most 65536 and never below default_item_points, in whole rounds of
-// 1024 threads with two trajectories each.  Measured on GB300 (300 steps): the
-// 256-frame animation 142.0 ms against 159.1 with items of 4096 throughout,
-// 151.2 of 16384 and 145.9 of 32768; 48 of its frames 27.3 against 29.4, 12 of
-// them 6.25 against 6.33.  A half instead of a quarter: 141.8 ms, but 5 frames
-// 3.11 ms against 2.66; an eighth 142.7 ms.
+// them.  So an item is a quarter of an equal share of the points that follow its
+// frame, at most 65536 and never below default_item_points, in whole rounds of
+// 1024 threads with two trajectories each.  (The frame's own points don't count:
+// nothing smaller fills the last round of the last frame's items, and one frame
+// of 2^22 points took 3.62 ms with them against 3.44, 2^23 7.13 and 6.72, four
+// of 2^22 11.4 and 11.2.)  Measured on GB300 (300 steps): the 256-frame
+// animation 142 ms against 159 with items of 4096 throughout, 151 of 16384 and
+// 146 of 32768 (136.7 with the later one-lookup choice).  A half instead of a
+// quarter, with the frame's own points: 141.8 ms, but 5 frames 3.11 ms against
+// 2.66; an eighth 142.7 ms.
 void created_items(cfs_batch* b)
 {
     const uint32_t grid =
@@ -240,9 +243,9 @@ void created_items(cfs_batch* b)
     const uint32_t least = cfs::default_item_points(points, grid);
     b->created.clear();
     for (const cfs_frame& fr : b->frames) {
+        points -= fr.n_points;
         const uint64_t share = std::min<uint64_t>(65536, points / (4ull * grid) / 2048 * 2048);
         b->created.push_back(std::max(least, (uint32_t)share));
-        points -= fr.n_points;
     }
     b->chunks = b->created;
 }
