@@ -339,21 +339,17 @@ _PALETTE_AT = cfs_target.palette.offset
 _PALETTE8_AT = cfs_target.palette8.offset
 
 
-def _palette_bytes(entries, dtype, ndim: int) -> bytes:
-    """The first MAX_MAPS rows of a palette (four columns where it has two
-    dimensions), in the layout of cfs_target; never longer than its field."""
-    p = np.asarray(entries, dtype=dtype)
-    if p.ndim < ndim:
-        if p.shape == (0,):
-            return b""
-        raise IndexError(f"a palette of this kind has {ndim} dimension(s)")
-    if p.shape[0] == 0:
-        return b""
-    if p.ndim > ndim:
-        raise TypeError(f"a palette of this kind has {ndim} dimension(s)")
+def _odd_palette(p, ndim: int):
+    """A palette of another shape than [<= MAX_MAPS] (x 4): its first rows and
+    columns, an empty one, or an error."""
+    if p.ndim > 0 and p.shape[0] == 0:
+        return p[:0]
+    if p.ndim != ndim:
+        raise (IndexError if p.ndim < ndim else TypeError)(
+            f"a palette of this kind has {ndim} dimension(s)")
     if ndim == 2 and p.shape[1] < 4:
         raise IndexError("a palette has four columns")
-    return p[:MAX_MAPS].tobytes() if ndim == 1 else p[:MAX_MAPS, :4].tobytes()
+    return p[:MAX_MAPS] if ndim == 1 else p[:MAX_MAPS, :4]
 
 
 def make_targets(descs, tensors=None, fake_ptr: bool = False):
@@ -378,14 +374,23 @@ def make_targets(descs, tensors=None, fake_ptr: bool = False):
                 raise ValueError(f"target {j}: shape {tuple(tt.shape)} != {shape}")
             t.data = tt.data_ptr()
         # palettes go over as one block each: element by element they were
-        # 15 us of every call (17.5 us to describe one target, 3 us this way)
+        # 15 us of every call (17.5 us to describe one target, 3 us this way).
+        # A block is never longer than its field
         palette = getattr(d, "palette", None)
         if palette is not None:
-            raw = _palette_bytes(palette, np.float32, 2)
+            p = np.asarray(palette, dtype=np.float32)
+            shape = p.shape
+            if len(shape) != 2 or shape[1] != 4 or not 0 < shape[0] <= MAX_MAPS:
+                p = _odd_palette(p, 2)
+            raw = p.tobytes()
             ctypes.memmove(ctypes.addressof(t) + _PALETTE_AT, raw, len(raw))
         palette8 = getattr(d, "palette8", None)
         if palette8 is not None:
-            raw = _palette_bytes(palette8, np.uint32, 1)
+            p8 = np.asarray(palette8, dtype=np.uint32)
+            shape = p8.shape
+            if len(shape) != 1 or not 0 < shape[0] <= MAX_MAPS:
+                p8 = _odd_palette(p8, 1)
+            raw = p8.tobytes()
             ctypes.memmove(ctypes.addressof(t) + _PALETTE8_AT, raw, len(raw))
     return arr, n
 
