@@ -318,13 +318,13 @@ cfs_cloud_kernel(const __grid_constant__ cfs_launch_args a)
                 cfs_gen_map(a, choose(r.z), x, y, z, sm);
                 cfs_gen_map(a, k = choose(r.w), x, y, z, sm);
             }
-            if (a.iters & 3u) {
-                uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
-#pragma unroll 1
-                for (u32 q = 0; q < (a.iters & 3u); ++q) {
-                    cfs_gen_map(a, k = choose(r.x), x, y, z, sm);
-                    r = make_uint4(r.y, r.z, r.w, 0u);
-                }
+            /* the last, cut block (as a rolled loop 5% of a three-step cloud) */
+            const u32 rest = a.iters & 3u;
+            if (rest) {
+                const uint4 r = cfs_stream_block(a.rk, ps, nb, sid);
+                cfs_gen_map(a, k = choose(r.x), x, y, z, sm);
+                if (rest > 1u) cfs_gen_map(a, k = choose(r.y), x, y, z, sm);
+                if (rest > 2u) cfs_gen_map(a, k = choose(r.z), x, y, z, sm);
             }
             xyz[j] = x;
             xyz[(size_t)n_pts + j] = y;
