@@ -754,7 +754,7 @@ __global__ void __launch_bounds__(512) part_reduce_kernel(const float* part, flo
 }
 
 // U [rows][D_IN] -> UT [D_IN][ldt] (the K-major operand of dW1; batches of
-// fewer than 128 rows)
+// fewer than 64 rows)
 __global__ void __launch_bounds__(256) transpose_in_kernel(const bf16r* __restrict__ U, int rows,
                                                            bf16r* UT, int ldt)
 {
@@ -2313,7 +2313,7 @@ struct cfs_sampler {
     float *Z1, *Z2, *Z3, *Y;
     bf16r *H1, *H2, *H3, *dZ1, *dZ2, *dZ3;
     // transposed copies [features][ldt]: the K-major operands of dW = dZ^T A
-    // of batches of fewer than TC_M rows
+    // of batches of fewer than DW_ROWS rows (written up to TC_M)
     bf16r *UT, *H1T, *H2T, *dZ1T, *dZ2T, *dZ3T;
 };
 
@@ -2457,7 +2457,7 @@ cfs_status back_rows(cfs_sampler* s, const bf16r* U, int B, float* col2, float* 
 }
 
 // the weight gradients of W1..W3 and the sums of the bias-gradient copies
-// (B >= 128 rows)
+// (B >= DW_ROWS rows)
 cfs_status tc_dw(cfs_sampler* s, const bf16r* U, int B, float* grads, cudaStream_t st)
 {
     const bf16r* dz[3] = {s->dZ3, s->dZ2, s->dZ1};
@@ -2498,7 +2498,7 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
 {
     const bf16r* wb = s->wb;
     // fewer rows than one tile: the register-staged GEMMs, whose weight
-    // gradients read transposed copies
+    // gradients read transposed copies (of fewer than DW_ROWS rows)
     const bool small = !rows_on_tma(B);
     // gradient sums of the output layer and of the biases gather in copies
     // (bias_part) first: fewer atomics on the same address
@@ -2525,8 +2525,12 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     };
     // (the K-major B operand is W3^T, then W2^T)
     r = rows(s->dZ3, s->wbT + HID * HID, s->dZ2, s->dZ2T, s->Z2, col2);
-    if (r == CFS_OK) r = rows(s->dZ2, s->wbT, nullptr, s->dZ1T, s->Z1, col1);
-    if (r != CFS_OK) return r;
+    // (from one chunk of tc_dw_kernel's rows on its one launch reads the row-major
+    // copies: 64 rows 115 -> 81 us for the whole backward, 127 rows 126 -> 89)
+    const bool dw_rows = B >= DW_ROWS;
+    if (r == CFS_OK)
+        r = rows(s->dZ2, s->wbT, dw_rows ? s->dZ1 : nullptr, s->dZ1T, s->Z1, col1);
+    if (r != CFS_OK || dw_rows) return r == CFS_OK ? tc_dw(s, U, B, grads, st) : r;
     part_reduce_kernel<<<1, 512, 0, st>>>(s->bias_part, grads);
     transpose_in_kernel<<<(B + 31) / 32, 256, 0, st>>>(U, B, s->UT, s->ldt);
     // weight gradients dW = dZ^T A from the transposed copies: K = the rows
