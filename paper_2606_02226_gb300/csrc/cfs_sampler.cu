@@ -2526,7 +2526,8 @@ cfs_status backward(cfs_sampler* s, const bf16r* U, int B, const float* dY, floa
     // (the K-major B operand is W3^T, then W2^T)
     r = rows(s->dZ3, s->wbT + HID * HID, s->dZ2, s->dZ2T, s->Z2, col2);
     // (from one chunk of tc_dw_kernel's rows on its one launch reads the row-major
-    // copies: 64 rows 115 -> 81 us for the whole backward, 127 rows 126 -> 89)
+    // copies: the whole backward of 127 rows 126 -> 89 us, 64 rows 81 where 63 on
+    // the GEMMs below take 113)
     const bool dw_rows = B >= DW_ROWS;
     if (r == CFS_OK)
         r = rows(s->dZ2, s->wbT, dw_rows ? s->dZ1 : nullptr, s->dZ1T, s->Z1, col1);
