@@ -702,7 +702,7 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
                 z = CFS_DIM == 3 ? (float)(r.z >> 8) * CFS_INV_2_24 : 0.0f;
             }
         };
-        /* (a copy of the step code for each kind of choice) */
+        /* (with a window a copy of the step code for each kind of choice) */
         auto run_item = [&](const auto& choose) {
 #if CFS_ILP == 2
             /* two trajectories per thread, stepped in lockstep: their
@@ -729,9 +729,15 @@ cfs_batch_kernel(const __grid_constant__ cfs_launch_args a)
             }
 #endif
         };
+#if CFS_TILE
         if (s_kt.more5 <= 1) run_item(CfsChooseOne{s_kt});
         else if (s_kt.more <= 1) run_item(CfsChooseKtab<false>{s_kt, 1});
         else run_item(CfsChooseKtab<true>{s_kt, s_kt.more});
+#else
+        /* (without a window two CTAs share an SM with 32 registers a thread: three
+         * copies spilled 1.3 to 2.5 KB and took up to 6% longer than one) */
+        run_item(CfsChooseKtab<true>{s_kt, s_kt.more});
+#endif
         __syncthreads();
     }
     if (cur >= 0) {
