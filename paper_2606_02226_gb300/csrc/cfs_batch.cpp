@@ -221,30 +221,64 @@ uint32_t default_item_points(uint64_t points, uint32_t grid)
 }  // namespace cfs
 
 namespace {
-// Points per item of each frame of a batch as created.  A CTA that leaves a
-// frame flushes its windows, up to 53248 reductions, so the fewer CTAs a frame
-// is dealt to the better; but the last items should be small, or CTAs wait for
-// them.  So an item is a quarter of an equal share of the points that follow its
-// frame, at most 65536 and never below default_item_points, in whole rounds of
-// 1024 threads with two trajectories each.  (The frame's own points don't count:
-// nothing smaller fills the last round of the last frame's items, and one frame
-// of 2^22 points took 3.62 ms with them against 3.44, 2^23 7.13 and 6.72, four
-// of 2^22 11.4 and 11.2.)  Measured on GB300 (300 steps): the 256-frame
-// animation 142 ms against 159 with items of 4096 throughout, 151 of 16384 and
-// 146 of 32768 (136.7 with the later one-lookup choice).  A half instead of a
-// quarter, with the frame's own points: 141.8 ms, but 5 frames 3.11 ms against
-// 2.66; an eighth 142.7 ms.
+// Points per item of each frame of a batch as created.  With a window, a CTA that
+// leaves a frame flushes it, up to 53248 reductions, so the fewer CTAs a frame
+// is dealt to the better; and the more frames are worked on at a time, the
+// thinner their reductions to the same pixels; but the last items should be
+// small, or CTAs wait for them.  So an item is a quarter of an equal share of the
+// points that follow its frame, at most `most` <= 65536 and never below
+// default_item_points, in whole rounds of 1024 threads with two trajectories
+// each.  (The frame's own points don't count: nothing smaller fills the last round
+// of the last frame's items, and one frame of 2^22 points took 3.62 ms with them
+// against 3.44, 2^23 7.13 and 6.72, four of 2^22 11.4 and 11.2.)  Measured on GB300
+// (300 steps): the 256-frame animation 142 ms against 159 with items of 4096
+// throughout, 151 of 16384 and 146 of 32768 (136.7 with the later one-lookup
+// choice).  A half instead of a quarter, with the frame's own points: 141.8 ms, but
+// 5 frames 3.11 ms against 2.66; an eighth 142.7 ms.
+// `most`: the layers of the frames at work should stay in half of the L2, as far
+// as splats may reach them.  32 frames of 2^20 points x 200 steps of a system that
+// fills its view: 50.4 ms with 65536 throughout and 27.5 so (items of 4096: 26.7)
+// with a 2048^2 histogram of 4 channels, 35.0 and 24.8 with one of 1 channel, 24.9
+// both with 1024^2; 64 such frames of attractors, which fill a tenth of 2048^2,
+// 28.9 and 31.5 (items of 4096: 37.3).  Without a window, x 60 steps: 35.5 and 19.1
+// over 2048^2 RGBA, 50.3 and 19.2 over two histograms of 2048^2; 64 frames of
+// attractors in 512^2 RGBA 74 both (items of 4096: 126).
+// Without a window nothing is flushed, so splats that add keep 4096 points rather
+// than fewer if that brings more frames to work, their layers and those of the
+// frame coming up stay in the L2 and every CTA has an item (8 frames of 2^18
+// points x 200 steps in 512^2 RGBA 6.4 ms with 2048, 5.4 with 4096).
 void created_items(cfs_batch* b)
 {
     const uint32_t grid =
         (uint32_t)std::max(1, b->kernel.max_blocks_per_sm * std::max(1, b->kernel.num_sms));
     uint64_t points = 0;
     for (const cfs_frame& fr : b->frames) points += fr.n_points;
-    const uint32_t least = cfs::default_item_points(points, grid);
+    uint32_t least = cfs::default_item_points(points, grid);
+    // frames worked on at a time with items of `size`, and the bytes of their
+    // layers that splats may reach: one word a pixel of a histogram, whose
+    // channels are images of different maps
+    const double n = (double)b->n_frames, per_frame = std::max(1.0, (double)points / n);
+    const double l2 = (double)device_l2_bytes();
+    double bytes = 0.0;
+    for (const cfs_frame& fr : b->frames)
+        for (int t = 0; t < b->n_targets; ++t)
+            bytes += (double)target_bytes(fr.targets[t]) /
+                     (fr.targets[t].kind == CFS_TARGET_HIST_U32 ? std::max(1, fr.targets[t].channels)
+                                                                : 1);
+    auto live = [&](double size) {
+        return std::min(n, std::max(1.0, (double)grid * size / per_frame));
+    };
+    bool sums = false;
+    for (const SplatSpec& sp : b->spec.splats) sums = sums || sp.kind != CFS_TARGET_DEPTH_U64;
+    if (!b->spec.tile && sums && least < 4096 && points >= 4096ull * grid &&
+        live(4096) > live(least) && std::min(n, live(4096) + 1.0) * bytes / n <= l2)
+        least = 4096;
+    uint64_t most = least;
+    while (most < 65536 && live(2.0 * (double)most) * bytes / n <= l2 / 2) most *= 2;
     b->created.clear();
     for (const cfs_frame& fr : b->frames) {
         points -= fr.n_points;
-        const uint64_t share = std::min<uint64_t>(65536, points / (4ull * grid) / 2048 * 2048);
+        const uint64_t share = std::min<uint64_t>(most, points / (4ull * grid) / 2048 * 2048);
         b->created.push_back(std::max(least, (uint32_t)share));
     }
     b->chunks = b->created;

@@ -13,8 +13,10 @@ TOP = 1 << 32
 
 
 @pytest.mark.parametrize("n,plan", [
-    (TOP - 8192, {}),                                # as created: items of 65536 points
+    (TOP - 8192, {}),
     (TOP - 8192, {"ilp": 1}),
+    (TOP - 8192, {"chunk": 65536}),                  # the largest items of a batch as created
+    (TOP - 8192, {"chunk": 1 << 20}),
     (TOP - 1, {"chunk": 4096}),
     (TOP - 32, {"chunk": 32 * 511, "ilp": 2}),       # items that end on n itself
     (TOP - 32, {"chunk": 32 * 511, "ilp": 1})])
