@@ -100,8 +100,8 @@ def measure_smem_atomic_peak(torch, cfs, dev, reps: int = 3):
 # GPU machine computes: the occupancy search (fewer blocks per SM while ptxas
 # spills) depends on the NVRTC build the process loads, so the generated text
 # can differ between machines.
-RENDER_TRAFFIC_BYTES = 16827648          # (27789056 + 5866240) / 2, launches 1 and 2 of a frame
-RENDER_TRAFFIC_SOURCE_SHA1 = "7f16ec55ccea8c6887503e65625ec4bb2379eb6f"
+RENDER_TRAFFIC_BYTES = 16778368          # (27741696 + 5815040) / 2, launches 1 and 2 of a frame
+RENDER_TRAFFIC_SOURCE_SHA1 = "4b577307c0580ca4bf33cec80151c653fd3b57cc"
 
 
 def _code_only(text: str) -> str:
@@ -571,8 +571,8 @@ def bench_square(torch, cfs, dev, stream, reps: int = 20):
 # hash of the batch program under the default knobs (the same device headers
 # and generator as every plan's program) matches, and for the tuned plan's
 # trajectories per thread with the window on and no warp aggregation.
-BATCH_WARP_INSTR = {1: 1.2899e11, 2: 1.2343e11}
-BATCH_INSTR_SOURCE_SHA1 = "cb8256875de5a571970df541df83c266b286c620"
+BATCH_WARP_INSTR = {1: 1.2900e11, 2: 1.2323e11}
+BATCH_INSTR_SOURCE_SHA1 = "c78a0dfbfbff32b30c6d8f3ec05a071c1c609c52"
 BATCH_INSTR_PLAN = {"tile": 1, "warp_agg": 0}
 SM_COUNT, SCHEDULERS_PER_SM, SM_MAX_MHZ = 152, 4, 2070.0
 

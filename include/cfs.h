@@ -354,8 +354,9 @@ cfs_status cfs_batch_windows(cfs_batch* batch, int32_t* out);
  * plan (ilp 2, window on when the chain splats once, into a histogram that is
  * target 0, 53248 words, warp aggregation off, 4096 points per item); the
  * items of a batch as created are of its own sizes instead, up to 65536 points
- * in large batches and fewer towards the end, below 4096 where those would
- * leave CTAs without work. */
+ * in large batches (as far as the layers of the frames at work stay in the
+ * L2) and fewer towards the end, below 4096 where those would leave CTAs
+ * without work. */
 typedef struct {
     int ilp;                /* trajectories stepped together per thread: 1 or 2 */
     int window;             /* privatized shared-memory window for the chain's histogram

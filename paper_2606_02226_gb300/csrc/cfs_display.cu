@@ -340,8 +340,8 @@ cfs_status display_enqueue(const DisplayLayer* one, const DisplayLayer* layers, 
     a.background = p.background;
     // one CTA an item, 8 per multiprocessor at most; where there are fewer items
     // than that, each goes to 2, 4 or 8 CTAs, which still have a load of four
-    // pixels for every thread (a 320 x 240 layer of 4 channels, 10 items: 16 + 33 us
-    // for both passes on 10 CTAs, 4.5 + 7.8 on 80; 1920 x 1080: 6.6 us a pass)
+    // pixels for every thread (a 321 x 243 layer of 3 channels, 10 items: 16 + 32 us
+    // for both passes on 10 CTAs, 4.6 + 7.9 on 80; 1920 x 1080: 6.6 us a pass)
     const uint64_t most = (uint64_t)std::max(1, device_sm_count()) * 8;
     while (a.parts_log2 < 3 && ((uint64_t)n_items << (a.parts_log2 + 1)) <= most) ++a.parts_log2;
     const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)n_items << a.parts_log2, most);
